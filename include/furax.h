@@ -54,8 +54,9 @@ typedef int32_t furax_status;
 typedef enum { FURAX_F32 = 0, FURAX_F64 = 1 } furax_dtype;
 
 /* Arithmetic of an operator application (furax_ptnp_apply): FURAX_F32, FURAX_F64, or
- * FURAX_PREC_F32X2 = FP64-accurate results computed on FP32 units (double-FP32 "Dot2" band
- * product with exact FP32 products and two-sums; FP64 gather and per-pixel sums). */
+ * FURAX_PREC_F32X2 = FP64-accurate results without FP64 arithmetic in the band product. Both
+ * FP64-accurate settings take the same path: the band product from exact integer digits on the tensor
+ * cores, FP64 gather and per-pixel sums. */
 #define FURAX_PREC_F32X2 2
 
 /* Accumulation of P^T into pixels. */
@@ -255,7 +256,7 @@ furax_status furax_blockdiag_precond(const furax_pointing_t *p, const furax_nois
 /* out = S P^T N^-1 P S^T x with S the valid-pixel selector (valid may be NULL: all pixels).
  * x, out: device FP64 [npix_total][3], must not overlap. precision FURAX_F32 runs the
  * projection, the noise stencil and the weights in FP32 (x rounded to FP32 once) with
- * accumulation `acc`; FURAX_F64 runs everything in FP64 (acc ignored). One fused pass:
+ * accumulation `acc`; FURAX_F64 runs everything in FP64 accuracy (acc ignored). One fused pass:
  * the time-ordered data never reaches device memory. */
 furax_status furax_ptnp_apply(const furax_pointing_t *p, const furax_noise_t *n, const double *x,
                               double *out, const uint8_t *valid, int32_t precision, int32_t acc,
@@ -408,8 +409,7 @@ furax_status furax_mapmaker_cg_deproject(const furax_templates_t *t, const void 
  * is the unconstrained realisation (the caller's random draws). Per detector, CG from 0 until
  * ||r|| <= tol ||r_0|| or maxiter iterations; precision FURAX_F64 applies N in FP64, FURAX_F32 in
  * FP32 (vectors and scalars stay FP64; the filled values are then good to ~1e-7 relative),
- * FURAX_PREC_F32X2 FP64-accurate in double-FP32 on the FP32 units (bands of up to 64 taps; a
- * longer band is applied as for FURAX_F64);
+ * FURAX_PREC_F32X2 as FURAX_F64 (the FP64-accurate band product on the tensor cores);
  * iters_out: host int32 [sum ndet] or NULL. The first call allocates TOD-sized workspaces in the
  * handle (3 FP64, plus 1 FP64 for FURAX_F64 / FURAX_PREC_F32X2 or 2 FP32 for FURAX_F32) that later calls reuse and
  * furax_noise_destroy frees, so calls on one handle must not run concurrently; synchronises
@@ -426,10 +426,8 @@ furax_status furax_gapfill(const furax_noise_t *cov, const void *d, const uint8_
  * grad_psi[j] = -2 sum_t (N^-1 r)_{j,t} * 2 (U_p cos 2psi - Q_p sin 2psi) (offsets included).
  * d device [nsamp_total] of d_t; m device FP64 [npix_total][3]; chi2 device FP64 [n_obs]
  * (per observation); grad_map device FP64 [npix_total][3] or NULL; grad_psi device FP64
- * [sum ndet] or NULL. precision FURAX_F64: everything in FP64; FURAX_F32: residual, N^-1 and
- * each thread's partial sums in FP32, sums across threads and the map gradient in FP64;
- * FURAX_PREC_F32X2: FP64-accurate in double-FP32 on the FP32 units (residual, compensated band
- * product, partial sums), sums across threads and the map gradient in FP64. */
+ * [sum ndet] or NULL. precision FURAX_F64 or FURAX_PREC_F32X2: everything in FP64 accuracy; FURAX_F32: residual, N^-1 and
+ * each thread's partial sums in FP32, sums across threads and the map gradient in FP64. */
 furax_status furax_chi2_grad(const furax_pointing_t *p, const furax_noise_t *n, const void *d, int32_t d_t,
                              const double *m, double *chi2, double *grad_map, double *grad_psi,
                              int32_t precision, void *stream);
@@ -466,7 +464,7 @@ furax_status furax_debug_hold_loader(furax_pointing_t *p, int32_t hold, void *st
 
 /* out32[i] = in64[i] rounded to binary32 (nearest even) and out64[i] = in32[i] widened, both by
  * the library's own encoding arithmetic (the conversions the gap-filling vector passes and the
- * FP64 accumulation of the double-FP32 path use). Either pair may be NULL. Device arrays of n
+ * FP64 readers of FP32 data use). Either pair may be NULL. Device arrays of n
  * elements; asynchronous on `stream`. FURAX_EINVAL for n < 0 or an input without its output. */
 furax_status furax_probe_convert(const double *in64, float *out32, const float *in32, double *out64, int64_t n,
                                  void *stream);
@@ -503,7 +501,8 @@ const char *furax_version(void);
  * kernels (FP32 and FP64) with CUDA events on the launching stream (also inside captured
  * graphs) and accumulates their durations, read at the solver's synchronisation points and
  * at furax_profile_read. kernel: 0 = FP32 fused apply, 1 = FP64 fused apply (incl. the FP64
- * right-hand side), 2 = double-FP32 fused apply (incl. its right-hand side). Writes the total milliseconds and the number of timed launches. */
+ * right-hand side), 2 = the same for
+ * FURAX_PREC_F32X2 and the mixed solver's outer steps. Writes the total milliseconds and the number of timed launches. */
 void furax_profile_enable(int32_t on);
 furax_status furax_profile_read(int32_t kernel, double *total_ms, int64_t *count);
 void furax_profile_reset(void);

@@ -207,7 +207,7 @@ void furax_profile_enable(int32_t on) { g_prof_on = on != 0; }
 
 furax_status furax_profile_read(int32_t kernel, double *total_ms, int64_t *count)
 {
-    REQUIRE(kernel >= 0 && kernel <= 2, "kernel must be 0 (FP32 fused), 1 (FP64 fused) or 2 (double-FP32 fused)");
+    REQUIRE(kernel >= 0 && kernel <= 2, "kernel must be 0 (FP32 fused), 1 (FP64 fused) or 2 (FP64-accurate steps of the mixed path)");
     prof_flush();
     std::lock_guard<std::mutex> lk(g_prof_mu);
     if (total_ms) *total_ms = g_prof_ms[kernel];
@@ -313,8 +313,8 @@ static void pointing_free(furax_pointing *p)
     cudaFree(p->d_obs); cudaFree(p->d_tiles); cudaFree(p->d_ptiles); cudaFree(p->d_psi_cs); cudaFree(p->d_hwp_cs);
     cudaFree(p->pix); cudaFree(p->c32); cudaFree(p->s32); cudaFree(p->c64); cudaFree(p->s64);
     cudaFree(p->c32lo); cudaFree(p->s32lo); cudaFree(p->ws_bore_m);
-    cudaFree(p->ws_map32); cudaFree(p->ws_acc_hi); cudaFree(p->ws_acc64); cudaFree(p->ws_df_lo); cudaFree(p->ws_x64);
-    cudaFree(p->ws_x2);
+    cudaFree(p->ws_map32); cudaFree(p->ws_acc_hi); cudaFree(p->ws_acc64); cudaFree(p->ws_x64);
+    cudaFree(p->ws_x4);
     cudaFree(p->ws_tod); cudaFree(p->ws_tod2); cudaFree(p->ws_hits); cudaFree(p->d_err);
     delete p;
 }
@@ -569,43 +569,54 @@ furax_status furax_noise_create(int32_t kind, const double *params, int32_t ntap
     n->ndet_total = ndet;
     n->nsamp_total = L.nsamp;
     n->n_tiles = (int64_t)L.tiles.size();
-    if (cudaMalloc((void **)&n->d_obs, sizeof(ObsInfo) * L.obs.size()) != cudaSuccess ||
-        cudaMalloc((void **)&n->d_tiles, sizeof(Tile) * std::max<size_t>(1, L.tiles.size())) != cudaSuccess ||
-        cudaMemcpyAsync(n->d_obs, L.obs.data(), sizeof(ObsInfo) * L.obs.size(), cudaMemcpyHostToDevice,
+    // one allocation for everything that is laid out here (each costs the caller some 0.2 ms)
+    const int64_t cnt = kind == FURAX_NOISE_WHITE ? ndet : ndet * ntaps;
+    const bool short_band = kind == FURAX_NOISE_BANDED && !long_band(n);
+    size_t bytes = 0;
+    auto part = [&](size_t b) { const size_t at = bytes; bytes += (b + 255) & ~size_t(255); return at; };
+    const size_t o_obs = part(sizeof(ObsInfo) * L.obs.size()), o_tiles = part(sizeof(Tile) * L.tiles.size()),
+                 o_p64 = part(sizeof(double) * cnt), o_diag = part(sizeof(double) * ndet), o_p32 = part(sizeof(float) * cnt),
+                 o_err = part(sizeof(unsigned) * kCtlWords),
+                 o_band2 = part(short_band ? sizeof(float) * kBandPairs * 2 * (size_t)ndet : 0),
+                 o_exp = part(short_band ? sizeof(int32_t) * (size_t)ndet : 0),
+                 o_taps = part(short_band ? tc_taps_bytes(ndet) : 0);
+    if (cudaMalloc((void **)&n->slab, bytes) != cudaSuccess) {
+        cudaGetLastError();
+        delete n;
+        return set_error(FURAX_ENOMEM, "noise allocation of %zu bytes failed", bytes);
+    }
+    n->d_obs = (ObsInfo *)(n->slab + o_obs);
+    n->d_tiles = (Tile *)(n->slab + o_tiles);
+    n->p64 = (double *)(n->slab + o_p64);
+    n->diag = (double *)(n->slab + o_diag);
+    n->p32 = (float *)(n->slab + o_p32);
+    n->d_err = (unsigned *)(n->slab + o_err);
+    if (short_band) {
+        n->band2 = (float *)(n->slab + o_band2);
+        n->tc_exp = (int32_t *)(n->slab + o_exp);
+        n->tc_taps = n->slab + o_taps;
+    }
+    if (cudaMemcpyAsync(n->d_obs, L.obs.data(), sizeof(ObsInfo) * L.obs.size(), cudaMemcpyHostToDevice,
                         (cudaStream_t)stream) != cudaSuccess ||
         cudaMemcpyAsync(n->d_tiles, L.tiles.data(), sizeof(Tile) * L.tiles.size(), cudaMemcpyHostToDevice,
                         (cudaStream_t)stream) != cudaSuccess ||
+        cudaMemsetAsync(n->d_err, 0, sizeof(unsigned) * kCtlWords, (cudaStream_t)stream) != cudaSuccess ||
         cudaStreamSynchronize((cudaStream_t)stream) != cudaSuccess) {
         cudaGetLastError();
-        cudaFree(n->d_obs); cudaFree(n->d_tiles);
+        cudaFree(n->slab);
         delete n;
-        return set_error(FURAX_ENOMEM, "noise layout allocation failed");
-    }
-    const int64_t cnt = kind == FURAX_NOISE_WHITE ? ndet : ndet * ntaps;
-    if (cudaMalloc((void **)&n->p64, sizeof(double) * cnt) != cudaSuccess ||
-        cudaMalloc((void **)&n->p32, sizeof(float) * cnt) != cudaSuccess ||
-        cudaMalloc((void **)&n->diag, sizeof(double) * ndet) != cudaSuccess) {
-        cudaGetLastError();
-        cudaFree(n->p64); cudaFree(n->p32); cudaFree(n->diag); cudaFree(n->d_obs); cudaFree(n->d_tiles);
-        delete n;
-        return set_error(FURAX_ENOMEM, "noise allocation failed");
+        return set_error(FURAX_ECUDA, "noise layout upload failed");
     }
     const int64_t m = std::max(cnt, ndet);
     noise_prep_kernel<<<(unsigned)((m + 255) / 256), 256, 0, (cudaStream_t)stream>>>(kind, params, cnt, ntaps, n->p64,
                                                                                     n->p32, n->diag, ndet);
     count_launches(1);
     if (!(rc = check_launch("noise create")) && long_band(n)) rc = prepare_noise_fft(n, L.obs, (cudaStream_t)stream);
-    if (!rc && kind == FURAX_NOISE_BANDED && !long_band(n)) {
-        if (cudaMalloc((void **)&n->band2, sizeof(float) * kBandPairs * 2 * (size_t)ndet) != cudaSuccess) {
-            cudaGetLastError();
-            rc = set_error(FURAX_ENOMEM, "noise band table allocation failed");
-        } else {
-            const int64_t nb = ndet * kBandPairs;
-            band_pairs_kernel<<<(unsigned)((nb + 255) / 256), 256, 0, (cudaStream_t)stream>>>(n->p32, ntaps, ndet,
-                                                                                              n->band2);
-            count_launches(1);
-            rc = check_launch("noise band table");
-        }
+    if (!rc && short_band) {
+        const int64_t nb = ndet * kBandPairs;
+        band_pairs_kernel<<<(unsigned)((nb + 255) / 256), 256, 0, (cudaStream_t)stream>>>(n->p32, ntaps, ndet, n->band2);
+        count_launches(1);
+        if (!(rc = check_launch("noise band table"))) rc = prepare_noise_tc(n, (cudaStream_t)stream);
     }
     if (rc) {
         furax_noise_destroy(n);
@@ -619,7 +630,7 @@ furax_status furax_noise_destroy(furax_noise_t *n)
 {
     if (!n) return FURAX_OK;
     cudaDeviceSynchronize();
-    cudaFree(n->p64); cudaFree(n->p32); cudaFree(n->diag); cudaFree(n->d_obs); cudaFree(n->d_tiles); cudaFree(n->band2);
+    cudaFree(n->slab);
     cudaFree(n->fft_items); cudaFree(n->tw64); cudaFree(n->tw32); cudaFree(n->spec64); cudaFree(n->spec32);
     cudaFree(n->gf_y); cudaFree(n->gf_r); cudaFree(n->gf_p); cudaFree(n->gf_q); cudaFree(n->gf_x32); cudaFree(n->gf_n32);
     cudaFree(n->gf_sc);
@@ -682,11 +693,11 @@ furax_status furax_rhs(const furax_pointing_t *p, const furax_noise_t *n, const 
     const bool prof = prof_on();
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     if (prof) { prof_pair(&e0, &e1); if (e0) cudaEventRecord(e0, st); }
-    // FP64-accurate on FP32 pipes (double-FP32 band product); FP64 arithmetic would be ~5x slower here.
+    // FP64-accurate, the band product on the tensor cores.
     // A band longer than the fused kernels hold: overlap-save N^-1 in FP64 with the TOD in HBM.
     if (long_band(n)) {
         if ((rc = tod_ws(p)) || (rc = launch_rhs_chain(p, n, d, d_t, pm->ws_acc64, st))) return rc;
-    } else if ((rc = launch_fused_df(p, n, nullptr, d, d_t, pm->ws_acc64, st))) {
+    } else if ((rc = launch_rhs_tc(p, n, d, d_t, pm->ws_acc64, false, st))) {
         return rc;
     }
     if (prof) { if (e1) cudaEventRecord(e1, st); prof_push(2, e0, e1); }

@@ -8,12 +8,6 @@
 
 namespace fx {
 
-__device__ __forceinline__ void split_df(double v, float &hi, float &lo)
-{
-    hi = (float)v;
-    lo = (float)(v - (double)hi);
-}
-
 // Compensated dot-product step with an exact FP32 input x (no input low word): S + E += (ch + cl) x
 // (Ogita, Rump & Oishi 2005, algorithm Dot2).
 __device__ __forceinline__ void dot2_step_x(float ch, float cl, float x, float &S, float &E)
@@ -41,16 +35,6 @@ __device__ __forceinline__ void df_add(float &h, float &l, float bh, float bl)
     const float bv = __fsub_rn(s, h);
     const float err = __fadd_rn(__fsub_rn(h, __fsub_rn(s, bv)), __fsub_rn(bh, bv));   // h + bh = s + err
     df_renorm(s, __fadd_rn(__fadd_rn(l, bl), err), h, l);
-}
-
-// One Horner step (h, l) <- (h, l) j + (eh, el) for an exact FP32 multiplier j.
-__device__ __forceinline__ void df_horner(float &h, float &l, float j, float eh, float el)
-{
-    const float p = __fmul_rn(h, j);
-    const float pl = __fmaf_rn(l, j, __fmaf_rn(h, j, -p));   // h j = p + (h j - p) exactly
-    h = p;
-    l = pl;
-    df_add(h, l, eh, el);
 }
 
 // binary32 -> binary64 from the IEEE 754 encodings: sign kept, exponent rebiased by

@@ -1,0 +1,301 @@
+// FP64-accurate operators on one tile (one detector, up to 4096 samples) per CTA: the normal operator
+// acc += P^T N^-1 P x, the right-hand side acc += P^T N^-1 d and N^-1 alone (Furax paper: the estimator
+// A = (H.T @ N.I @ H).I @ H.T @ N.I of the Software Design listing, with the block decomposition
+// P^T N^-1 P = sum_i P_i^T N_i^-1 P_i of "Algebraic reductions"), for FURAX_F64 and FURAX_PREC_F32X2.
+//
+// Each CTA forms the tile's samples with their 63-sample halos in registers, applies the band on the tensor
+// cores (band_tc.cuh) and scatters y (1, cos 2psi, sin 2psi) in time order as whole FP64 pixel records; the
+// pointing is read a second time for the scatter (from L2), which leaves the shared memory to the digits.
+// What bounds it: the L2's FP64 reductions (3 per sample, 18,000 cycles per tile and SM at the rate of
+// furax_probe_l2 kind 5) and the latency of the phases before them (fill, digits 4,000, products 9,000,
+// accumulators to y 6,000-10,000 cycles), which two CTAs per SM overlap in part; then the FP64 pipe (4
+// instructions per sample). Measured (GB300), before (FP64 FMAs; double-FP32 for the right-hand side) and now:
+//   normal operator, 32 x 262,147 samples, nside 256, FP64 cache   2277 -> 324 us
+//   right-hand side, 128 x 524,288 FP32 samples, mixed cache       3437 -> 1730 us
+//   N^-1 alone inside gap filling, 32 x 131,071 samples            1011 -> 60 us
+#include "tc_sample.cuh"
+#include "tpl_eval.cuh"
+
+namespace fx {
+
+// Template correction of the right-hand side, y -= (W T) b for amplitudes b already solved from d: in the
+// interior of a stream a cubic in the offset j of the sample from the middle of the tile's own samples
+// (no extrapolation in tau), summed term by term near the stream's ends.
+struct TplCorr {
+    double e[4];
+    __device__ __forceinline__ void init(const TplView &tv, const Tile &tl, const ObsInfo &ob, int64_t gdet)
+    {
+        const double h = ob.nsamp > 1 ? 2.0 / (double)(ob.nsamp - 1) : 0.0;
+        const double2 m = tv.mom[gdet];
+        const double bv[4] = {tv.b[4 * gdet], tv.b[4 * gdet + 1], tv.b[4 * gdet + 2], tv.b[4 * gdet + 3]};
+        double c[4];
+        tpl_cubic(m.x, m.y * h * h * 0.5, bv, c);
+        cubic_shift(c, tpl_tau_ref(tl.t0 + (tl.len >> 1), ob.nsamp), h, e);
+    }
+    __device__ __forceinline__ double apply(double y, const NoiseView &nv, const TplView &tv, const Tile &tl,
+                                            const ObsInfo &ob, int64_t gdet, int k) const
+    {
+        const int64_t t = tl.t0 + k;
+        if (tpl_interior(tv, t, ob.nsamp)) {
+            const double j = (double)(k - (tl.len >> 1));
+            return y - fma(fma(fma(e[3], j, e[2]), j, e[1]), j, e[0]);
+        }
+        double w[4];
+        wt_eval<double>(nv, tv, gdet, ob.nsamp, t, w);
+#pragma unroll
+        for (int l = 0; l < 4; ++l) y -= tv.b[4 * gdet + l] * w[l];
+        return y;
+    }
+};
+
+// FROM_TOD: samples d, else P x. TPL (FROM_TOD only): with the template correction.
+template <int MODE, bool FROM_TOD, bool TPL, typename DT>
+__global__ void __launch_bounds__(FT, 2) tc_operator_kernel(const Tile *__restrict__ tiles, PointingView pv, NoiseView nv,
+                                                            const double4_32a *__restrict__ x, const DT *__restrict__ d,
+                                                            double *__restrict__ acc64, unsigned *__restrict__ err,
+                                                            bool f64, TplView tv)
+{
+    extern __shared__ __align__(128) unsigned char sm[];
+    __shared__ TplCorr corr;
+    const Tile tl = tiles[blockIdx.x];
+    const ObsInfo ob = pv.obs[tl.obs];
+    const int64_t gdet = ob.det_off + tl.det;
+    const TcPsi psi(pv, gdet);
+    tc_begin(sm, nv, gdet);
+    if constexpr (TPL)
+        if (threadIdx.x == 0) corr.init(tv, tl, ob, gdet);
+    {
+        double v[kTcPer];
+        const TcSlots sl(tl, ob);
+        if constexpr (FROM_TOD) tc_fill_tod(v, sl, d);
+        else tc_fill_map<MODE, false>(sm, v, sl, pv, ob, tl, psi, x, d);
+        tc_band<false>(sm, v, nv, gdet, err, f64, sl.in0, sl.in1);
+    }
+    const double *ys = tc_ys(sm);
+    double *rec = acc64 + 3 * ob.map_off;
+    tc_each<MODE>(pv, ob, tl, psi, [&](int k, int32_t pix, double c, double s) {
+        double y = pix >= 0 ? ys[spos(k)] : 0.0;
+        if constexpr (TPL)
+            if (pix >= 0) y = corr.apply(y, nv, tv, tl, ob, gdet, k);
+        const double v[3] = {y, y * c, y * s};
+        red_add_f64_records_warp<3, double>(rec, pix, v, tc_stage(sm), tc_stage_pix(sm));
+    });
+}
+
+// White noise: no neighbours, so each sample goes straight from the gather to its records.
+template <int MODE, bool FROM_TOD, bool TPL, typename DT>
+__global__ void __launch_bounds__(FT) white_operator_kernel(const Tile *__restrict__ tiles, PointingView pv, NoiseView nv,
+                                                            const double4_32a *__restrict__ x, const DT *__restrict__ d,
+                                                            double *__restrict__ acc64, TplView tv)
+{
+    __shared__ double stage[FT / 32][96];
+    __shared__ int32_t spix[FT / 32][32];
+    __shared__ TplCorr corr;
+    const Tile tl = tiles[blockIdx.x];
+    const ObsInfo ob = pv.obs[tl.obs];
+    const int64_t gdet = ob.det_off + tl.det;
+    const TcPsi psi(pv, gdet);
+    if constexpr (TPL) {
+        if (threadIdx.x == 0) corr.init(tv, tl, ob, gdet);
+        __syncthreads();
+    }
+    const double w = nv.p64[gdet];
+    const DT *row = d + ob.tod_off + (int64_t)tl.det * ob.nsamp + tl.t0;
+    double *rec = acc64 + 3 * ob.map_off;
+    const int warp = threadIdx.x >> 5;
+    tc_each<MODE>(pv, ob, tl, psi, [&](int k, int32_t pix, double c, double s) {
+        double y = 0.0;
+        if (pix >= 0) {
+            if constexpr (FROM_TOD) y = tod_f64(row[k]) * w;
+            else {
+                TcPix m;
+                m.load(x, ob.map_off + pix);
+                y = m.project(pix, c, s) * w;
+            }
+            if constexpr (TPL) y = corr.apply(y, nv, tv, tl, ob, gdet, k);
+        }
+        const double v[3] = {y, y * c, y * s};
+        red_add_f64_records_warp<3, double>(rec, pix, v, stage[warp], spix[warp]);
+    });
+}
+
+// out = N^-1 in on an FP64 TOD, banded.
+template <bool MASKED>
+__global__ void __launch_bounds__(FT, 2) tc_ninv_kernel(const Tile *__restrict__ tiles, const ObsInfo *__restrict__ obs,
+                                                        NoiseView nv, const double *__restrict__ in,
+                                                        double *__restrict__ out, unsigned *__restrict__ err, bool f64)
+{
+    extern __shared__ __align__(128) unsigned char sm[];
+    const Tile tl = tiles[blockIdx.x];
+    const ObsInfo ob = obs[tl.obs];
+    const int64_t gdet = ob.det_off + tl.det;
+    const int64_t row = ob.tod_off + (int64_t)tl.det * ob.nsamp;
+    tc_begin(sm, nv, gdet);
+    double v[kTcPer];
+    const TcSlots sl(tl, ob);
+    tc_fill_tod(v, sl, in);
+    tc_band<MASKED>(sm, v, nv, gdet, err, f64, sl.in0, sl.in1);
+    const double *ys = tc_ys(sm);
+    for (int k = threadIdx.x; k < tl.len; k += FT) out[row + tl.t0 + k] = ys[spos(k)];
+}
+
+furax_status launch_ninv_tc(const furax_noise *n, const double *in, double *out, bool masked, bool f64, cudaStream_t st)
+{
+    if (n->n_tiles == 0) return FURAX_OK;
+    furax_status rc = launch_dyn(masked ? tc_ninv_kernel<true> : tc_ninv_kernel<false>, (unsigned)n->n_tiles, FT, kTcSmem, st,
+                                 n->d_tiles, n->d_obs, n->view(), in, out, n->d_err, f64);
+    if (rc) return rc;
+    count_launches(1);
+    return check_launch("N^-1 apply (FP64, banded)");
+}
+
+template <int MODE, bool FROM_TOD, bool TPL, typename DT>
+static furax_status run_tc(const furax_pointing *p, const furax_noise *n, const double4_32a *x, const DT *d, double *a64,
+                           bool f64, const TplView &tv, cudaStream_t st)
+{
+    if (n->kind == FURAX_NOISE_BANDED)
+        return launch_dyn(tc_operator_kernel<MODE, FROM_TOD, TPL, DT>, (unsigned)p->n_tiles, FT, kTcSmem, st, p->d_tiles,
+                          p->view(), n->view(), x, d, a64, p->d_err, f64, tv);
+    white_operator_kernel<MODE, FROM_TOD, TPL, DT><<<(unsigned)p->n_tiles, FT, 0, st>>>(p->d_tiles, p->view(), n->view(), x,
+                                                                                         d, a64, tv);
+    return FURAX_OK;
+}
+
+template <bool FROM_TOD, bool TPL, typename DT>
+static furax_status dispatch_tc(const furax_pointing *p, const furax_noise *n, const double4_32a *x, const DT *d, double *a64,
+                                bool f64, const TplView &tv, cudaStream_t st)
+{
+    if (p->n_tiles == 0) return FURAX_OK;
+    furax_status rc;
+    switch (p->mode) {
+    case FURAX_POINTING_ON_THE_FLY: rc = run_tc<0, FROM_TOD, TPL, DT>(p, n, x, d, a64, f64, tv, st); break;
+    case FURAX_POINTING_CACHE_F32: rc = run_tc<1, FROM_TOD, TPL, DT>(p, n, x, d, a64, f64, tv, st); break;
+    case FURAX_POINTING_CACHE_MIXED: rc = run_tc<3, FROM_TOD, TPL, DT>(p, n, x, d, a64, f64, tv, st); break;
+    default: rc = run_tc<2, FROM_TOD, TPL, DT>(p, n, x, d, a64, f64, tv, st);
+    }
+    if (rc) return rc;
+    count_launches(1);
+    return check_launch(FROM_TOD ? "right-hand side P^T N^-1 d" : "fused P^T N^-1 P (FP64)");
+}
+
+__global__ void pack_x4_kernel(const double *__restrict__ x, const uint8_t *__restrict__ valid, double4_32a *__restrict__ x4,
+                               int64_t np)
+{
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < np; i += (int64_t)gridDim.x * blockDim.x) {
+        const bool ok = !valid || valid[i];
+        x4[i] = ok ? double4_32a{x[3 * i], x[3 * i + 1], x[3 * i + 2], 0.0} : double4_32a{0.0, 0.0, 0.0, 0.0};
+    }
+}
+
+furax_status launch_pack_x4(const furax_pointing *p, const double *x, const uint8_t *valid, cudaStream_t st)
+{
+    furax_pointing *pm = const_cast<furax_pointing *>(p);
+    const int64_t np = p->npix_total;
+    furax_status rc = ensure_ws(pm, (void **)&pm->ws_x4, sizeof(double4_32a) * (size_t)np);
+    if (rc) return rc;
+    const unsigned g = (unsigned)std::max<int64_t>(1, std::min<int64_t>((np + 255) / 256, 8LL * p->n_sm));
+    pack_x4_kernel<<<g, 256, 0, st>>>(x, valid, pm->ws_x4, np);
+    count_launches(1);
+    return check_launch("pack FP64 map");
+}
+
+furax_status launch_fused_tc(const furax_pointing *p, const furax_noise *n, const double *x, const uint8_t *valid, double *a64,
+                             bool f64, cudaStream_t st)
+{
+    furax_status rc = launch_pack_x4(p, x, valid, st);
+    if (rc) return rc;
+    return dispatch_tc<false, false, double>(p, n, p->ws_x4, nullptr, a64, f64, TplView{}, st);
+}
+
+furax_status launch_rhs_tc(const furax_pointing *p, const furax_noise *n, const void *d, int d_t, double *a64, bool f64,
+                           cudaStream_t st, const furax_templates *tp)
+{
+    const double *d64 = (const double *)d;
+    const float *d32 = (const float *)d;
+    if (tp) {
+        const TplView tv = tp->view();
+        return d_t == FURAX_F64 ? dispatch_tc<true, true, double>(p, n, nullptr, d64, a64, f64, tv, st)
+                                : dispatch_tc<true, true, float>(p, n, nullptr, d32, a64, f64, tv, st);
+    }
+    return d_t == FURAX_F64 ? dispatch_tc<true, false, double>(p, n, nullptr, d64, a64, f64, TplView{}, st)
+                            : dispatch_tc<true, false, float>(p, n, nullptr, d32, a64, f64, TplView{}, st);
+}
+
+// Digits of a detector's taps (one CTA each): integers relative to 2^ec, balanced base-256
+// digits, stored as the distinct core matrices of the operand (band_tc.cuh): [digit][matrix h][row r][column e]
+// is the tap of lag index 8 h - 8 + e - r (0 .. 126).
+__global__ void __launch_bounds__(128) tap_digits_kernel(const double *__restrict__ taps, int ntaps,
+                                                         unsigned char *__restrict__ out, int32_t *__restrict__ exps)
+{
+    __shared__ double c[MAXTAPS];
+    const int64_t det = blockIdx.x;
+    if (threadIdx.x < MAXTAPS) c[threadIdx.x] = threadIdx.x < ntaps ? taps[det * ntaps + threadIdx.x] : 0.0;
+    __syncthreads();
+    double m = 0.0, off = 0.0;   // largest tap, weight off the diagonal
+    bool finite = true;
+    for (int k = 0; k < MAXTAPS; ++k) {
+        m = fmax(m, fabs(c[k]));
+        if (k > 0) off += 2.0 * fabs(c[k]);
+        finite = finite && isfinite(c[k]);
+    }
+    const bool ok = finite && ntaps >= kTcMinTaps && off >= m / 16 && m > 0.0;
+    // |c| 2^(55 - ec) <= 0x7f7f7f7f7f7f7f, the largest integer of seven balanced digits
+    int ec = ok ? ilogb(m) + 1 : 0;
+    if (scalbn(m, -ec) > 0.99) ++ec;
+    if (threadIdx.x == 0) exps[det] = ok ? ec : kTcNoTaps;
+    __half *o = reinterpret_cast<__half *>(out + det * kTcDetBytes);
+    for (int i = threadIdx.x; i < kTcCores * 64; i += 128) {
+        const int j = 8 * (i >> 6) - 8 + (i & 7) - ((i >> 3) & 7);
+        const int lag = j < kHalo ? kHalo - j : j - kHalo;
+        const double v = ok && j >= 0 && j < kBand ? scalbn(c[lag], 55 - ec) : 0.0;
+        const uint64_t w = (uint64_t)__double2ll_rn(v) + 0x80808080808080ull;
+        for (int g = 0; g < kTcCDig; ++g)
+            o[g * kTcCores * 64 + i] = __int2half_rn((int)((w >> (8 * (kTcCDig - 1 - g))) & 0xff) - 128);
+    }
+}
+
+size_t tc_taps_bytes(int64_t ndet) { return (size_t)kTcDetBytes * (size_t)ndet; }
+
+furax_status prepare_noise_tc(furax_noise *n, cudaStream_t st)
+{
+    furax_status rc;
+    const size_t nd = (size_t)n->ndet_total;
+    if ((rc = allow_smem((const void *)tc_ninv_kernel<false>, kTcSmem))) return rc;
+    if ((rc = allow_smem((const void *)tc_ninv_kernel<true>, kTcSmem))) return rc;
+    tap_digits_kernel<<<(unsigned)nd, 128, 0, st>>>(n->p64, n->ntaps, n->tc_taps, n->tc_exp);
+    count_launches(1);
+    return check_launch("tap digits");
+}
+
+template <int MODE>
+static furax_status prep_tc_mode()
+{
+    furax_status rc = FURAX_OK;
+    if (!rc) rc = allow_smem((const void *)tc_operator_kernel<MODE, false, false, double>, kTcSmem);
+    if (!rc) rc = allow_smem((const void *)tc_operator_kernel<MODE, true, false, double>, kTcSmem);
+    if (!rc) rc = allow_smem((const void *)tc_operator_kernel<MODE, true, false, float>, kTcSmem);
+    if (!rc) rc = allow_smem((const void *)tc_operator_kernel<MODE, true, true, double>, kTcSmem);
+    if (!rc) rc = allow_smem((const void *)tc_operator_kernel<MODE, true, true, float>, kTcSmem);
+    return rc;
+}
+
+furax_status prepare_fused_tc()
+{
+    furax_status rc = prep_tc_mode<0>();
+    if (!rc) rc = prep_tc_mode<1>();
+    if (!rc) rc = prep_tc_mode<2>();
+    if (!rc) rc = prep_tc_mode<3>();
+    return rc;
+}
+
+furax_status prepare_kernels()
+{
+    static furax_status done = 1;
+    if (done == FURAX_OK) return FURAX_OK;
+    furax_status rc = prepare_fused_f32();
+    if (!rc) rc = prepare_fused_tc();
+    done = rc;
+    return rc;
+}
+
+}  // namespace fx

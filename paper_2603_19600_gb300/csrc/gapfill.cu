@@ -194,11 +194,11 @@ furax_status gapfill(const furax_noise *n, const void *d, const uint8_t *valid, 
                      int maxiter, double tol, int precision, int32_t *iters_out, cudaStream_t st)
 {
     const bool f32 = precision == FURAX_F32;   // band product in FP32, vectors and scalars in FP64
-    // FURAX_PREC_F32X2: the FP64 path with its band products in double-FP32 (short bands; a long
-    // band keeps the FP64 overlap-save product)
-    const bool df = precision == FURAX_PREC_F32X2 && !long_band(n);
+    // N on masked vectors (zero in the gaps): short bands on the tensor cores, FURAX_PREC_F32X2 with the
+    // compensated product for tiles outside the digits' range
     auto ninv64 = [&](const double *in, double *o) {
-        return df ? launch_ninv_df(n, in, o, st) : launch_ninv(n, in, o, FURAX_F64, st);
+        return long_band(n) ? launch_ninv(n, in, o, FURAX_F64, st)
+                            : launch_ninv_tc(n, in, o, true, precision == FURAX_F64, st);
     };
     const int64_t ns = n->nsamp_total, nd = n->ndet_total;
     if (ns == 0 || nd == 0) return FURAX_OK;
@@ -286,9 +286,13 @@ furax_status gapfill(const furax_noise *n, const void *d, const uint8_t *valid, 
         count_launches(1);
         rc = check_launch("gap filling (fill)");
     }
+    unsigned gave_up = 0;
     if (!rc) rc = check_cuda(cudaMemcpyAsync(h.data(), sc, sizeof(GfDet) * nd, cudaMemcpyDeviceToHost, st), "read");
+    if (!rc) rc = check_cuda(cudaMemcpyAsync(&gave_up, n->d_err, sizeof gave_up, cudaMemcpyDeviceToHost, st), "read");
+    if (!rc) rc = check_cuda(cudaMemsetAsync(n->d_err, 0, sizeof gave_up, st), "clear");
     if (!rc) rc = check_cuda(cudaStreamSynchronize(st), "gap filling");
     if (rc) return rc;
+    if (gave_up) return set_error(FURAX_ETIMEOUT, "a bounded device-side wait gave up during gap filling");
     all_done = true;
     for (int64_t i = 0; i < nd; ++i) {
         all_done = all_done && h[i].done;

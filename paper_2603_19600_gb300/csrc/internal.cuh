@@ -89,6 +89,8 @@ struct NoiseView {
     const double *p64;      // white: inverse variance [ndet]; banded: taps [ndet][ntaps]
     const float *p32;
     const double *diag;     // diagonal of N^-1 per detector [ndet] (FP64)
+    const unsigned char *tc_taps;  // banded (<= MAXTAPS taps): tap digits per detector (band_tc.cuh)
+    const int32_t *tc_exp;         // [ndet] exponent of the tap digits
     const float *band2;     // banded (<= MAXTAPS taps): [ndet][2 kBandPad] band in tap order as duplicated pairs
 };
 
@@ -179,8 +181,7 @@ struct furax_pointing {
     float4 *ws_acc_hi = nullptr;      // [2 npix] FP32 accumulator (I,Q,U,-): plain hi[i], or compensated
                                       // hi[2i] with its compensation at hi[2i + 1] (atomics.cuh)
     double *ws_acc64 = nullptr;       // [npix][3] FP64 accumulator
-    float4 *ws_df_lo = nullptr;       // [npix] FP32 low-word accumulator of the double-FP32 RHS and operator
-    float4 *ws_x2 = nullptr;          // [npix][2] double-FP32 split (high, low words) of an FP64 map
+    double4_32a *ws_x4 = nullptr;     // [npix] FP64 map in 32-byte records for the FP64-accurate gathers
     double *ws_x64 = nullptr;         // [npix][3] masked FP64 copy
     void *ws_tod = nullptr;           // [nsamp] scratch TOD (FP64 size)
     void *ws_tod2 = nullptr;
@@ -226,6 +227,7 @@ struct furax_noise {
     int32_t ntaps = 0;
     int64_t ndet_total = 0;
     int64_t nsamp_total = 0;
+    unsigned char *slab = nullptr;    // the allocation that holds the arrays below up to d_err
     double *p64 = nullptr;
     float *p32 = nullptr;
     double *diag = nullptr;
@@ -245,7 +247,10 @@ struct furax_noise {
     float *gf_x32 = nullptr, *gf_n32 = nullptr;
     void *gf_sc = nullptr;
     float *band2 = nullptr;     // banded, <= MAXTAPS taps: [ndet][256] band in tap order as duplicated pairs
-    fx::NoiseView view() const { return fx::NoiseView{kind, ntaps, p64, p32, diag, band2}; }
+    unsigned char *tc_taps = nullptr;   // banded, <= MAXTAPS taps: digits of the taps for the tensor cores
+    int32_t *tc_exp = nullptr;          // [ndet]
+    unsigned *d_err = nullptr;          // device control block (kCtlWords) of the kernels run on this handle alone
+    fx::NoiseView view() const { return fx::NoiseView{kind, ntaps, p64, p32, diag, tc_taps, tc_exp, band2}; }
 };
 
 namespace fx {
@@ -268,8 +273,12 @@ furax_status launch_bj(const furax_pointing *p, const furax_noise *n, double rco
 
 // ---- launchers (noise.cu)
 furax_status launch_ninv(const furax_noise *n, const void *in, void *out, int dtype, cudaStream_t st);
-// FP64 in, FP64 out, band product in double-FP32 (bands of up to MAXTAPS taps; fused_df.cu)
-furax_status launch_ninv_df(const furax_noise *n, const double *in, double *out, cudaStream_t st);
+// FP64 in, FP64 out, bands of up to MAXTAPS taps on the tensor cores (fused_tc.cu). masked: zero samples of
+// `in` are masked ones; f64 as below.
+furax_status launch_ninv_tc(const furax_noise *n, const double *in, double *out, bool masked, bool f64, cudaStream_t st);
+// Digits of the taps of a short band (fused_tc.cu).
+furax_status prepare_noise_tc(furax_noise *n, cudaStream_t st);
+size_t tc_taps_bytes(int64_t ndet);
 // Bands longer than the fused kernels hold go through the TOD in HBM (overlap-save N^-1).
 inline bool long_band(const furax_noise *n) { return n->kind == FURAX_NOISE_BANDED && n->ntaps > MAXTAPS; }
 // noise_fft.cu: blocks, twiddles and spectra of a long band (synchronises st); the N^-1 apply.
@@ -318,19 +327,18 @@ furax_status launch_fused_f32(const furax_pointing *p, const furax_noise *n, con
                               float4 *acc_hi, float4 *acc_lo, double *acc64, cudaStream_t st,
                               const FusedTpl *ft = nullptr);
 bool fused_f32_projects_templates(const furax_pointing *p);
-furax_status launch_fused_f64(const furax_pointing *p, const furax_noise *n, const double *x, double *acc64,
-                              cudaStream_t st);
-// FP64-accurate operator on FP32 units (double-FP32 band product): acc64 += P^T N^-1 P x, or
-// acc64 += P^T N^-1 d when d != nullptr.
-// tp (FP32 d only): fold the template correction -P^T (W T) b of the deprojected right-hand side into
-// the same pass, with b already solved by launch_tpl_rhs_amplitudes.
-furax_status launch_chi2_df(const furax_pointing *p, const furax_noise *n, const void *d, int d_t, const double *m,
-                            double *chi2, double *grad_map, double *grad_psi, cudaStream_t st);
-furax_status launch_fused_df(const furax_pointing *p, const furax_noise *n, const double *x, const void *d, int d_t,
-                             double *acc64, cudaStream_t st, const furax_templates *tp = nullptr);
-// b = P^T N^-1 d accumulated into acc64 (FP64 stencil)
-furax_status launch_rhs_f64(const furax_pointing *p, const furax_noise *n, const void *d, int d_t, double *acc64,
-                            cudaStream_t st);
+// FP64-accurate operator and right-hand side (fused_tc.cu): acc64 += P^T N^-1 P S^T x (valid may be NULL:
+// every pixel) and acc64 += P^T N^-1 d. tp: the template correction -P^T (W T) b is folded into the same pass,
+// with b already solved by launch_tpl_rhs_amplitudes. f64: tiles outside the digits' range take the FP64
+// FMA chain, else the compensated double-FP32 product (band_tc.cuh).
+furax_status launch_fused_tc(const furax_pointing *p, const furax_noise *n, const double *x, const uint8_t *valid, double *acc64,
+                             bool f64, cudaStream_t st);
+furax_status launch_rhs_tc(const furax_pointing *p, const furax_noise *n, const void *d, int d_t, double *acc64, bool f64,
+                           cudaStream_t st, const furax_templates *tp = nullptr);
+// ws_x4 = x (zero where valid is 0) in 32-byte records.
+furax_status launch_pack_x4(const furax_pointing *p, const double *x, const uint8_t *valid, cudaStream_t st);
+furax_status launch_chi2_tc(const furax_pointing *p, const furax_noise *n, const void *d, int d_t, const double *m,
+                            double *chi2, double *grad_map, double *grad_psi, bool f64, cudaStream_t st);
 
 // ---- vector helpers (solver.cu)
 furax_status launch_pack_x32(const furax_pointing *p, const double *x, const uint8_t *valid, float4 *x32,

@@ -233,18 +233,15 @@ furax_status ptnp_apply(const furax_pointing *p, const furax_noise *n, const dou
     }
     if (precision == FURAX_F64 || precision == FURAX_PREC_F32X2) {
         if ((rc = ensure_ws(pm, (void **)&pm->ws_acc64, sizeof(double) * 3 * np))) return rc;
-        const double *xin = x;
-        if (valid) {
+        const double *xin = x;   // the templates' pass reads a masked map
+        if (valid && tp) {
             if ((rc = ensure_ws(pm, (void **)&pm->ws_x64, sizeof(double) * 3 * np))) return rc;
             if ((rc = launch_mask_copy(p, x, valid, pm->ws_x64, st))) return rc;
             xin = pm->ws_x64;
         }
         if ((rc = check_cuda(cudaMemsetAsync(pm->ws_acc64, 0, sizeof(double) * 3 * np, st), "memset"))) return rc;
-        if (precision == FURAX_F64) {
-            if ((rc = timed(1, st, [&] { return launch_fused_f64(p, n, xin, pm->ws_acc64, st); }))) return rc;
-        } else {
-            if ((rc = timed(2, st, [&] { return launch_fused_df(p, n, xin, nullptr, 0, pm->ws_acc64, st); }))) return rc;
-        }
+        const bool f64 = precision == FURAX_F64;
+        if ((rc = timed(f64 ? 1 : 2, st, [&] { return launch_fused_tc(p, n, x, valid, pm->ws_acc64, f64, st); }))) return rc;
         if (tp && (rc = launch_tpl_map(tp, FURAX_F64, FURAX_ACC_F64, nullptr, xin, nullptr, nullptr, pm->ws_acc64, st)))
             return rc;
         return launch_finalize_acc(p, FURAX_ACC_F64, nullptr, nullptr, pm->ws_acc64, valid, out, st);
@@ -588,7 +585,7 @@ static furax_status body(const Body &b, cudaStream_t st, cudaEvent_t e0, cudaEve
             return rc;
         acc = FURAX_ACC_F64;
     } else if (b.precision == FURAX_F64) {
-        if ((rc = launch_fused_f64(p, b.n, w->p, w->acc64, st))) return rc;
+        if ((rc = launch_fused_tc(p, b.n, w->p, nullptr, w->acc64, true, st))) return rc;
         acc = FURAX_ACC_F64;
     } else {
         FusedTpl ft{0, nullptr, 0, 0};
@@ -645,7 +642,7 @@ static int64_t graph_nodes_per_iter(const Body &b)
 {
     if (b.aug) return 6;
     const bool lb = long_band(b.n);
-    int64_t k = 5 + (lb ? 3 : 1);
+    int64_t k = 5 + (lb ? 3 : b.precision == FURAX_F64 ? 2 : 1);
     if (b.tp) k += (!lb && b.precision != FURAX_F64 && tpl_fused_target(b.tp, b.p)) ? 2 : 3;
     return k;
 }
@@ -748,14 +745,11 @@ static furax_status true_residual(const Body &b, const double *x, double *rtrue,
     const furax_pointing *p = b.p;
     furax_status rc;
     if ((rc = check_cuda(cudaMemsetAsync(w->acc64, 0, sizeof(double) * 3 * p->npix_total, st), "memset"))) return rc;
-    // The plain FP64 solve checks itself with the FP64 operator; the mixed solve with the
-    // FP64-accurate double-FP32 operator (same system, ~2^-48 arithmetic, FP32 pipes).
     if (long_band(b.n)) {
         if ((rc = launch_ata_chain(p, b.n, x, FURAX_F64, w->acc64, st))) return rc;
-    } else if (b.precision == FURAX_F64) {
-        if ((rc = timed(1, st, [&] { return launch_fused_f64(p, b.n, x, w->acc64, st); }))) return rc;
     } else {
-        if ((rc = timed(2, st, [&] { return launch_fused_df(p, b.n, x, nullptr, 0, w->acc64, st); }))) return rc;
+        const bool f64 = b.precision == FURAX_F64;
+        if ((rc = timed(f64 ? 1 : 2, st, [&] { return launch_fused_tc(p, b.n, x, nullptr, w->acc64, f64, st); }))) return rc;
     }
     if (b.tp && (rc = launch_tpl_map(b.tp, FURAX_F64, FURAX_ACC_F64, nullptr, x, nullptr, nullptr, w->acc64, st)))
         return rc;
@@ -785,6 +779,8 @@ furax_status mapmaker_cg(const furax_pointing *p, const furax_noise *n, const vo
     furax_status rc;
     if ((rc = get_ws(pm, o->maxiter + 1, &w))) return rc;
     const int64_t np = p->npix_total;
+    // the FP64-accurate operator's map records exist before any stream capture of the iteration
+    if (!long_band(n) && (rc = ensure_ws(pm, (void **)&pm->ws_x4, sizeof(double4_32a) * (size_t)np))) return rc;
     const unsigned pg = (unsigned)std::max<int64_t>(1, p->n_ptiles);
 
     const AllReduce ar{o->allreduce, o->allreduce_user};
@@ -796,19 +792,17 @@ furax_status mapmaker_cg(const furax_pointing *p, const furax_noise *n, const vo
     if (o->d_ready && (rc = check_cuda(cudaStreamWaitEvent(st, (cudaEvent_t)o->d_ready, 0), "wait for d")))
         return rc;
     if ((rc = check_cuda(cudaMemsetAsync(w->acc64, 0, sizeof(double) * 3 * np, st), "memset"))) return rc;
-    // the double-FP32 pass from FP32 data subtracts the template correction itself, with the
-    // amplitudes solved beforehand
-    const bool tpl_folded = tp && !long_band(n) && o->precision != FURAX_F64 && d_t == FURAX_F32;
+    // the pass that forms P^T N^-1 d subtracts the template correction itself, with the amplitudes
+    // solved beforehand
+    const bool tpl_folded = tp && !long_band(n);
     if (tpl_folded && (rc = launch_tpl_rhs_amplitudes(tp, d, d_t, st))) return rc;
     if (long_band(n)) {
         // TOD workspaces exist before any stream capture of the iteration
         if ((rc = tod_ws(p))) return rc;
         if ((rc = launch_rhs_chain(p, n, d, d_t, w->acc64, st))) return rc;
-    } else if (o->precision == FURAX_F64) {
-        if ((rc = timed(1, st, [&] { return launch_rhs_f64(p, n, d, d_t, w->acc64, st); }))) return rc;
-    } else {
-        if ((rc = timed(2, st, [&] { return launch_fused_df(p, n, nullptr, d, d_t, w->acc64, st, tpl_folded ? tp : nullptr); })))
-            return rc;
+    } else if ((rc = timed(o->precision == FURAX_F64 ? 1 : 2, st,
+                           [&] { return launch_rhs_tc(p, n, d, d_t, w->acc64, o->precision == FURAX_F64, st, tp); }))) {
+        return rc;
     }
     if (tp && !tpl_folded && (rc = launch_tpl_rhs(tp, d, d_t, w->acc64, st))) return rc;
     if (ar.on() && (rc = ar(w->acc64, 3 * np, FURAX_REDUCE_F64, st))) return rc;

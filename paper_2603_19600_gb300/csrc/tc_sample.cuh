@@ -1,0 +1,214 @@
+// Per-sample pointing and data in FP64 for the tensor-core tile kernels (fused_tc.cu, chi2_tc.cu). The
+// loads of a sample are unconditional (clamped indices), so that a thread's samples can be in flight
+// together; FP32 words widen on the integer pipe.
+#pragma once
+#include "band_tc.cuh"
+
+namespace fx {
+
+// FP32 -> FP64 without a conversion instruction (the FP64 pipe is scarce) and without a branch, for
+// cached weights: finite, and words below 2^-126 count as zero (an absolute error of 1e-38).
+__device__ __forceinline__ double weight_f64(float f)
+{
+    const uint32_t b = __float_as_uint(f);
+    const uint32_t hi = ((b & 0x7fffffffu) >> 3) + 0x38000000u;
+    return (b & 0x7f800000u) ? __hiloint2double((int)(hi | (b & 0x80000000u)), (int)(b << 29)) : 0.0;
+}
+
+struct TcPsi {   // the detector's offset rotation
+    double c2 = 1.0, s2 = 0.0;
+    bool on = false;
+    __device__ __forceinline__ TcPsi(const PointingView &pv, int64_t gdet)
+    {
+        if (pv.psi_cs) { const double2 cs = pv.psi_cs[gdet]; c2 = cs.x; s2 = cs.y; on = true; }
+    }
+};
+
+// The cached words of one sample's weights as they are stored, so that their loads need not be waited for
+// one by one.
+template <int MODE> struct TcRaw { float c, s; };
+template <> struct TcRaw<2> { double c, s; };
+template <> struct TcRaw<3> { float c, s, cl, sl; };
+
+template <int MODE>
+__device__ __forceinline__ TcRaw<MODE> tc_load(const PointingView &pv, int64_t i)
+{
+    if constexpr (MODE == 2) return {__ldg(pv.c64 + i), __ldg(pv.s64 + i)};
+    else if constexpr (MODE == 3) return {__ldg(pv.c32 + i), __ldg(pv.s32 + i), __ldg(pv.c32lo + i), __ldg(pv.s32lo + i)};
+    else return {__ldg(pv.c32 + i), __ldg(pv.s32 + i)};
+}
+
+template <int MODE>
+__device__ __forceinline__ void tc_weights(const TcRaw<MODE> &w, const TcPsi &psi, double &c, double &s)
+{
+    if constexpr (MODE == 2) {
+        c = w.c;
+        s = w.s;
+    } else {
+        c = weight_f64(w.c);
+        s = weight_f64(w.s);
+        if constexpr (MODE == 3) {
+            c += weight_f64(w.cl);
+            s += weight_f64(w.sl);
+        }
+    }
+    if (psi.on) {
+        const double r = c * psi.c2 - s * psi.s2;
+        s = s * psi.c2 + c * psi.s2;
+        c = r;
+    }
+}
+
+template <typename DT>
+__device__ __forceinline__ double tod_f64(DT v)
+{
+    if constexpr (sizeof(DT) == 8) return v;
+    else return f32_to_f64_bits(v);
+}
+
+// One pixel of an FP64 map padded to 32-byte records (I, Q, U, 0): one 32-byte load and one L2 sector per
+// random gather, where a 24-byte record takes two or three loads and 1.5 sectors (fill phase of the normal
+// operator: 43,600 cycles per tile with three loads, sample by sample; 30,200 with two and the batches below;
+// 25,700 with this; the pass that packs the map costs 8 us at nside 256).
+struct TcPix {
+    double i, q, u;
+    __device__ __forceinline__ void load(const double4_32a *__restrict__ x4, int64_t gp)
+    {
+        double pad;
+        asm("ld.global.nc.v4.f64 {%0, %1, %2, %3}, [%4];" : "=d"(i), "=d"(q), "=d"(u), "=d"(pad) : "l"(x4 + gp));
+    }
+    __device__ __forceinline__ double project(int32_t pix, double c, double s) const
+    {
+        return pix >= 0 ? fma(u, s, fma(q, c, i)) : 0.0;
+    }
+};
+
+// The tile's slots that lie in the stream: [tc_in0, tc_in1).
+__device__ __forceinline__ int tc_in0(const Tile &tl) { return tl.t0 < kHalo ? (int)(kHalo - tl.t0) : 0; }
+__device__ __forceinline__ int tc_in1(const Tile &tl, const ObsInfo &ob)
+{
+    return (int)min((int64_t)(tl.len + 2 * kHalo), ob.nsamp - tl.t0 + kHalo);
+}
+
+// This thread's slot k and the sample it stands for, clamped into the tile's loaded range.
+struct TcSlots {
+    int64_t row;   // flat index of slot 0
+    int in0, in1;
+    __device__ __forceinline__ TcSlots(const Tile &tl, const ObsInfo &ob)
+        : row(ob.tod_off + (int64_t)tl.det * ob.nsamp + tl.t0 - kHalo), in0(tc_in0(tl)), in1(tc_in1(tl, ob))
+    {
+    }
+    __device__ __forceinline__ int slot(int k) const { return (int)threadIdx.x + k * FT; }
+    __device__ __forceinline__ bool in(int k) const { return slot(k) >= in0 && slot(k) < in1; }
+    __device__ __forceinline__ int64_t index(int k) const { return row + max(in0, min(slot(k), in1 - 1)); }
+};
+
+// v[k] = time-ordered data of this thread's slots (zero outside the stream): every load in flight at once.
+template <typename DT>
+__device__ __forceinline__ void tc_fill_tod(double (&v)[kTcPer], const TcSlots &sl, const DT *__restrict__ d)
+{
+    DT raw[kTcPer];
+#pragma unroll
+    for (int k = 0; k < kTcPer; ++k) raw[k] = __ldg(d + sl.index(k));
+#pragma unroll
+    for (int k = 0; k < kTcPer; ++k) v[k] = sl.in(k) ? tod_f64(raw[k]) : 0.0;
+}
+
+// v[k] = (P x)_t, or d_t - (P x)_t with RESID, of this thread's slots. Cached pointing: every pixel index is
+// loaded first, then weights, data and map records a few samples at a time (registers). On the fly: one
+// sample at a time (the FP64 recipe is too long to unroll), through shared memory.
+template <int MODE, bool RESID, typename DT>
+__device__ __forceinline__ void tc_fill_map(unsigned char *sm, double (&v)[kTcPer], const TcSlots &sl, const PointingView &pv,
+                                            const ObsInfo &ob, const Tile &tl, const TcPsi &psi,
+                                            const double4_32a *__restrict__ x, const DT *__restrict__ d)
+{
+    if constexpr (MODE == 0) {
+        double *tmp = tc_ys(sm);   // read back by the thread that wrote it
+#pragma unroll 1
+        for (int k = 0; k < kTcPer; ++k) {
+            double r = 0.0;
+            if (sl.in(k)) {
+                double c, s;
+                const int32_t pix = get_sample<0, double>(pv, ob, tl.det, tl.t0 - kHalo + sl.slot(k), c, s);
+                TcPix m;
+                m.load(x, ob.map_off + max(pix, 0));
+                r = m.project(pix, c, s);
+                if constexpr (RESID) r = tod_f64(__ldg(d + sl.index(k))) - r;
+            }
+            tmp[sl.slot(k)] = r;
+        }
+#pragma unroll
+        for (int k = 0; k < kTcPer; ++k) v[k] = tmp[sl.slot(k)];
+    } else {
+        constexpr int B = RESID ? 4 : 5;
+        int32_t pix[kTcPer];
+#pragma unroll
+        for (int k = 0; k < kTcPer; ++k) pix[k] = __ldg(pv.pix + sl.index(k));
+#pragma unroll
+        for (int k0 = 0; k0 < kTcPer; k0 += B) {
+            TcRaw<MODE> w[B];
+            TcPix m[B];
+            DT dd[B];
+#pragma unroll
+            for (int b = 0; b < B; ++b) {
+                const int k = k0 + b;
+                if (k < kTcPer) {
+                    w[b] = tc_load<MODE>(pv, sl.index(k));
+                    m[b].load(x, ob.map_off + max(pix[k], 0));
+                    if constexpr (RESID) dd[b] = __ldg(d + sl.index(k));
+                }
+            }
+#pragma unroll
+            for (int b = 0; b < B; ++b) {
+                const int k = k0 + b;
+                if (k < kTcPer) {
+                    double c, s;
+                    tc_weights<MODE>(w[b], psi, c, s);
+                    double r = m[b].project(pix[k], c, s);
+                    if constexpr (RESID) r = tod_f64(dd[b]) - r;
+                    v[k] = sl.in(k) ? r : 0.0;
+                }
+            }
+        }
+    }
+}
+static_assert(sizeof(double) * kTcPer * FT <= kTcOffCtl - kTcOffX, "the on-the-fly fill fits the samples' region");
+
+// Core samples of the tile in time order, 32 consecutive ones per warp: f(k, pix, c, s) for every lane of
+// a warp together (pix = -1 past the tile or without a pixel). The pointing of eight samples per thread
+// is loaded before the first is used.
+template <int MODE, typename F>
+__device__ __forceinline__ void tc_each(const PointingView &pv, const ObsInfo &ob, const Tile &tl, const TcPsi &psi, F &&f)
+{
+    const int64_t row = ob.tod_off + (int64_t)tl.det * ob.nsamp + tl.t0;
+    if constexpr (MODE == 0) {
+#pragma unroll 1
+        for (int k = threadIdx.x; k - (int)(threadIdx.x & 31) < tl.len; k += FT) {
+            double c = 0.0, s = 0.0;
+            const int32_t pix = k < tl.len ? get_sample<0, double>(pv, ob, tl.det, tl.t0 + k, c, s) : -1;
+            f(k, pix, c, s);
+        }
+    } else {
+        constexpr int B = 8;
+#pragma unroll 1
+        for (int k0 = threadIdx.x; k0 - (int)(threadIdx.x & 31) < tl.len; k0 += B * FT) {
+            int32_t pix[B];
+            TcRaw<MODE> w[B];
+#pragma unroll
+            for (int b = 0; b < B; ++b) {
+                const int64_t i = row + min(k0 + b * FT, tl.len - 1);
+                pix[b] = __ldg(pv.pix + i);
+                w[b] = tc_load<MODE>(pv, i);
+            }
+#pragma unroll
+            for (int b = 0; b < B; ++b) {
+                const int k = k0 + b * FT;
+                double c, s;
+                tc_weights<MODE>(w[b], psi, c, s);
+                f(k, k < tl.len ? pix[b] : -1, c, s);
+            }
+        }
+    }
+}
+
+}  // namespace fx

@@ -11,8 +11,8 @@
 //   project  a_det = (W T)^T u over the detector's stream (u = P x, or a TOD),
 //   solve    b_det = G_det^-1 a_det,
 //   scatter  acc -= P^T (W T) b   (or, for a TOD, y -= (W T) b).
-// For the right-hand side of FP32 data in the mixed-precision solver the scatter is not a pass of
-// its own: the double-FP32 pass that forms P^T W d subtracts (W T) b from W d per sample.
+// For the right-hand side the scatter is not a pass of its own: the pass that forms P^T W d subtracts
+// (W T) b from W d per sample (short bands).
 //
 // (W T)(t) needs no band product. For a polynomial p of degree <= 3 and a symmetric band whose
 // full width fits around t,

@@ -35,12 +35,10 @@ __device__ __forceinline__ T white_scale(const NoiseView &nv, int64_t gdet)
 }
 
 constexpr size_t kF32Smem = sizeof(float) * (XS + MAXTAPS + 2 * XS) + sizeof(int32_t) * XS;
-constexpr size_t kF64Smem = sizeof(double) * (XS + MAXTAPS + 2 * CS) + sizeof(int32_t) * CS;
 
 // Kernel shared-memory setup for each translation unit (called once, outside stream capture).
 furax_status prepare_fused_f32();
-furax_status prepare_fused_f64();
-furax_status prepare_fused_df();
+furax_status prepare_fused_tc();
 furax_status prepare_fused_tma();
 
 // Cached FP32 pointing: persistent TMA-pipelined operator (cache rows must be readable up to the

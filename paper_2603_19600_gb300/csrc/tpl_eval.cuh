@@ -1,5 +1,5 @@
 // Evaluation of the Legendre templates and of W applied to them, shared by the template kernels
-// and by the double-FP32 right-hand-side kernel that folds the template correction in.
+// and by the right-hand-side kernel that folds the template correction in.
 //
 // For a polynomial p of degree <= 3 and a symmetric band of half-width halo whose full width fits
 // around sample t,
