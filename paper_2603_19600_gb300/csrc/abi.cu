@@ -138,6 +138,11 @@ void build_layout(const furax_obs_desc *desc, Layout &L)
 {
     int64_t det = 0, bore = 0, tod = 0, map = 0, ptile = 0;
     std::unordered_map<int32_t, int> first_of;   // map_id -> first observation with it
+    for (int i = 0; i < desc->n_obs; ++i)
+        if (!desc->map_id || first_of.emplace(desc->map_id[i], i).second) map += 12LL * desc->nside[i] * desc->nside[i];
+    L.ptile = pixel_tile(map);
+    map = 0;
+    first_of.clear();
     for (int i = 0; i < desc->n_obs; ++i) {
         ObsInfo o{};
         o.nsamp = desc->nsamp[i];
@@ -154,12 +159,12 @@ void build_layout(const furax_obs_desc *desc, Layout &L)
         } else {
             o.map_off = map;
             o.ptile0 = ptile;
-            o.nptile = (int32_t)((o.npix + PTILE - 1) / PTILE);
+            o.nptile = (int32_t)((o.npix + L.ptile - 1) / L.ptile);
             for (int64_t k = 0; k < o.nptile; ++k) {
                 PTile t;
-                t.p0 = map + k * PTILE;
+                t.p0 = map + k * L.ptile;
                 t.obs = i;
-                t.len = (int32_t)std::min<int64_t>(PTILE, o.npix - k * PTILE);
+                t.len = (int32_t)std::min<int64_t>(L.ptile, o.npix - k * L.ptile);
                 L.ptiles.push_back(t);
             }
             map += o.npix;
@@ -374,6 +379,7 @@ furax_status furax_pointing_create(const furax_obs_desc *desc, int32_t mode, voi
     p->obs = L.obs; p->tiles = L.tiles; p->ptiles = L.ptiles;
     p->ndet_total = L.ndet; p->nbore_total = L.nbore; p->nsamp_total = L.nsamp; p->npix_total = L.npix;
     p->max_ndet = L.max_ndet;
+    p->ptile = L.ptile;
     const int64_t det = L.ndet, tod = L.nsamp;
     p->n_tiles = (int64_t)p->tiles.size();
     p->n_ptiles = (int64_t)p->ptiles.size();

@@ -226,7 +226,7 @@ bool fused_f32_projects_templates(const furax_pointing *p)
 }
 
 furax_status launch_fused_f32(const furax_pointing *p, const furax_noise *n, const float4 *x32, int acc, float4 *hi,
-                              float4 *lo, double *a64, cudaStream_t st, const FusedTpl *ft)
+                              float4 *lo, double *a64, cudaStream_t st, const FusedTpl *ft, const unsigned *done)
 {
     if (p->n_tiles == 0) return FURAX_OK;
     furax_status rc;
@@ -247,7 +247,7 @@ furax_status launch_fused_f32(const furax_pointing *p, const furax_noise *n, con
              sorted_active(p) && !long_band(n))
         rc = launch_fused_sorted(p, n, x32, acc, hi, lo, a64, st);   // pixel-sorted schedule
     else if (p->mode == FURAX_POINTING_CACHE_F32 || p->mode == FURAX_POINTING_CACHE_MIXED)  // FP32 weights: hi
-        rc = launch_fused_tma(p, n, x32, acc, hi, lo, a64, st, ft);
+        rc = launch_fused_tma(p, n, x32, acc, hi, lo, a64, st, ft, done);
     else rc = dispatch_fused_f32<2>(p, n, x32, acc, hi, lo, a64, st);
     if (rc) return rc;
     count_launches(1);

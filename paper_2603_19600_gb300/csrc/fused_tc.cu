@@ -53,10 +53,11 @@ template <int MODE, bool FROM_TOD, bool TPL, typename DT>
 __global__ void __launch_bounds__(FT, 2) tc_operator_kernel(const Tile *__restrict__ tiles, PointingView pv, NoiseView nv,
                                                             const double4_32a *__restrict__ x, const DT *__restrict__ d,
                                                             double *__restrict__ acc64, unsigned *__restrict__ err,
-                                                            bool f64, TplView tv)
+                                                            bool f64, TplView tv, const unsigned *__restrict__ done, unsigned n_obs)
 {
     extern __shared__ __align__(128) unsigned char sm[];
     __shared__ TplCorr corr;
+    if (done && *done == n_obs) return;
     const Tile tl = tiles[blockIdx.x];
     const ObsInfo ob = pv.obs[tl.obs];
     const int64_t gdet = ob.det_off + tl.det;
@@ -86,12 +87,15 @@ __global__ void __launch_bounds__(FT, 2) tc_operator_kernel(const Tile *__restri
 template <int MODE, bool FROM_TOD, bool TPL, typename DT>
 __global__ void __launch_bounds__(FT) white_operator_kernel(const Tile *__restrict__ tiles, PointingView pv, NoiseView nv,
                                                             const double4_32a *__restrict__ x, const DT *__restrict__ d,
-                                                            double *__restrict__ acc64, TplView tv)
+                                                            double *__restrict__ acc64, TplView tv,
+                                                            const unsigned *__restrict__ done, unsigned n_obs)
 {
     __shared__ double stage[FT / 32][96];
     __shared__ int32_t spix[FT / 32][32];
     __shared__ TplCorr corr;
-    const Tile tl = tiles[blockIdx.x];
+    if (done && *done == n_obs) return;
+    const Tile tl = tile_part(tiles[blockIdx.x]);
+    if (tl.len <= 0) return;
     const ObsInfo ob = pv.obs[tl.obs];
     const int64_t gdet = ob.det_off + tl.det;
     const TcPsi psi(pv, gdet);
@@ -151,27 +155,28 @@ furax_status launch_ninv_tc(const furax_noise *n, const double *in, double *out,
 
 template <int MODE, bool FROM_TOD, bool TPL, typename DT>
 static furax_status run_tc(const furax_pointing *p, const furax_noise *n, const double4_32a *x, const DT *d, double *a64,
-                           bool f64, const TplView &tv, cudaStream_t st)
+                           bool f64, const TplView &tv, const unsigned *done, cudaStream_t st)
 {
     if (n->kind == FURAX_NOISE_BANDED)
         return launch_dyn(tc_operator_kernel<MODE, FROM_TOD, TPL, DT>, (unsigned)p->n_tiles, FT, kTcSmem, st, p->d_tiles,
-                          p->view(), n->view(), x, d, a64, p->d_err, f64, tv);
-    white_operator_kernel<MODE, FROM_TOD, TPL, DT><<<(unsigned)p->n_tiles, FT, 0, st>>>(p->d_tiles, p->view(), n->view(), x,
-                                                                                         d, a64, tv);
+                          p->view(), n->view(), x, d, a64, p->d_err, f64, tv, done, (unsigned)p->n_obs);
+    white_operator_kernel<MODE, FROM_TOD, TPL, DT><<<tile_grid(p), FT, 0, st>>>(p->d_tiles, p->view(), n->view(), x,
+                                                                                         d, a64, tv, done,
+                                                                                         (unsigned)p->n_obs);
     return FURAX_OK;
 }
 
 template <bool FROM_TOD, bool TPL, typename DT>
 static furax_status dispatch_tc(const furax_pointing *p, const furax_noise *n, const double4_32a *x, const DT *d, double *a64,
-                                bool f64, const TplView &tv, cudaStream_t st)
+                                bool f64, const TplView &tv, const unsigned *done, cudaStream_t st)
 {
     if (p->n_tiles == 0) return FURAX_OK;
     furax_status rc;
     switch (p->mode) {
-    case FURAX_POINTING_ON_THE_FLY: rc = run_tc<0, FROM_TOD, TPL, DT>(p, n, x, d, a64, f64, tv, st); break;
-    case FURAX_POINTING_CACHE_F32: rc = run_tc<1, FROM_TOD, TPL, DT>(p, n, x, d, a64, f64, tv, st); break;
-    case FURAX_POINTING_CACHE_MIXED: rc = run_tc<3, FROM_TOD, TPL, DT>(p, n, x, d, a64, f64, tv, st); break;
-    default: rc = run_tc<2, FROM_TOD, TPL, DT>(p, n, x, d, a64, f64, tv, st);
+    case FURAX_POINTING_ON_THE_FLY: rc = run_tc<0, FROM_TOD, TPL, DT>(p, n, x, d, a64, f64, tv, done, st); break;
+    case FURAX_POINTING_CACHE_F32: rc = run_tc<1, FROM_TOD, TPL, DT>(p, n, x, d, a64, f64, tv, done, st); break;
+    case FURAX_POINTING_CACHE_MIXED: rc = run_tc<3, FROM_TOD, TPL, DT>(p, n, x, d, a64, f64, tv, done, st); break;
+    default: rc = run_tc<2, FROM_TOD, TPL, DT>(p, n, x, d, a64, f64, tv, done, st);
     }
     if (rc) return rc;
     count_launches(1);
@@ -199,12 +204,18 @@ furax_status launch_pack_x4(const furax_pointing *p, const double *x, const uint
     return check_launch("pack FP64 map");
 }
 
+furax_status launch_fused_tc_packed(const furax_pointing *p, const furax_noise *n, double *a64, bool f64,
+                                    const unsigned *done, cudaStream_t st)
+{
+    return dispatch_tc<false, false, double>(p, n, p->ws_x4, nullptr, a64, f64, TplView{}, done, st);
+}
+
 furax_status launch_fused_tc(const furax_pointing *p, const furax_noise *n, const double *x, const uint8_t *valid, double *a64,
                              bool f64, cudaStream_t st)
 {
     furax_status rc = launch_pack_x4(p, x, valid, st);
     if (rc) return rc;
-    return dispatch_tc<false, false, double>(p, n, p->ws_x4, nullptr, a64, f64, TplView{}, st);
+    return launch_fused_tc_packed(p, n, a64, f64, nullptr, st);
 }
 
 furax_status launch_rhs_tc(const furax_pointing *p, const furax_noise *n, const void *d, int d_t, double *a64, bool f64,
@@ -214,11 +225,11 @@ furax_status launch_rhs_tc(const furax_pointing *p, const furax_noise *n, const 
     const float *d32 = (const float *)d;
     if (tp) {
         const TplView tv = tp->view();
-        return d_t == FURAX_F64 ? dispatch_tc<true, true, double>(p, n, nullptr, d64, a64, f64, tv, st)
-                                : dispatch_tc<true, true, float>(p, n, nullptr, d32, a64, f64, tv, st);
+        return d_t == FURAX_F64 ? dispatch_tc<true, true, double>(p, n, nullptr, d64, a64, f64, tv, nullptr, st)
+                                : dispatch_tc<true, true, float>(p, n, nullptr, d32, a64, f64, tv, nullptr, st);
     }
-    return d_t == FURAX_F64 ? dispatch_tc<true, false, double>(p, n, nullptr, d64, a64, f64, TplView{}, st)
-                            : dispatch_tc<true, false, float>(p, n, nullptr, d32, a64, f64, TplView{}, st);
+    return d_t == FURAX_F64 ? dispatch_tc<true, false, double>(p, n, nullptr, d64, a64, f64, TplView{}, nullptr, st)
+                            : dispatch_tc<true, false, float>(p, n, nullptr, d32, a64, f64, TplView{}, nullptr, st);
 }
 
 // Digits of a detector's taps (one CTA each): integers relative to 2^ec, balanced base-256

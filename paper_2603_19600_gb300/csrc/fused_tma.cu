@@ -135,8 +135,10 @@ template <int ACC, bool BANDED, int TPL, int KC>
 __global__ void __launch_bounds__(tma_threads<KC>(), 1)
     fused_tma_kernel(const Tile *__restrict__ tiles, int64_t n_tiles, PointingView pv, NoiseView nv,
                      const float4 *__restrict__ x32, float4 *__restrict__ acc_hi, float4 *__restrict__ acc_lo,
-                     double *__restrict__ acc64, unsigned *__restrict__ err, FusedTpl tpl, int l2_hint)
+                     double *__restrict__ acc64, unsigned *__restrict__ err, FusedTpl tpl, int l2_hint,
+                     const unsigned *__restrict__ done, unsigned n_obs)
 {
+    if (done && *done == n_obs) return;   // a PCG iteration after every observation has converged
     constexpr int kTmaConsumer = KC;
     constexpr int kConsOut = cons_out<KC>();
     extern __shared__ __align__(128) unsigned char tsm[];
@@ -390,47 +392,48 @@ __global__ void __launch_bounds__(tma_threads<KC>(), 1)
 
 template <int ACC, bool BANDED, int TPL, int KC>
 static furax_status run_tma_kc(const furax_pointing *p, const furax_noise *n, const float4 *x32, float4 *hi,
-                               float4 *lo, double *a64, const FusedTpl &ft, cudaStream_t st)
+                               float4 *lo, double *a64, const FusedTpl &ft, const unsigned *done, cudaStream_t st)
 {
     const unsigned g = (unsigned)std::min<int64_t>(p->n_tiles, p->n_sm);
     return launch_dyn(fused_tma_kernel<ACC, BANDED, TPL, KC>, g, tma_threads<KC>(), tma_smem<ACC, KC>(), st, p->d_tiles,
-                      p->n_tiles, p->view(), n->view(), x32, hi, lo, a64, p->d_err, ft, (int)p->sched.l2_evict_first);
+                      p->n_tiles, p->view(), n->view(), x32, hi, lo, a64, p->d_err, ft, (int)p->sched.l2_evict_first,
+                      done, (unsigned)p->n_obs);
 }
 
 // 16 consumer warps when the schedule asks for them (plain operator only; the template modes keep 8).
 template <int ACC, bool BANDED, int TPL>
 static furax_status run_tma(const furax_pointing *p, const furax_noise *n, const float4 *x32, float4 *hi, float4 *lo,
-                            double *a64, const FusedTpl &ft, cudaStream_t st)
+                            double *a64, const FusedTpl &ft, const unsigned *done, cudaStream_t st)
 {
     if constexpr (TPL == 0)
-        if (p->sched.consumer_warps == 16) return run_tma_kc<ACC, BANDED, TPL, 16>(p, n, x32, hi, lo, a64, ft, st);
-    return run_tma_kc<ACC, BANDED, TPL, 8>(p, n, x32, hi, lo, a64, ft, st);
+        if (p->sched.consumer_warps == 16) return run_tma_kc<ACC, BANDED, TPL, 16>(p, n, x32, hi, lo, a64, ft, done, st);
+    return run_tma_kc<ACC, BANDED, TPL, 8>(p, n, x32, hi, lo, a64, ft, done, st);
 }
 
 template <bool BANDED, int TPL>
 static furax_status dispatch_tma(const furax_pointing *p, const furax_noise *n, const float4 *x32, int acc, float4 *hi,
-                                 float4 *lo, double *a64, const FusedTpl &ft, cudaStream_t st)
+                                 float4 *lo, double *a64, const FusedTpl &ft, const unsigned *done, cudaStream_t st)
 {
-    if (acc == FURAX_ACC_F32) return run_tma<FURAX_ACC_F32, BANDED, TPL>(p, n, x32, hi, lo, a64, ft, st);
-    if (acc == FURAX_ACC_F32_KAHAN) return run_tma<FURAX_ACC_F32_KAHAN, BANDED, TPL>(p, n, x32, hi, lo, a64, ft, st);
-    return run_tma<FURAX_ACC_F64, BANDED, TPL>(p, n, x32, hi, lo, a64, ft, st);
+    if (acc == FURAX_ACC_F32) return run_tma<FURAX_ACC_F32, BANDED, TPL>(p, n, x32, hi, lo, a64, ft, done, st);
+    if (acc == FURAX_ACC_F32_KAHAN) return run_tma<FURAX_ACC_F32_KAHAN, BANDED, TPL>(p, n, x32, hi, lo, a64, ft, done, st);
+    return run_tma<FURAX_ACC_F64, BANDED, TPL>(p, n, x32, hi, lo, a64, ft, done, st);
 }
 
 template <int TPL>
 static furax_status dispatch_tma_band(const furax_pointing *p, const furax_noise *n, const float4 *x32, int acc,
-                                      float4 *hi, float4 *lo, double *a64, const FusedTpl &ft, cudaStream_t st)
+                                      float4 *hi, float4 *lo, double *a64, const FusedTpl &ft, const unsigned *done, cudaStream_t st)
 {
-    return n->kind == FURAX_NOISE_BANDED ? dispatch_tma<true, TPL>(p, n, x32, acc, hi, lo, a64, ft, st)
-                                         : dispatch_tma<false, TPL>(p, n, x32, acc, hi, lo, a64, ft, st);
+    return n->kind == FURAX_NOISE_BANDED ? dispatch_tma<true, TPL>(p, n, x32, acc, hi, lo, a64, ft, done, st)
+                                         : dispatch_tma<false, TPL>(p, n, x32, acc, hi, lo, a64, ft, done, st);
 }
 
 furax_status launch_fused_tma(const furax_pointing *p, const furax_noise *n, const float4 *x32, int acc, float4 *hi,
-                              float4 *lo, double *a64, cudaStream_t st, const FusedTpl *ft)
+                              float4 *lo, double *a64, cudaStream_t st, const FusedTpl *ft, const unsigned *done)
 {
     const FusedTpl none{0, nullptr, 0, 0};
-    if (!ft || ft->mode == 0) return dispatch_tma_band<0>(p, n, x32, acc, hi, lo, a64, none, st);
-    if (ft->mode == 1) return dispatch_tma_band<1>(p, n, x32, acc, hi, lo, a64, *ft, st);
-    return dispatch_tma_band<2>(p, n, x32, acc, hi, lo, a64, *ft, st);
+    if (!ft || ft->mode == 0) return dispatch_tma_band<0>(p, n, x32, acc, hi, lo, a64, none, done, st);
+    if (ft->mode == 1) return dispatch_tma_band<1>(p, n, x32, acc, hi, lo, a64, *ft, done, st);
+    return dispatch_tma_band<2>(p, n, x32, acc, hi, lo, a64, *ft, done, st);
 }
 
 template <bool BANDED, int TPL, int KC>

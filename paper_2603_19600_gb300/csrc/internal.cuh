@@ -12,7 +12,11 @@
 namespace fx {
 
 constexpr int TILE = 4096;      // samples per work tile (one detector, contiguous in time)
-constexpr int PTILE = 4096;     // pixels per pixel tile (vector kernels, per-observation reductions)
+// Pixels per pixel tile (one block of the vector kernels, one partial sum of the per-observation
+// reductions). A block's 256 threads take 1 or 4 pixels each: with 16 (4096 pixels) a coarse map ran on one
+// block (x, r, z update 34 us at nside 16, 9 us now) and a medium one on too few (59 us at nside 256, 44 us
+// now); with 1 on large maps the last block's sum over all partials would grow longer than the pass itself.
+inline int pixel_tile(int64_t npix_total) { return npix_total <= (1 << 18) ? 256 : 1024; }
 constexpr int MAXTAPS = 64;     // longest band of the fused kernels (c_0..c_63)
 constexpr int kLongTaps = 2048; // longest band of the overlap-save N^-1 (TOD in HBM)
 constexpr int kCtlWords = 4;    // device control block of a pointing handle (error, hold, wait budget)
@@ -146,6 +150,16 @@ furax_status launch_dyn(void (*kern)(KArgs...), unsigned grid, unsigned block, s
     return FURAX_OK;
 }
 
+// Kernels without neighbours (no band) split a tile over gridDim.y blocks when there are few tiles
+// (tile_grid), so that a small observation still fills the GPU: this block's part of the tile (len may be <= 0).
+__device__ __forceinline__ Tile tile_part(Tile t)
+{
+    const int part = TILE / (int)gridDim.y, at = part * (int)blockIdx.y;
+    t.t0 += at;
+    t.len = t.len - at < part ? t.len - at : part;
+    return t;
+}
+
 struct CgWs;
 
 }  // namespace fx
@@ -162,6 +176,7 @@ struct furax_pointing {
     std::vector<fx::PTile> ptiles;
     fx::PTile *d_ptiles = nullptr;
     int64_t n_ptiles = 0;
+    int32_t ptile = 1024;             // pixels per pixel tile
     const double *q_bore = nullptr, *q_det = nullptr;
     double2 *d_psi_cs = nullptr;
     bool has_psi = false;
@@ -201,6 +216,15 @@ struct furax_pointing {
                                 has_hwp ? d_hwp_cs : nullptr};
     }
 };
+
+namespace fx {
+// Four blocks per tile below two tiles per SM, one above (block-Jacobi blocks of 4 x 65,536 samples: 25 us on
+// 64 blocks, 20 us on 256; with more tiles than that the SMs are full either way).
+inline dim3 tile_grid(const furax_pointing *p)
+{
+    return dim3((unsigned)p->n_tiles, p->n_tiles < 2LL * p->n_sm ? 4u : 1u);
+}
+}  // namespace fx
 
 struct furax_templates {
     const furax_pointing *p = nullptr;   // layout and pointing (caller-owned, outlives the handle)
@@ -300,6 +324,7 @@ struct Layout {
     std::vector<PTile> ptiles;
     int64_t ndet = 0, nbore = 0, nsamp = 0, npix = 0;
     int32_t max_ndet = 0;
+    int32_t ptile = 1024;   // pixels per pixel tile
 };
 void build_layout(const furax_obs_desc *d, Layout &L);
 furax_status prepare_kernels();
@@ -322,10 +347,10 @@ furax_status prepare_fused_sorted();
 // ---- launchers (fused.cu)
 // acc_* workspaces must be zeroed by the caller; x32 is the padded FP32 copy of the (masked) input.
 // With ft (cached FP32 pointing only: see fused_f32_projects_templates), the kernel also does
-// the template work of ft->mode.
+// the template work of ft->mode. The cached time-ordered kernel returns at once when *done == n_obs.
 furax_status launch_fused_f32(const furax_pointing *p, const furax_noise *n, const float4 *x32, int acc,
                               float4 *acc_hi, float4 *acc_lo, double *acc64, cudaStream_t st,
-                              const FusedTpl *ft = nullptr);
+                              const FusedTpl *ft = nullptr, const unsigned *done = nullptr);
 bool fused_f32_projects_templates(const furax_pointing *p);
 // FP64-accurate operator and right-hand side (fused_tc.cu): acc64 += P^T N^-1 P S^T x (valid may be NULL:
 // every pixel) and acc64 += P^T N^-1 d. tp: the template correction -P^T (W T) b is folded into the same pass,
@@ -333,6 +358,9 @@ bool fused_f32_projects_templates(const furax_pointing *p);
 // FMA chain, else the compensated double-FP32 product (band_tc.cuh).
 furax_status launch_fused_tc(const furax_pointing *p, const furax_noise *n, const double *x, const uint8_t *valid, double *acc64,
                              bool f64, cudaStream_t st);
+// The same on the map already in ws_x4; returns at once when *done == n_obs (PCG iterations after convergence).
+furax_status launch_fused_tc_packed(const furax_pointing *p, const furax_noise *n, double *acc64, bool f64,
+                                    const unsigned *done, cudaStream_t st);
 furax_status launch_rhs_tc(const furax_pointing *p, const furax_noise *n, const void *d, int d_t, double *acc64, bool f64,
                            cudaStream_t st, const furax_templates *tp = nullptr);
 // ws_x4 = x (zero where valid is 0) in 32-byte records.

@@ -116,7 +116,7 @@ template <int MODE, typename T, typename MT, typename TT>
 __global__ void __launch_bounds__(256) P_kernel(const Tile *__restrict__ tiles, PointingView pv,
                                                 const MT *__restrict__ map, TT *__restrict__ tod)
 {
-    const Tile tl = tiles[blockIdx.x];
+    const Tile tl = tile_part(tiles[blockIdx.x]);
     const ObsInfo ob = pv.obs[tl.obs];
     for (int k = threadIdx.x; k < tl.len; k += blockDim.x) {
         const int64_t t = tl.t0 + k;
@@ -134,7 +134,7 @@ __global__ void __launch_bounds__(256) P_kernel(const Tile *__restrict__ tiles, 
 template <int MODE>
 static void dispatch_P(const furax_pointing *p, const void *map, int map_t, void *tod, int tod_t, cudaStream_t st)
 {
-    const unsigned g = (unsigned)p->n_tiles;
+    const dim3 g = tile_grid(p);
     const PointingView pv = p->view();
     if (map_t == FURAX_F64 && tod_t == FURAX_F64)
         P_kernel<MODE, double, double, double><<<g, 256, 0, st>>>(p->d_tiles, pv, (const double *)map, (double *)tod);
@@ -166,7 +166,7 @@ __global__ void __launch_bounds__(256) PT_kernel(const Tile *__restrict__ tiles,
                                                  float4 *__restrict__ lo, double *__restrict__ acc64,
                                                  int32_t *__restrict__ hits)
 {
-    const Tile tl = tiles[blockIdx.x];
+    const Tile tl = tile_part(tiles[blockIdx.x]);
     const ObsInfo ob = pv.obs[tl.obs];
     if constexpr (ACC == FURAX_ACC_F64) {
         // three FP64 sums per sample, issued as whole pixel records by the warp (launched with
@@ -235,7 +235,7 @@ template <int MODE, int ACC>
 static void dispatch_PT_acc(const furax_pointing *p, const void *tod, int tod_t, float4 *hi, float4 *lo, double *a64,
                             int32_t *hits, cudaStream_t st)
 {
-    const unsigned g = (unsigned)p->n_tiles;
+    const dim3 g = tile_grid(p);
     const PointingView pv = p->view();
     if (tod_t == FURAX_F64)
         PT_kernel<MODE, ACC, double, double><<<g, 256, 0, st>>>(p->d_tiles, pv, (const double *)tod, hi, lo, a64, hits);
@@ -315,7 +315,7 @@ __global__ void __launch_bounds__(256) bj_accum_kernel(const Tile *__restrict__ 
     // per-warp staging of the six block entries: the warp issues them as whole 48-byte records
     __shared__ double stage[8][32 * 6];
     __shared__ int32_t spix[8][32];
-    const Tile tl = tiles[blockIdx.x];
+    const Tile tl = tile_part(tiles[blockIdx.x]);
     const ObsInfo ob = pv.obs[tl.obs];
     const double w0 = ninv_diag[ob.det_off + tl.det];
     const int warp = threadIdx.x >> 5;
@@ -403,7 +403,7 @@ furax_status launch_bj(const furax_pointing *p, const furax_noise *n, double rco
     if ((rc = check_cuda(cudaMemsetAsync(blocks_inv, 0, sizeof(double) * 6 * np, st), "memset"))) return rc;
     if ((rc = check_cuda(cudaMemsetAsync(h, 0, sizeof(int32_t) * np, st), "memset"))) return rc;
     if (p->n_tiles > 0) {
-        const unsigned g = (unsigned)p->n_tiles;
+        const dim3 g = tile_grid(p);
         const PointingView pv = p->view();
         if (p->mode == FURAX_POINTING_ON_THE_FLY)
             bj_accum_kernel<0><<<g, 256, 0, st>>>(p->d_tiles, pv, n->diag, blocks_inv, h);

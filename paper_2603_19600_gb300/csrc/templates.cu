@@ -609,11 +609,11 @@ static furax_status build_aug_layout(furax_templates *tp, cudaStream_t st)
         for (int64_t t = 0; t < p->obs[k].nptile; ++t) pt.push_back(p->ptiles[p->obs[k].ptile0 + t]);
         for (size_t i = k; i < p->obs.size(); ++i) {
             if (owner[i] != (int)k) continue;
-            for (int32_t d0 = 0; d0 < p->obs[i].ndet; d0 += PTILE) {
+            for (int32_t d0 = 0; d0 < p->obs[i].ndet; d0 += p->ptile) {
                 PTile t;
                 t.p0 = base + p->obs[i].det_off + d0;
                 t.obs = (int32_t)k;
-                t.len = std::min<int32_t>(PTILE, p->obs[i].ndet - d0);
+                t.len = std::min<int32_t>(p->ptile, p->obs[i].ndet - d0);
                 pt.push_back(t);
             }
         }

@@ -45,6 +45,7 @@ furax_status prepare_fused_tma();
 // next 16-byte boundary past the last sample).
 // With ft, also does the template work of ft->mode (projection, or the augmented system).
 furax_status launch_fused_tma(const furax_pointing *p, const furax_noise *n, const float4 *x32, int acc, float4 *hi,
-                              float4 *lo, double *a64, cudaStream_t st, const FusedTpl *ft = nullptr);
+                              float4 *lo, double *a64, cudaStream_t st, const FusedTpl *ft = nullptr,
+                              const unsigned *done = nullptr);
 
 }  // namespace fx
