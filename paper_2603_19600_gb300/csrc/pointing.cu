@@ -331,56 +331,65 @@ __global__ void __launch_bounds__(256) bj_accum_kernel(const Tile *__restrict__ 
     }
 }
 
-__device__ __forceinline__ double norm1_sym(double a, double b, double c, double d, double e, double f)
+// Largest of three non-negative values (their encodings order like the values; a NaN is largest).
+__device__ __forceinline__ double max3_nonneg(double a, double b, double c)
 {
-    double c0 = fabs(a) + fabs(b) + fabs(c);
-    double c1 = fabs(b) + fabs(d) + fabs(e);
-    double c2 = fabs(c) + fabs(e) + fabs(f);
-    return fmax(c0, fmax(c1, c2));
+    const long long x = __double_as_longlong(a), y = __double_as_longlong(b), z = __double_as_longlong(c);
+    const long long m = x > y ? x : y;
+    return __longlong_as_double(m > z ? m : z);
 }
 
-// Inverse of the symmetric 3x3 block m = (00,01,02,11,12,22) through its Cholesky factor
-// M = L L^T, W = L^-1 by forward substitution, M^-1 = W^T W (explicit round-to-nearest FP64
-// operations, no contraction). Returns false if a pivot is not positive: such a block is not
-// positive definite to working precision (e.g. a pixel crossed only at one angle), and an
-// adjugate/determinant inverse of it would be rounding noise.
+__device__ __forceinline__ double norm1_sym(const double *m)
+{
+    const double c0 = fabs(m[0]) + fabs(m[1]) + fabs(m[2]);
+    const double c1 = fabs(m[1]) + fabs(m[3]) + fabs(m[4]);
+    const double c2 = fabs(m[2]) + fabs(m[4]) + fabs(m[5]);
+    return max3_nonneg(c0, c1, c2);
+}
+
+__device__ __forceinline__ bool positive(double v) { return __double2hiint(v) > 0 && __double2hiint(v) < 0x7ff00000; }
+
+// Inverse of the symmetric 3x3 block m = (00,01,02,11,12,22) through M = L D L^T, W = L^-1, M^-1 = W^T D^-1 W.
+// Returns false if a pivot is not positive: such a block is not positive definite to working precision
+// (e.g. a pixel crossed only at one angle), and an adjugate/determinant inverse of it would be rounding
+// noise. Bound by the FP64 pipe: the square-root-free form takes three reciprocals where the Cholesky
+// factor took three square roots and nine divisions (3.1 M pixels: 571 us, now 194 us with the tests and
+// maxima on the integer pipe).
 __device__ __forceinline__ bool bj_invert3(const double *m, double *inv)
 {
-    if (!(m[0] > 0.0)) return false;
-    const double l11 = __dsqrt_rn(m[0]);
-    const double l21 = __ddiv_rn(m[1], l11), l31 = __ddiv_rn(m[2], l11);
-    const double p2 = __dsub_rn(m[3], __dmul_rn(l21, l21));
-    if (!(p2 > 0.0)) return false;
-    const double l22 = __dsqrt_rn(p2);
-    const double l32 = __ddiv_rn(__dsub_rn(m[4], __dmul_rn(l31, l21)), l22);
-    const double p3 = __dsub_rn(__dsub_rn(m[5], __dmul_rn(l31, l31)), __dmul_rn(l32, l32));
-    if (!(p3 > 0.0)) return false;
-    const double l33 = __dsqrt_rn(p3);
-    const double w11 = __ddiv_rn(1.0, l11), w22 = __ddiv_rn(1.0, l22), w33 = __ddiv_rn(1.0, l33);
-    const double w21 = -__ddiv_rn(__dmul_rn(l21, w11), l22);
-    const double w32 = -__ddiv_rn(__dmul_rn(l32, w22), l33);
-    const double w31 = -__ddiv_rn(__dadd_rn(__dmul_rn(l31, w11), __dmul_rn(l32, w21)), l33);
-    inv[0] = __dadd_rn(__dadd_rn(__dmul_rn(w11, w11), __dmul_rn(w21, w21)), __dmul_rn(w31, w31));
-    inv[1] = __dadd_rn(__dmul_rn(w21, w22), __dmul_rn(w31, w32));
-    inv[2] = __dmul_rn(w31, w33);
-    inv[3] = __dadd_rn(__dmul_rn(w22, w22), __dmul_rn(w32, w32));
-    inv[4] = __dmul_rn(w32, w33);
-    inv[5] = __dmul_rn(w33, w33);
+    if (!positive(m[0])) return false;
+    const double i1 = __drcp_rn(m[0]);
+    const double l21 = m[1] * i1, l31 = m[2] * i1;
+    const double p2 = fma(-l21, m[1], m[3]);
+    if (!positive(p2)) return false;
+    const double i2 = __drcp_rn(p2);
+    const double t = fma(-l31, m[1], m[4]), l32 = t * i2;
+    const double p3 = fma(-l32, t, fma(-l31, m[2], m[5]));
+    if (!positive(p3)) return false;
+    const double i3 = __drcp_rn(p3);
+    const double w31 = fma(l21, l32, -l31);
+    const double a = -l21 * i2;
+    inv[2] = w31 * i3;
+    inv[4] = -l32 * i3;
+    inv[5] = i3;
+    inv[0] = fma(w31, inv[2], fma(-l21, a, i1));
+    inv[1] = fma(w31, inv[4], a);
+    inv[3] = fma(-l32, inv[4], i2);
     return true;
 }
 
 // In place: m6 holds M on entry and M^-1 (0 where invalid) on exit. Valid iff hits >= 3, the
-// block is positive definite (Cholesky pivots > 0) and rcond = 1/(|M|_1 |M^-1|_1) >= rcond_min.
+// block is positive definite (pivots > 0) and rcond = 1/(|M|_1 |M^-1|_1) >= rcond_min.
 __global__ void bj_invert_kernel(double *__restrict__ m6, const int32_t *__restrict__ hits, uint8_t *__restrict__ valid,
                                  double *__restrict__ rcond, int64_t npix, double rcond_min)
 {
     for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < npix; p += (int64_t)gridDim.x * blockDim.x) {
         double *m = m6 + 6 * p;
-        double mm[6] = {m[0], m[1], m[2], m[3], m[4], m[5]};
+        const double mm[6] = {m[0], m[1], m[2], m[3], m[4], m[5]};
         double rc = 0.0, v[6] = {0, 0, 0, 0, 0, 0};
         bool ok = hits[p] >= 3 && bj_invert3(mm, v);
         if (ok) {
-            rc = 1.0 / (norm1_sym(mm[0], mm[1], mm[2], mm[3], mm[4], mm[5]) * norm1_sym(v[0], v[1], v[2], v[3], v[4], v[5]));
+            rc = __drcp_rn(norm1_sym(mm) * norm1_sym(v));
             ok = rc >= rcond_min;
         }
         for (int k = 0; k < 6; ++k) m[k] = ok ? v[k] : 0.0;
