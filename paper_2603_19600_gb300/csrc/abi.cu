@@ -64,7 +64,11 @@ furax_status ensure_ws(furax_pointing *p, void **ptr, size_t bytes)
 {
     if (*ptr) return FURAX_OK;
     if (bytes == 0) bytes = 16;
+    // a first call may come inside a stream capture, which an allocation does not concern
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    cudaThreadExchangeStreamCaptureMode(&mode);
     cudaError_t e = cudaMalloc(ptr, bytes);
+    cudaThreadExchangeStreamCaptureMode(&mode);
     if (e != cudaSuccess) {
         cudaGetLastError();
         *ptr = nullptr;

@@ -804,8 +804,7 @@ furax_status mapmaker_cg(const furax_pointing *p, const furax_noise *n, const vo
     furax_status rc;
     if ((rc = get_ws(pm, o->maxiter + 1, &w))) return rc;
     const int64_t np = p->npix_total;
-    // the FP64-accurate operator's map records exist before any stream capture of the iteration
-    if (!long_band(n) && (rc = ensure_ws(pm, (void **)&pm->ws_x4, sizeof(double4_32a) * (size_t)np))) return rc;
+    if ((rc = ensure_ws(pm, (void **)&pm->ws_x4, sizeof(double4_32a) * (size_t)np))) return rc;   // written by cg_init
     const unsigned pg = (unsigned)std::max<int64_t>(1, p->n_ptiles);
 
     const AllReduce ar{o->allreduce, o->allreduce_user};

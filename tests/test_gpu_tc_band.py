@@ -115,3 +115,33 @@ def test_operators_with_tiles_of_both_kinds(fx, dev, orc, mode):
     for precision in ("f64", "f32x2"):
         got = fx.ptnp_apply(P, N, torch.as_tensor(x, device=dev), precision=precision).cpu().numpy()
         assert rel(got, ref) < 1e-12, precision
+
+
+@pytest.mark.parametrize("what", ["project", "chi2", "normal"])
+def test_first_call_inside_a_stream_capture(fx, dev, what):
+    """The workspaces of a handle's first call are allocated without disturbing a capture in progress."""
+    nd, ns = 4, 20000
+    o = synth.Observation(8, synth.satellite_scan(ns), synth.hex_focal_plane(nd))
+    taps = np.tile(synth.inverse_noise_taps(), (nd, 1))
+    m = torch.as_tensor(synth.gaussian_sky(8, np.random.default_rng(2)), device=dev)
+
+    def call(P, N, d, m):
+        if what == "project":
+            return P.apply(m)
+        if what == "chi2":
+            return fx.chi2_grad(P, N, d, m)[1]
+        return fx.ptnp_apply(P, N, m, precision="f64")
+
+    make = lambda: fx.Pointing.from_observations([o], mode="cache_f64", device=dev)  # noqa: E731
+    P0 = make()
+    N = fx.Noise.banded(P0, taps)
+    d = P0.apply(m) + 1.0
+    ref = call(P0, N, d, m)
+    P = make()
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        got = call(P, N, d, m)
+    graph.replay()
+    torch.cuda.synchronize()
+    assert rel(got, ref.cpu().numpy()) < 1e-13
