@@ -20,7 +20,7 @@ __global__ void __launch_bounds__(FT, 2) chi2_tc_kernel(const Tile *__restrict__
     const Tile tl = tiles[blockIdx.x];
     const ObsInfo ob = pv.obs[tl.obs];
     const int64_t gdet = ob.det_off + tl.det;
-    const TcPsi psi(pv, gdet);
+    const DetOffset psi(pv, gdet);
     const DT *row = d + ob.tod_off + (int64_t)tl.det * ob.nsamp;
     double w = 0.0, *stage;
     int32_t *spix;

@@ -91,9 +91,7 @@ __global__ void __launch_bounds__(FT, 3) fused_f32_kernel(const Tile *__restrict
             qn = 0;
         }
         __syncthreads();
-        float dh[3], dl[3], oh[3], ol[3];
-#pragma unroll
-        for (int k = 0; k < 3; ++k) { dh[k] = sdet[k]; dl[k] = sdet[3 + k]; oh[k] = sdet[6 + k]; ol[k] = sdet[9 + k]; }
+        const DetAxes ax(sdet);
         float2 psf = make_float2(1.f, 0.f);   // the detector's offset rotation, rounded once
         if (pv.psi_cs) psf = make_float2((float)pv.psi_cs[gdet].x, (float)pv.psi_cs[gdet].y);
         int32_t *queue = reinterpret_cast<int32_t *>(xs);   // xs is written only after the pointing
@@ -102,8 +100,7 @@ __global__ void __launch_bounds__(FT, 3) fused_f32_kernel(const Tile *__restrict
             float c = 0.f, s = 0.f;
             int32_t pix = -1;
             if (t >= 0 && t < ob.nsamp) {
-                if (sdet_ok &&
-                    certified_sample(bm + 18 * (ob.bore_off + t), dh, dl, oh, ol, (int32_t)ob.nside, pix, c, s)) {
+                if (sdet_ok && certified_sample(bm + kBoreRow * (ob.bore_off + t), ax, (int32_t)ob.nside, pix, c, s)) {
                     if (pv.hwp_cs) apply_hwp<float>(c, s, pv.hwp_cs[ob.bore_off + t]);
                     if (pv.psi_cs) rotate_psi_f(c, s, psf.x, psf.y);
                 } else {
@@ -235,7 +232,7 @@ furax_status launch_fused_f32(const furax_pointing *p, const furax_noise *n, con
     if (p->mode == FURAX_POINTING_ON_THE_FLY) {
         // the boresight matrices of the certified pointing, from the handle's current quaternions
         furax_pointing *pm = const_cast<furax_pointing *>(p);
-        if ((rc = ensure_ws(pm, (void **)&pm->ws_bore_m, sizeof(float) * 18 * std::max<int64_t>(1, p->nbore_total))))
+        if ((rc = ensure_ws(pm, (void **)&pm->ws_bore_m, sizeof(float) * kBoreRow * std::max<int64_t>(1, p->nbore_total))))
             return rc;
         const unsigned bg = (unsigned)std::max<int64_t>(1, std::min<int64_t>((p->nbore_total + 255) / 256, 16LL * p->n_sm));
         bore_matrix_kernel<<<bg, 256, 0, st>>>(p->q_bore, p->nbore_total, pm->ws_bore_m);

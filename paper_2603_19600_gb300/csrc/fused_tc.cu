@@ -61,7 +61,7 @@ __global__ void __launch_bounds__(FT, 2) tc_operator_kernel(const Tile *__restri
     const Tile tl = tiles[blockIdx.x];
     const ObsInfo ob = pv.obs[tl.obs];
     const int64_t gdet = ob.det_off + tl.det;
-    const TcPsi psi(pv, gdet);
+    const DetOffset psi(pv, gdet);
     tc_begin(sm, nv, gdet);
     if constexpr (TPL)
         if (threadIdx.x == 0) corr.init(tv, tl, ob, gdet);
@@ -98,7 +98,7 @@ __global__ void __launch_bounds__(FT) white_operator_kernel(const Tile *__restri
     if (tl.len <= 0) return;
     const ObsInfo ob = pv.obs[tl.obs];
     const int64_t gdet = ob.det_off + tl.det;
-    const TcPsi psi(pv, gdet);
+    const DetOffset psi(pv, gdet);
     if constexpr (TPL) {
         if (threadIdx.x == 0) corr.init(tv, tl, ob, gdet);
         __syncthreads();

@@ -201,7 +201,7 @@ struct furax_pointing {
     void *ws_tod = nullptr;           // [nsamp] scratch TOD (FP64 size)
     void *ws_tod2 = nullptr;
     int32_t *ws_hits = nullptr;       // [npix] hit counts when the caller passes none
-    float *ws_bore_m = nullptr;       // [nbore][18] boresight rotation matrices (double-FP32)
+    float *ws_bore_m = nullptr;       // [nbore][20] boresight rotation matrices (double-FP32, pointing_fast.cuh)
     fx::CgWs *cg = nullptr;           // solver workspace (allocated by the first solve)
     // operator schedule (furax_pointing_set_schedule); pixel-sorted tiles and their permutation
     furax_schedule sched{};

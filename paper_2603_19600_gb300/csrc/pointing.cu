@@ -118,16 +118,46 @@ __global__ void __launch_bounds__(256) P_kernel(const Tile *__restrict__ tiles, 
 {
     const Tile tl = tile_part(tiles[blockIdx.x]);
     const ObsInfo ob = pv.obs[tl.obs];
-    for (int k = threadIdx.x; k < tl.len; k += blockDim.x) {
-        const int64_t t = tl.t0 + k;
-        T c, s;
-        const int32_t pix = get_sample<MODE, T>(pv, ob, tl.det, t, c, s);
-        T v = (T)0;
-        if (pix >= 0) {
-            const MT *m = map + 3 * (ob.map_off + pix);
-            v = (T)m[0] + (T)m[1] * c + (T)m[2] * s;
+    const int64_t row = ob.tod_off + (int64_t)tl.det * ob.nsamp + tl.t0;
+    if constexpr (MODE != 0 && sizeof(T) == 8) {
+        // FP64 from a cache: four samples per thread, each stage's loads in flight together (widening is
+        // branch-free): 12.6 M samples at nside 256 99 -> 85 us, 148 G random gathers/s of the 166 G/s that
+        // furax_probe_l2 measures (padding the map to one 32-byte load per sample: 87 us; eight samples: 102 us)
+        constexpr int B = 4;
+        const DetOffset psi(pv, ob.det_off + tl.det);
+        for (int k0 = threadIdx.x; k0 < tl.len; k0 += 256 * B) {
+            int32_t pix[B];
+            RawWeights<MODE> w[B];
+            T m[B][3];
+#pragma unroll
+            for (int b = 0; b < B; ++b) pix[b] = __ldg(pv.pix + row + min(k0 + 256 * b, tl.len - 1));
+#pragma unroll
+            for (int b = 0; b < B; ++b) {
+                w[b] = load_weights<MODE>(pv, row + min(k0 + 256 * b, tl.len - 1));
+                const MT *q = map + 3 * (ob.map_off + max(pix[b], 0));
+#pragma unroll
+                for (int i = 0; i < 3; ++i) m[b][i] = (T)__ldg(q + i);
+            }
+#pragma unroll
+            for (int b = 0; b < B; ++b) {
+                const int k = k0 + 256 * b;
+                double c, s;
+                widen_weights<MODE>(w[b], psi, c, s);
+                const double v = pix[b] >= 0 ? fma(m[b][2], s, fma(m[b][1], c, m[b][0])) : 0.0;
+                if (k < tl.len) tod[row + k] = (TT)v;
+            }
         }
-        tod[ob.tod_off + tl.det * ob.nsamp + t] = convert_bits<TT>(v);
+    } else {
+        for (int k = threadIdx.x; k < tl.len; k += blockDim.x) {
+            T c, s;
+            const int32_t pix = get_sample<MODE, T>(pv, ob, tl.det, tl.t0 + k, c, s);
+            T v = (T)0;
+            if (pix >= 0) {
+                const MT *m = map + 3 * (ob.map_off + pix);
+                v = (T)m[0] + (T)m[1] * c + (T)m[2] * s;
+            }
+            tod[row + k] = convert_bits<TT>(v);
+        }
     }
 }
 

@@ -5,7 +5,7 @@
 // ~150 FP64 operations per sample. Here each sample is computed on the FP32 pipes and the
 // exact recipe runs only where the FP32 result could differ from it:
 //   * R(q_bore(t)) is formed once per boresight sample in FP64 and stored as double-FP32
-//     (hi + lo, 18 floats); the detector axes R(q_det) z^, R(q_det) x^ once per tile.
+//     (hi + lo, 18 floats of an 80-byte row); the detector axes R(q_det) z^, R(q_det) x^ once per tile.
 //     d = R(q_bore) d_det and o = R(q_bore) o_det are then evaluated with exact FP32 products
 //     and two-sums, so the FP32 line of sight and orientation are within ~1 ulp of the exact
 //     values (R(a (x) b) = R(a) R(b) for unit quaternions).
@@ -30,34 +30,44 @@
 
 namespace fx {
 
-// Bore matrices: M_t = R(q_bore(t)) row-major, hi[9] then lo[9]; hi[0] = NaN marks a
-// boresight quaternion that must take the exact path (not finite, or |q|^2 not within 4u of 1).
+// Boresight rows: M_t = R(q_bore(t)) in the layout of kBoreRow; [0] = NaN marks a boresight quaternion
+// that must take the exact path (not finite, or |q|^2 not within 4u of 1).
 __global__ void bore_matrix_kernel(const double *__restrict__ q_bore, int64_t n, float *__restrict__ m)
 {
     for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < n; t += (int64_t)gridDim.x * blockDim.x) {
         const Quat q = load_quat(q_bore, t);
-        const double n2 = q.w * q.w + q.x * q.x + q.y * q.y + q.z * q.z;
-        float *o = m + 18 * t;
-        if (!(fabs(n2 - 1.0) <= 4.0 * 5.9604644775390625e-8)) {
-            o[0] = __int_as_float(0x7fc00000);
+        const double off = fabs(q.w * q.w + q.x * q.x + q.y * q.y + q.z * q.z - 1.0);
+        float4 *o = reinterpret_cast<float4 *>(m + kBoreRow * t);
+        if (!(off <= kUnitTol)) {
+            o[0] = make_float4(__int_as_float(0x7fc00000), 0.f, 0.f, 0.f);
             continue;
         }
         const double xx = q.x * q.x, yy = q.y * q.y, zz = q.z * q.z;
         const double xy = q.x * q.y, xz = q.x * q.z, yz = q.y * q.z;
         const double wx = q.w * q.x, wy = q.w * q.y, wz = q.w * q.z;
-        const double r[9] = {1.0 - 2.0 * (yy + zz), 2.0 * (xy - wz), 2.0 * (xz + wy),
-                             2.0 * (xy + wz), 1.0 - 2.0 * (xx + zz), 2.0 * (yz - wx),
-                             2.0 * (xz - wy), 2.0 * (yz + wx), 1.0 - 2.0 * (xx + yy)};
+        // columns of rows 0 and 1 in pairs, then row 2
+        const double r[9] = {1.0 - 2.0 * (yy + zz), 2.0 * (xy + wz), 2.0 * (xy - wz), 1.0 - 2.0 * (xx + zz),
+                             2.0 * (xz + wy), 2.0 * (yz - wx), 2.0 * (xz - wy), 2.0 * (yz + wx), 1.0 - 2.0 * (xx + yy)};
+        float h[9], l[9];
 #pragma unroll
         for (int k = 0; k < 9; ++k) {
-            const float h = (float)r[k];
-            o[k] = h;
-            o[9 + k] = (float)(r[k] - (double)h);
+            h[k] = (float)r[k];
+            l[k] = (float)(r[k] - (double)h[k]);
         }
+        o[0] = make_float4(h[0], h[1], h[2], h[3]);
+        o[1] = make_float4(h[4], h[5], l[0], l[1]);
+        o[2] = make_float4(l[2], l[3], l[4], l[5]);
+        o[3] = make_float4(h[6], h[7], h[8], l[6]);
+        o[4] = make_float4(l[7], l[8], 0.f, 0.f);
     }
 }
 
-__global__ void __launch_bounds__(256) expand_fast_kernel(const Tile *__restrict__ tiles, const ObsInfo *__restrict__ obs,
+// Bound by FP32 issue (the certified evaluation) and the FP64 pipe (the exact recipe for 1.56 % of the samples
+// at nside 512, half of the pipe's time). A refresh of 28.8 M samples: 637 us with scalar two-sums, 4-byte loads of the
+// boresight matrices and integer remainders; 537 us packed, with 16-byte loads and without remainders. Smaller
+// blocks (128 threads: 545 us; 64: 681 us) load the detector axes more often. Tighter margins would send fewer samples
+// to the exact recipe, but those would change their weights' rounding.
+__global__ void __launch_bounds__(256, 4) expand_fast_kernel(const Tile *__restrict__ tiles, const ObsInfo *__restrict__ obs,
                                                           const double *__restrict__ q_bore, const double *__restrict__ q_det,
                                                           const float *__restrict__ bm, const double2 *__restrict__ hwp_cs,
                                                           int32_t *__restrict__ pix_out,
@@ -77,16 +87,14 @@ __global__ void __launch_bounds__(256) expand_fast_kernel(const Tile *__restrict
         qn = 0;
     }
     __syncthreads();
-    float dh[3], dl[3], oh[3], ol[3];
-#pragma unroll
-    for (int k = 0; k < 3; ++k) { dh[k] = sdet[k]; dl[k] = sdet[3 + k]; oh[k] = sdet[6 + k]; ol[k] = sdet[9 + k]; }
+    const DetAxes ax(sdet);
     const bool det_ok = sdet_ok != 0;
     const int64_t row = ob.tod_off + tl.det * ob.nsamp;
     for (int k = threadIdx.x; k < tl.len; k += blockDim.x) {
         const int64_t t = tl.t0 + k;
         int32_t p = -1;
         float c = 1.f, s = 0.f;
-        bool ok = det_ok && certified_sample(bm + 18 * (ob.bore_off + t), dh, dl, oh, ol, (int32_t)ob.nside, p, c, s);
+        bool ok = det_ok && certified_sample(bm + kBoreRow * (ob.bore_off + t), ax, (int32_t)ob.nside, p, c, s);
         if (ok && hwp_cs) apply_hwp<float>(c, s, hwp_cs[ob.bore_off + t]);
         if (ok) {
             pix_out[row + t] = p;
@@ -120,7 +128,7 @@ furax_status launch_expand_fast(const furax_pointing *p, unsigned long long *n_i
 {
     furax_pointing *pm = const_cast<furax_pointing *>(p);
     furax_status rc;
-    if ((rc = ensure_ws(pm, (void **)&pm->ws_bore_m, sizeof(float) * 18 * std::max<int64_t>(1, p->nbore_total))))
+    if ((rc = ensure_ws(pm, (void **)&pm->ws_bore_m, sizeof(float) * kBoreRow * std::max<int64_t>(1, p->nbore_total))))
         return rc;
     const unsigned g = (unsigned)std::max<int64_t>(1, std::min<int64_t>((p->nbore_total + 255) / 256, 16LL * p->n_sm));
     bore_matrix_kernel<<<g, 256, 0, st>>>(p->q_bore, p->nbore_total, pm->ws_bore_m);

@@ -5,26 +5,61 @@
 // is recomputed by the caller with the exact FP64 recipe, so pixels equal the recipe's.
 #pragma once
 #include "pointing_math.cuh"
+#include "stencil.cuh"
 
 namespace fx {
 
 constexpr float kU = 5.9604645e-8f;   // 2^-24
 
-// Row . vector in double-FP32 (exact products of the hi parts, two-sums), rounded to FP32.
-__device__ __forceinline__ float dot3_df(const float *mh, const float *ml, const float (&vh)[3], const float (&vl)[3])
+// Boresight rotation matrices in double-FP32, kBoreRow floats per boresight sample: hi words of rows 0 and 1
+// as pairs (m00, m10), (m01, m11), (m02, m12), their lo words, row 2 hi, row 2 lo. [0] NaN marks a quaternion for the exact path.
+constexpr int kBoreRow = 20;
+constexpr double kUnitTol = 4.0 * 5.9604644775390625e-8;       // |q|^2 within this of 1: FP32 path
+
+__device__ __forceinline__ unsigned long long f2_neg(unsigned long long a) { return a ^ 0x8000000080000000ull; }
+__device__ __forceinline__ unsigned long long f2_add_rn(unsigned long long a, unsigned long long b)
 {
-    float s = 0.f, err = 0.f;
+    unsigned long long d;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+__device__ __forceinline__ unsigned long long f2_sub_rn(unsigned long long a, unsigned long long b)
+{
+    unsigned long long d;
+    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+__device__ __forceinline__ unsigned long long f2_mul_rn(unsigned long long a, unsigned long long b)
+{
+    unsigned long long d;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+__device__ __forceinline__ unsigned long long f2_fma_rn(unsigned long long a, unsigned long long b, unsigned long long c)
+{
+    unsigned long long d;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+    return d;
+}
+
+// Two dot products of three terms in double-FP32 (exact products of the hi parts, two-sums), rounded to
+// FP32: packed, so that the six of a sample are three of these (half the instructions, the same roundings).
+__device__ __forceinline__ unsigned long long dot3_df_x2(const unsigned long long (&mh)[3], const unsigned long long (&ml)[3],
+                                                         const unsigned long long (&vh)[3], const unsigned long long (&vl)[3])
+{
+    unsigned long long s = f2_mul_rn(mh[0], vh[0]);
+    unsigned long long err = f2_fma_rn(mh[0], vl[0], f2_fma_rn(ml[0], vh[0], f2_fma_rn(mh[0], vh[0], f2_neg(s))));
 #pragma unroll
-    for (int j = 0; j < 3; ++j) {
-        const float p = __fmul_rn(mh[j], vh[j]);
-        const float e = __fmaf_rn(mh[j], vh[j], -p);
-        const float t = __fadd_rn(s, p);
-        const float bv = __fsub_rn(t, s);
-        const float te = __fadd_rn(__fsub_rn(s, __fsub_rn(t, bv)), __fsub_rn(p, bv));
+    for (int j = 1; j < 3; ++j) {
+        const unsigned long long p = f2_mul_rn(mh[j], vh[j]);
+        const unsigned long long e = f2_fma_rn(mh[j], vh[j], f2_neg(p));
+        const unsigned long long t = f2_add_rn(s, p);
+        const unsigned long long bv = f2_sub_rn(t, s);
+        const unsigned long long te = f2_add_rn(f2_sub_rn(s, f2_sub_rn(t, bv)), f2_sub_rn(p, bv));
         s = t;
-        err = __fmaf_rn(mh[j], vl[j], __fmaf_rn(ml[j], vh[j], __fadd_rn(err, __fadd_rn(te, e))));
+        err = f2_fma_rn(mh[j], vl[j], f2_fma_rn(ml[j], vh[j], f2_add_rn(err, f2_add_rn(te, e))));
     }
-    return __fadd_rn(s, err);
+    return f2_add_rn(s, err);
 }
 
 __device__ __forceinline__ float frac_dist(float v)
@@ -40,7 +75,6 @@ __device__ __forceinline__ bool fast_ring_pixel(float dx, float dy, float dz, in
 {
     const float rho2 = fmaf(dx, dx, dy * dy);
     if (!(rho2 >= 0.0025f)) return false;              // within ~3 deg of a pole (or NaN)
-    const float rho = sqrtf(rho2);
     const float za = fabsf(dz);
     if (fabsf(za - 0.6666667f) <= 64.f * kU) return false;   // zone decision
     const float N = (float)nside;
@@ -55,15 +89,16 @@ __device__ __forceinline__ bool fast_ring_pixel(float dx, float dy, float dz, in
         const int32_t jp = (int32_t)floorf(a1), jm = (int32_t)floorf(a2);
         const int32_t ir = nside + 1 + jp - jm;
         const int32_t kshift = 1 - (ir & 1);
-        int32_t ip = (jp + jm - nside + kshift) / 2;
         const int32_t nl4 = 4 * nside;
-        ip %= nl4;
+        int32_t ip = (jp + jm - nside + kshift) >> 1;   // an even number in [-2, 8 nside]
+        if (ip >= nl4) ip -= nl4;
         if (ip < 0) ip += nl4;
         const int32_t p = 2 * nside * (nside - 1) + (ir - 1) * nl4 + ip;
         if (p < 0 || p >= 12 * nside * nside) return false;
         pix = p;
         return true;
     }
+    const float rho = sqrtf(rho2);
     const float ft = tt - floorf(tt);
     if (fminf(ft, 1.f - ft) <= 16.f * kU / rho + 64.f * kU) return false;   // facet edge
     const float tmp = N * sqrtf(3.f * (rho2 / (1.f + za)));
@@ -76,7 +111,7 @@ __device__ __forceinline__ bool fast_ring_pixel(float dx, float dy, float dz, in
     if (frac_dist(b3) <= 96.f * N * kU + 16.f * kU / rho + 64.f * kU) return false;
     int32_t ip = (int32_t)floorf(b3);
     const int32_t nl = 4 * ir;
-    ip %= nl;
+    if (ip >= nl) ip -= nl;
     if (ip < 0) ip += nl;
     const int32_t p = dz > 0.f ? 2 * ir * (ir - 1) + ip : 12 * nside * nside - 2 * ir * (ir + 1) + ip;
     if (p < 0 || p >= 12 * nside * nside) return false;
@@ -85,8 +120,8 @@ __device__ __forceinline__ bool fast_ring_pixel(float dx, float dy, float dz, in
 }
 
 // Third and first columns of R(q_det) (line of sight and orientation of the detector) in
-// double-FP32: out = d hi[3], d lo[3], o hi[3], o lo[3]. False if |q_det|^2 is not within 4u of 1
-// (every sample of that detector then takes the exact recipe). FP64: call once per detector.
+// double-FP32: out = d hi[3], d lo[3], o hi[3], o lo[3]. False if |q_det|^2 is not within 4u of 1 (every
+// sample of that detector then takes the exact recipe). FP64: call once per detector.
 __device__ __forceinline__ bool det_axes_df(const Quat &qd, float *out)
 {
     const double n2 = qd.w * qd.w + qd.x * qd.x + qd.y * qd.y + qd.z * qd.z;
@@ -103,24 +138,42 @@ __device__ __forceinline__ bool det_axes_df(const Quat &qd, float *out)
         out[6 + k] = g;
         out[9 + k] = (float)(ov[k] - (double)g);
     }
-    return fabs(n2 - 1.0) <= 4.0 * 5.9604644775390625e-8;
+    return fabs(n2 - 1.0) <= kUnitTol;
 }
 
-// Pixel and FP32 weights (cos 2psi, sin 2psi) of one sample from its boresight matrix m (18
-// floats: hi[9], lo[9]; hi[0] NaN marks a boresight quaternion for the exact path) and the
-// detector axes; false if the exact recipe must decide. No half-wave plate or offset rotation.
-__device__ __forceinline__ bool certified_sample(const float *m, const float (&dh)[3], const float (&dl)[3],
-                                                 const float (&oh)[3], const float (&ol)[3], int32_t nside,
-                                                 int32_t &pix, float &c, float &s)
-{
-    float mh[9], ml[9];
+// The detector's axes as the packed operands of dot3_df_x2.
+struct DetAxes {
+    unsigned long long dh[3], dl[3], oh[3], ol[3], bh[3], bl[3];   // (d, d), (o, o), (d, o): hi and lo words
+    __device__ __forceinline__ explicit DetAxes(const float *ax)
+    {
 #pragma unroll
-    for (int j = 0; j < 9; ++j) { mh[j] = m[j]; ml[j] = m[9 + j]; }
-    if (isnan(mh[0])) return false;
-    const float dx = dot3_df(mh + 0, ml + 0, dh, dl), dy = dot3_df(mh + 3, ml + 3, dh, dl),
-                dz = dot3_df(mh + 6, ml + 6, dh, dl);
-    const float ox = dot3_df(mh + 0, ml + 0, oh, ol), oy = dot3_df(mh + 3, ml + 3, oh, ol),
-                oz = dot3_df(mh + 6, ml + 6, oh, ol);
+        for (int k = 0; k < 3; ++k) {
+            dh[k] = pack_f32x2(ax[k], ax[k]);
+            dl[k] = pack_f32x2(ax[3 + k], ax[3 + k]);
+            oh[k] = pack_f32x2(ax[6 + k], ax[6 + k]);
+            ol[k] = pack_f32x2(ax[9 + k], ax[9 + k]);
+            bh[k] = pack_f32x2(ax[k], ax[6 + k]);
+            bl[k] = pack_f32x2(ax[3 + k], ax[9 + k]);
+        }
+    }
+};
+
+// Pixel and FP32 weights (cos 2psi, sin 2psi) of one sample from its boresight row m and the detector
+// axes; false if the exact recipe must decide. No half-wave plate or offset rotation.
+__device__ __forceinline__ bool certified_sample(const float *m, const DetAxes &ax, int32_t nside, int32_t &pix, float &c,
+                                                 float &s)
+{
+    const float4 *q = reinterpret_cast<const float4 *>(m);
+    const float4 q0 = __ldg(q), q1 = __ldg(q + 1), q2 = __ldg(q + 2), q3 = __ldg(q + 3), q4 = __ldg(q + 4);
+    if (isnan(q0.x)) return false;
+    const unsigned long long ph[3] = {pack_f32x2(q0.x, q0.y), pack_f32x2(q0.z, q0.w), pack_f32x2(q1.x, q1.y)};
+    const unsigned long long pl[3] = {pack_f32x2(q1.z, q1.w), pack_f32x2(q2.x, q2.y), pack_f32x2(q2.z, q2.w)};
+    const unsigned long long zh[3] = {pack_f32x2(q3.x, q3.x), pack_f32x2(q3.y, q3.y), pack_f32x2(q3.z, q3.z)};
+    const unsigned long long zl[3] = {pack_f32x2(q3.w, q3.w), pack_f32x2(q4.x, q4.x), pack_f32x2(q4.y, q4.y)};
+    float dx, dy, dz, ox, oy, oz;
+    unpack_f32x2(dot3_df_x2(ph, pl, ax.dh, ax.dl), dx, dy);
+    unpack_f32x2(dot3_df_x2(ph, pl, ax.oh, ax.ol), ox, oy);
+    unpack_f32x2(dot3_df_x2(zh, zl, ax.bh, ax.bl), dz, oz);
     if (!fast_ring_pixel(dx, dy, dz, nside, pix)) return false;
     // psi from local north through east (same convention as the exact recipe)
     const float rho2 = fmaf(dx, dx, dy * dy);
@@ -133,7 +186,7 @@ __device__ __forceinline__ bool certified_sample(const float *m, const float (&d
     return true;
 }
 
-// Boresight rotation matrices for certified_sample ([n][18], pointing_fast.cu).
+// Boresight rows for certified_sample ([n][kBoreRow], pointing_fast.cu).
 __global__ void bore_matrix_kernel(const double *__restrict__ q_bore, int64_t n, float *__restrict__ m);
 
 }  // namespace fx

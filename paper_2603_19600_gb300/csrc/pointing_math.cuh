@@ -71,6 +71,13 @@ __device__ __forceinline__ double azimuth(double x, double y)
     return a;
 }
 
+// i modulo n in [0, n); called only outside that range (64-bit remainders are long).
+__device__ __forceinline__ int64_t wrap(int64_t i, int64_t n)
+{
+    i %= n;
+    return i < 0 ? i + n : i;
+}
+
 // HEALPix RING index from z = cos(theta), |z|, tt = 2 phi / pi in [0, 4] and 1 - |z|.
 // Equatorial belt (|z| <= 2/3): the pixel lies between edge lines of the two families
 // N (1/2 + tt - 3z/4) and N (1/2 + tt + 3z/4) = integer; their integer parts give the
@@ -84,25 +91,23 @@ __device__ __forceinline__ int64_t ring_pixel(int64_t nside, double z, double za
     if (za <= 2.0 / 3.0) {
         double temp1 = dmul(n, dadd(0.5, tt));
         double temp2 = dmul(n, dmul(z, 0.75));
-        int64_t jp = (int64_t)floor(dsub(temp1, temp2));
-        int64_t jm = (int64_t)floor(dadd(temp1, temp2));
+        int64_t jp = __double2ll_rd(dsub(temp1, temp2));   // floor
+        int64_t jm = __double2ll_rd(dadd(temp1, temp2));
         int64_t ir = nside + 1 + jp - jm;            // 1 .. 2N+1
         int64_t kshift = 1 - (ir & 1);
         int64_t ip = (jp + jm - nside + kshift) / 2;
         int64_t nl4 = 4 * nside;
-        ip %= nl4;
-        if (ip < 0) ip += nl4;
+        if (ip < 0 || ip >= nl4) ip = wrap(ip, nl4);
         return 2 * nside * (nside - 1) + (ir - 1) * nl4 + ip;
     }
     double tp = dsub(tt, floor(tt));
     double tmp = dmul(n, __dsqrt_rn(dmul(3.0, one_minus_za)));
-    int64_t jp = (int64_t)floor(dmul(tp, tmp));
-    int64_t jm = (int64_t)floor(dmul(dsub(1.0, tp), tmp));
+    int64_t jp = __double2ll_rd(dmul(tp, tmp));
+    int64_t jm = __double2ll_rd(dmul(dsub(1.0, tp), tmp));
     int64_t ir = jp + jm + 1;
-    int64_t ip = (int64_t)floor(dmul(tt, (double)ir));
+    int64_t ip = __double2ll_rd(dmul(tt, (double)ir));
     int64_t nl = 4 * ir;
-    ip %= nl;
-    if (ip < 0) ip += nl;
+    if (ip < 0 || ip >= nl) ip = wrap(ip, nl);
     if (z > 0.0) return 2 * ir * (ir - 1) + ip;
     return 12 * nside * nside - 2 * ir * (ir + 1) + ip;
 }
@@ -255,6 +260,59 @@ __device__ __forceinline__ int32_t get_sample(const PointingView &pv, const ObsI
         else { c = (T)pv.c64[i]; s = (T)pv.s64[i]; }
         if (pv.psi_cs && pix >= 0) rotate_psi<T>(c, s, pv.psi_cs[gdet]);
         return pix;
+    }
+}
+
+// FP32 -> FP64 without a conversion instruction (the FP64 pipe is scarce) and without a branch, for
+// cached weights: finite, and words below 2^-126 count as zero (an absolute error of 1e-38).
+__device__ __forceinline__ double weight_f64(float f)
+{
+    const uint32_t b = __float_as_uint(f);
+    const uint32_t hi = ((b & 0x7fffffffu) >> 3) + 0x38000000u;
+    return (b & 0x7f800000u) ? __hiloint2double((int)(hi | (b & 0x80000000u)), (int)(b << 29)) : 0.0;
+}
+
+struct DetOffset {   // the detector's offset rotation
+    double c2 = 1.0, s2 = 0.0;
+    bool on = false;
+    __device__ __forceinline__ DetOffset(const PointingView &pv, int64_t gdet)
+    {
+        if (pv.psi_cs) { const double2 cs = pv.psi_cs[gdet]; c2 = cs.x; s2 = cs.y; on = true; }
+    }
+};
+
+// The cached words of one sample's weights as they are stored, so that their loads need not be waited for
+// one by one.
+template <int MODE> struct RawWeights { float c, s; };
+template <> struct RawWeights<2> { double c, s; };
+template <> struct RawWeights<3> { float c, s, cl, sl; };
+
+template <int MODE>
+__device__ __forceinline__ RawWeights<MODE> load_weights(const PointingView &pv, int64_t i)
+{
+    if constexpr (MODE == 2) return {__ldg(pv.c64 + i), __ldg(pv.s64 + i)};
+    else if constexpr (MODE == 3) return {__ldg(pv.c32 + i), __ldg(pv.s32 + i), __ldg(pv.c32lo + i), __ldg(pv.s32lo + i)};
+    else return {__ldg(pv.c32 + i), __ldg(pv.s32 + i)};
+}
+
+template <int MODE>
+__device__ __forceinline__ void widen_weights(const RawWeights<MODE> &w, const DetOffset &psi, double &c, double &s)
+{
+    if constexpr (MODE == 2) {
+        c = w.c;
+        s = w.s;
+    } else {
+        c = weight_f64(w.c);
+        s = weight_f64(w.s);
+        if constexpr (MODE == 3) {
+            c += weight_f64(w.cl);
+            s += weight_f64(w.sl);
+        }
+    }
+    if (psi.on) {
+        const double r = c * psi.c2 - s * psi.s2;
+        s = s * psi.c2 + c * psi.s2;
+        c = r;
     }
 }
 

@@ -6,59 +6,6 @@
 
 namespace fx {
 
-// FP32 -> FP64 without a conversion instruction (the FP64 pipe is scarce) and without a branch, for
-// cached weights: finite, and words below 2^-126 count as zero (an absolute error of 1e-38).
-__device__ __forceinline__ double weight_f64(float f)
-{
-    const uint32_t b = __float_as_uint(f);
-    const uint32_t hi = ((b & 0x7fffffffu) >> 3) + 0x38000000u;
-    return (b & 0x7f800000u) ? __hiloint2double((int)(hi | (b & 0x80000000u)), (int)(b << 29)) : 0.0;
-}
-
-struct TcPsi {   // the detector's offset rotation
-    double c2 = 1.0, s2 = 0.0;
-    bool on = false;
-    __device__ __forceinline__ TcPsi(const PointingView &pv, int64_t gdet)
-    {
-        if (pv.psi_cs) { const double2 cs = pv.psi_cs[gdet]; c2 = cs.x; s2 = cs.y; on = true; }
-    }
-};
-
-// The cached words of one sample's weights as they are stored, so that their loads need not be waited for
-// one by one.
-template <int MODE> struct TcRaw { float c, s; };
-template <> struct TcRaw<2> { double c, s; };
-template <> struct TcRaw<3> { float c, s, cl, sl; };
-
-template <int MODE>
-__device__ __forceinline__ TcRaw<MODE> tc_load(const PointingView &pv, int64_t i)
-{
-    if constexpr (MODE == 2) return {__ldg(pv.c64 + i), __ldg(pv.s64 + i)};
-    else if constexpr (MODE == 3) return {__ldg(pv.c32 + i), __ldg(pv.s32 + i), __ldg(pv.c32lo + i), __ldg(pv.s32lo + i)};
-    else return {__ldg(pv.c32 + i), __ldg(pv.s32 + i)};
-}
-
-template <int MODE>
-__device__ __forceinline__ void tc_weights(const TcRaw<MODE> &w, const TcPsi &psi, double &c, double &s)
-{
-    if constexpr (MODE == 2) {
-        c = w.c;
-        s = w.s;
-    } else {
-        c = weight_f64(w.c);
-        s = weight_f64(w.s);
-        if constexpr (MODE == 3) {
-            c += weight_f64(w.cl);
-            s += weight_f64(w.sl);
-        }
-    }
-    if (psi.on) {
-        const double r = c * psi.c2 - s * psi.s2;
-        s = s * psi.c2 + c * psi.s2;
-        c = r;
-    }
-}
-
 template <typename DT>
 __device__ __forceinline__ double tod_f64(DT v)
 {
@@ -119,7 +66,7 @@ __device__ __forceinline__ void tc_fill_tod(double (&v)[kTcPer], const TcSlots &
 // sample at a time (the FP64 recipe is too long to unroll), through shared memory.
 template <int MODE, bool RESID, typename DT>
 __device__ __forceinline__ void tc_fill_map(unsigned char *sm, double (&v)[kTcPer], const TcSlots &sl, const PointingView &pv,
-                                            const ObsInfo &ob, const Tile &tl, const TcPsi &psi,
+                                            const ObsInfo &ob, const Tile &tl, const DetOffset &psi,
                                             const double4_32a *__restrict__ x, const DT *__restrict__ d)
 {
     if constexpr (MODE == 0) {
@@ -146,14 +93,14 @@ __device__ __forceinline__ void tc_fill_map(unsigned char *sm, double (&v)[kTcPe
         for (int k = 0; k < kTcPer; ++k) pix[k] = __ldg(pv.pix + sl.index(k));
 #pragma unroll
         for (int k0 = 0; k0 < kTcPer; k0 += B) {
-            TcRaw<MODE> w[B];
+            RawWeights<MODE> w[B];
             TcPix m[B];
             DT dd[B];
 #pragma unroll
             for (int b = 0; b < B; ++b) {
                 const int k = k0 + b;
                 if (k < kTcPer) {
-                    w[b] = tc_load<MODE>(pv, sl.index(k));
+                    w[b] = load_weights<MODE>(pv, sl.index(k));
                     m[b].load(x, ob.map_off + max(pix[k], 0));
                     if constexpr (RESID) dd[b] = __ldg(d + sl.index(k));
                 }
@@ -163,7 +110,7 @@ __device__ __forceinline__ void tc_fill_map(unsigned char *sm, double (&v)[kTcPe
                 const int k = k0 + b;
                 if (k < kTcPer) {
                     double c, s;
-                    tc_weights<MODE>(w[b], psi, c, s);
+                    widen_weights<MODE>(w[b], psi, c, s);
                     double r = m[b].project(pix[k], c, s);
                     if constexpr (RESID) r = tod_f64(dd[b]) - r;
                     v[k] = sl.in(k) ? r : 0.0;
@@ -178,7 +125,7 @@ static_assert(sizeof(double) * kTcPer * FT <= kTcOffCtl - kTcOffX, "the on-the-f
 // a warp together (pix = -1 past the tile or without a pixel). The pointing of eight samples per thread
 // is loaded before the first is used.
 template <int MODE, typename F>
-__device__ __forceinline__ void tc_each(const PointingView &pv, const ObsInfo &ob, const Tile &tl, const TcPsi &psi, F &&f)
+__device__ __forceinline__ void tc_each(const PointingView &pv, const ObsInfo &ob, const Tile &tl, const DetOffset &psi, F &&f)
 {
     const int64_t row = ob.tod_off + (int64_t)tl.det * ob.nsamp + tl.t0;
     if constexpr (MODE == 0) {
@@ -193,18 +140,18 @@ __device__ __forceinline__ void tc_each(const PointingView &pv, const ObsInfo &o
 #pragma unroll 1
         for (int k0 = threadIdx.x; k0 - (int)(threadIdx.x & 31) < tl.len; k0 += B * FT) {
             int32_t pix[B];
-            TcRaw<MODE> w[B];
+            RawWeights<MODE> w[B];
 #pragma unroll
             for (int b = 0; b < B; ++b) {
                 const int64_t i = row + min(k0 + b * FT, tl.len - 1);
                 pix[b] = __ldg(pv.pix + i);
-                w[b] = tc_load<MODE>(pv, i);
+                w[b] = load_weights<MODE>(pv, i);
             }
 #pragma unroll
             for (int b = 0; b < B; ++b) {
                 const int k = k0 + b * FT;
                 double c, s;
-                tc_weights<MODE>(w[b], psi, c, s);
+                widen_weights<MODE>(w[b], psi, c, s);
                 f(k, k < tl.len ? pix[b] : -1, c, s);
             }
         }
