@@ -48,8 +48,10 @@ constexpr int kTcXDig = 8, kTcCDig = 7;                 // digits of the samples
 constexpr int kTcDiag = 8;                              // weights kept
 constexpr int kTcOut = 16;                              // outputs per row (columns per weight)
 constexpr int kTcSteps = 9;                             // K = 144 in steps of 16
+constexpr int TT = 512;                                 // threads per CTA
+constexpr int TR = TILE / TT;                           // outputs per thread
 constexpr int kTcSlots = TILE + 128;                    // samples read by the 256 rows
-constexpr int kTcPer = (kTcSlots + FT - 1) / FT;        // samples per thread
+constexpr int kTcPer = (kTcSlots + TT - 1) / TT;        // samples per thread
 constexpr int kTcPitch = kTcSlots / 16 * 16 + 32;       // bytes per plane; +32 spreads the planes over the banks
 constexpr int kTcRun = 18 * 128;                        // one digit, one half: 18 core matrices
 constexpr int kTcCores = 19;                            // distinct core matrices per digit
@@ -61,16 +63,16 @@ constexpr int kTcRangeMasked = 20;                      // masked vectors: see t
 constexpr int kTcNoTaps = -(1 << 20);                   // exponent of taps that have no digits
 constexpr int kTcMinTaps = 8;                           // shorter bands take the chain (see above)
 constexpr unsigned kTcTmemCols = 256;                   // 2 row blocks x 8 weights x 16 columns
-static_assert(kTcOut == FR && TILE == FT * FR, "thread t owns row t of the tile");
+static_assert(TT == 512 && TR == 8 && kTcOut == 2 * TR, "each of 16 warps owns half of 32 rows");
 static_assert(kTcOffX % 128 == 0 && kTcPitch % 16 == 0 && kTcRun % 16 == 0, "16-byte units");
 static_assert(7 * 127 * 128 * 128 < (1 << 24), "accumulators must stay exact in FP32");
-static_assert(sizeof(double) * XS + (sizeof(double) * 96 + 128) * (FT / 32) <= kTcOffCtl - kTcOffX,
+static_assert(sizeof(double) * XS + (sizeof(double) * 96 + 128) * (TT / 32) <= kTcOffCtl - kTcOffX,
               "the samples' region also holds y and the record staging afterwards");
 
 struct TcCtl {
     uint64_t taps_full, mma_done;
     uint32_t tmem;
-    unsigned wmax[FT / 32], wmin[FT / 32];
+    unsigned wmax[TT / 32], wmin[TT / 32];
 };
 constexpr size_t kTcSmem = kTcOffCtl + sizeof(TcCtl);
 // Two CTAs per SM (one loads and scatters while the other multiplies) and no more: each holds half of TMEM.
@@ -152,10 +154,10 @@ __device__ __forceinline__ void tc_issue(unsigned char *sm, uint32_t tmem)
     }
 }
 
-__device__ __forceinline__ void tc_load8(uint32_t addr, uint32_t (&r)[8])
+__device__ __forceinline__ void tc_load4(uint32_t addr, uint32_t (&r)[4])
 {
-    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
-                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0, %1, %2, %3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
                  : "r"(addr));
 }
 
@@ -202,24 +204,24 @@ __device__ __forceinline__ void tc_put2(unsigned char *p, uint32_t w, uint32_t s
 // With finite samples the zeros past the band's last tap add nothing and are skipped.
 static __device__ __noinline__ void tc_chain(double *xs, const double *__restrict__ c, int ntaps, bool finite)
 {
-    const int base = threadIdx.x * FR;
-    double y[FR];
+    const int base = threadIdx.x * TR;
+    double y[TR];
 #pragma unroll
-    for (int r = 0; r < FR; ++r) y[r] = 0.0;
+    for (int r = 0; r < TR; ++r) y[r] = 0.0;
     const int skip = finite ? kHalo + 1 - ntaps : 0;
 #pragma unroll 1
     for (int j = skip; j < kBand - skip; ++j) {
         const int k = j < kHalo ? kHalo - j : j - kHalo;
         const double t = k < ntaps ? c[k] : 0.0;
 #pragma unroll
-        for (int r = 0; r < FR; ++r) y[r] = fma(t, xs[spos(base + r + j)], y[r]);
+        for (int r = 0; r < TR; ++r) y[r] = fma(t, xs[spos(base + r + j)], y[r]);
     }
     __syncthreads();
 #pragma unroll
-    for (int r = 0; r < FR; ++r) xs[spos(base + r)] = y[r];
+    for (int r = 0; r < TR; ++r) xs[spos(base + r)] = y[r];
 }
 
-// Compensated dot product in double-FP32 on output pairs (y_i, y_{i+8}) (Ogita, Rump & Oishi 2005,
+// Compensated dot product in double-FP32 on output pairs (y_i, y_{i+4}) (Ogita, Rump & Oishi 2005,
 // algorithm Dot2; packed FP32): every product of the high words is split exactly by an FMA, the products
 // are summed with Knuth's two-sum, and errors and cross terms gather in a second word; the product is
 // negated once so that no packed negation is needed. C4[j] = (c_hi, c_hi, -c_hi, -c_hi) and CL2[j] =
@@ -334,19 +336,19 @@ static __device__ __noinline__ void tc_dot2(float *xh, const double *__restrict_
         CL2[j] = make_float2(l, l);
     }
     __syncthreads();
-    float S[FR], E[FR];
-    const int base = threadIdx.x * FR;
-    band_product_dfx2<FR>(xh, xl, C4, CL2, base, S, E);
+    float S[TR], E[TR];
+    const int base = threadIdx.x * TR;
+    band_product_dfx2<TR>(xh, xl, C4, CL2, base, S, E);
     __syncthreads();
     double *ys = reinterpret_cast<double *>(xh);
 #pragma unroll
-    for (int r = 0; r < FR; ++r) ys[spos(base + r)] = (double)S[r] + (double)E[r];
+    for (int r = 0; r < TR; ++r) ys[spos(base + r)] = (double)S[r] + (double)E[r];
 }
 static_assert((2 * XS + 4) % 4 == 0 && sizeof(float) * (2 * XS + 4) + (16 + 8) * kBandPad <= kTcOffCtl - kTcOffX,
               "the compensated product fits the samples' region");
 
 // tc_ys(sm)[spos(t)] = sum_k c_|k| x_{t+k} for the tile's outputs t. v[k]: the sample of slot u = threadIdx.x +
-// 256 k (slot 63 is the tile's first output; zero past the loaded samples). Every thread calls it after
+// 512 k (slot 63 is the tile's first output; zero past the loaded samples). Every thread calls it after
 // tc_begin; on return the results are visible to the CTA and no TMEM is held. Slots [in0, in1) lie in the
 // stream. f64: FP64 accuracy of every output (else that of the compensated product). MASKED: zero
 // samples are masked ones whose own outputs are not used (the vectors of gap filling): all-zero groups do not
@@ -364,13 +366,13 @@ __device__ __forceinline__ void tc_band(unsigned char *sm, const double (&v)[kTc
     for (int k = 0; k < kTcPer; ++k) {
         const unsigned m = __reduce_max_sync(0xffffffffu, (unsigned)__double2hiint(v[k]) & 0x7fffffffu);
         gmax = max(gmax, m);
-        const int u0 = 32 * warp + k * FT;
+        const int u0 = 32 * warp + k * TT;
         if (MASKED ? m != 0u : u0 >= in0 && u0 + 32 <= in1) gmin = min(gmin, m);   // whole groups of the stream
     }
     if (lane == 0) { C.wmax[warp] = gmax; C.wmin[warp] = gmin; }
     __syncthreads();
 #pragma unroll
-    for (int w = 0; w < FT / 32; ++w) { gmax = max(gmax, C.wmax[w]); gmin = min(gmin, C.wmin[w]); }
+    for (int w = 0; w < TT / 32; ++w) { gmax = max(gmax, C.wmax[w]); gmin = min(gmin, C.wmin[w]); }
     const int emax = (int)(gmax >> 20), ec = nv.tc_exp[gdet];
     const int ey = emax - 1022 + ec - 69;   // y = (H 2^32 + L) 2^ey
     const int range = MASKED ? kTcRangeMasked : f64 ? kTcRange : kTcRangeDot2;
@@ -380,7 +382,7 @@ __device__ __forceinline__ void tc_band(unsigned char *sm, const double (&v)[kTc
         unsigned char *px = sm + kTcOffX;
 #pragma unroll
         for (int k = 0; k < kTcPer; ++k) {
-            const int u = threadIdx.x + k * FT;
+            const int u = threadIdx.x + k * TT;
             if (u < kTcSlots) {
                 // 62-bit integer x 2^(62 - ex) with |x| < 2^ex, then offset digits (byte = digit + 128)
                 const uint32_t hi = (uint32_t)__double2hiint(v[k]), lo = (uint32_t)__double2loint(v[k]);
@@ -409,23 +411,24 @@ __device__ __forceinline__ void tc_band(unsigned char *sm, const double (&v)[kTc
         __syncwarp();
         mbar_wait(&C.mma_done, 0, err, budget);
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        // row 16 t: lane t & 127 of TMEM, row block t >> 7
-        const uint32_t row = tmem + ((uint32_t)(warp & 3) << 21) + 128u * (warp >> 2);
-        double *ys = tc_ys(sm);
+        // warps 4 b .. 4 b + 3 hold the 128 rows of block b & 1, one lane each, and half b >> 1 of their columns
+        const int half = warp >> 3, r0 = 128 * ((warp >> 2) & 1) + 32 * (warp & 3) + lane;
+        const uint32_t at = tmem + ((uint32_t)(warp & 3) << 21) + 128u * ((warp >> 2) & 1) + 8u * half;
+        double *ys = tc_ys(sm) + spos(kTcOut * r0);   // a row's 16 slots are consecutive
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
-            uint32_t d[kTcDiag][8];
+            uint32_t d[kTcDiag][4];
 #pragma unroll
-            for (int w = 0; w < kTcDiag; ++w) tc_load8(row + 16 * w + 8 * h, d[w]);
+            for (int w = 0; w < kTcDiag; ++w) tc_load4(at + 16 * w + 4 * h, d[w]);
             asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
-            for (int r = 0; r < 8; ++r) {
+            for (int r = 0; r < 4; ++r) {
                 int q[kTcDiag];
 #pragma unroll
                 for (int w = 0; w < kTcDiag; ++w) q[w] = __float2int_rn(__uint_as_float(d[w][r]));
                 const long long H = (long long)q[0] * (1 << 24) + ((long long)q[1] * (1 << 16) + ((long long)q[2] * 256 + q[3]));
                 const long long L = (long long)q[4] * (1 << 24) + ((long long)q[5] * (1 << 16) + ((long long)q[6] * 256 + q[7]));
-                ys[spos(threadIdx.x * FR + 8 * (1 - h) + r)] = tc_value(H, L, ey);
+                ys[8 * (1 - half) + 4 * h + r] = tc_value(H, L, ey);
             }
         }
         asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -436,7 +439,7 @@ __device__ __forceinline__ void tc_band(unsigned char *sm, const double (&v)[kTc
         float *xh = reinterpret_cast<float *>(xs);
 #pragma unroll
         for (int k = 0; k < kTcPer; ++k) {
-            const int u = threadIdx.x + k * FT;
+            const int u = threadIdx.x + k * TT;
             if (u < TILE + 2 * kHalo) {
                 if (dot2) {
                     const float h = (float)v[k];

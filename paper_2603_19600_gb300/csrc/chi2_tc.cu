@@ -2,21 +2,22 @@
 // in the detectors' polarisation angles (the paper's differentiability, "Summary"), FP64-accurate, for
 // FURAX_F64 and FURAX_PREC_F32X2: the tile skeleton of fused_tc.cu, the band on the tensor cores.
 //
-// r is formed twice, once into the digits and once in time order beside y (keeping it would cost the second
-// CTA its shared memory). Bound by the FP64 pipe (13 instructions per sample, where the FMA chain took 127 for
-// the band alone) and the phases' latency: 128 x 131,072 samples, nside 256, FP64 cache: 4561 -> 920 us.
+// r stays in the registers it was formed in until y is known; the map records are gathered a second time for the
+// angle gradient. Bound by the FP64 pipe (10 instructions per sample and 8 more for angle offsets, where the FMA chain
+// took 127 for the band alone) and the phases' latency: 128 x 131,072 samples, nside 256, FP64 cache: 4561 us with the
+// chain, 919 us with r formed a second time beside y and 256 threads, 882 us now.
 #include "tc_sample.cuh"
 
 namespace fx {
 
 template <int MODE, bool BANDED, typename DT>
-__global__ void __launch_bounds__(FT, 2) chi2_tc_kernel(const Tile *__restrict__ tiles, PointingView pv, NoiseView nv,
+__global__ void __launch_bounds__(TT, 2) chi2_tc_kernel(const Tile *__restrict__ tiles, PointingView pv, NoiseView nv,
                                                         const DT *__restrict__ d, const double4_32a *__restrict__ m,
                                                         double *__restrict__ chi2, double *__restrict__ grad_map,
                                                         double *__restrict__ grad_psi, unsigned *__restrict__ err, bool f64)
 {
     extern __shared__ __align__(128) unsigned char sm[];
-    __shared__ double red[2][FT / 32];
+    __shared__ double red[2][TT / 32];
     const Tile tl = tiles[blockIdx.x];
     const ObsInfo ob = pv.obs[tl.obs];
     const int64_t gdet = ob.det_off + tl.det;
@@ -24,6 +25,8 @@ __global__ void __launch_bounds__(FT, 2) chi2_tc_kernel(const Tile *__restrict__
     const DT *row = d + ob.tod_off + (int64_t)tl.det * ob.nsamp;
     double w = 0.0, *stage;
     int32_t *spix;
+    double part_chi2 = 0.0, part_psi = 0.0;
+    const double *ys = tc_ys(sm);
     if constexpr (BANDED) {
         stage = tc_stage(sm);
         spix = tc_stage_pix(sm);
@@ -32,28 +35,42 @@ __global__ void __launch_bounds__(FT, 2) chi2_tc_kernel(const Tile *__restrict__
         const TcSlots sl(tl, ob);
         tc_fill_map<MODE, true>(sm, v, sl, pv, ob, tl, psi, m, d);
         tc_band<false>(sm, v, nv, gdet, err, f64, sl.in0, sl.in1);
+        // r^T N^-1 r over this thread's own slots: r is still at hand
+#pragma unroll
+        for (int k = 0; k < kTcPer; ++k) {
+            const int t = sl.slot(k) - kHalo;
+            if (t >= 0 && t < tl.len) part_chi2 = fma(v[k], ys[spos(t)], part_chi2);
+        }
     } else {
-        __shared__ double wstage[FT / 32][96];
-        __shared__ int32_t wpix[FT / 32][32];
+        __shared__ double wstage[TT / 32][96];
+        __shared__ int32_t wpix[TT / 32][32];
         stage = wstage[threadIdx.x >> 5];
         spix = wpix[threadIdx.x >> 5];
         w = nv.p64[gdet];
     }
-    const double *ys = tc_ys(sm);
     double *rec = grad_map ? grad_map + 3 * ob.map_off : nullptr;
-    double part_chi2 = 0.0, part_psi = 0.0;
-    tc_each<MODE>(pv, ob, tl, psi, [&](int k, int32_t pix, double c, double s) {
+    struct In {
+        TcPix m;
+        DT d;
+    };
+    tc_each<MODE, TT, 2>(pv, ob, tl, psi, [&](int k, int32_t pix) {
+        In in;
+        in.m.load(m, ob.map_off + max(pix, 0));
+        if constexpr (!BANDED) in.d = __ldg(row + tl.t0 + k);
+        return in;
+    }, [&](int k, int32_t pix, double c, double s, const In &in) {
         double g = 0.0;
         if (k < tl.len) {
-            TcPix mm;
-            mm.load(m, ob.map_off + max(pix, 0));
-            const double r = tod_f64(__ldg(row + tl.t0 + k)) - mm.project(pix, c, s);
             double y;
-            if constexpr (BANDED) y = ys[spos(k)];
-            else y = r * w;
-            part_chi2 = fma(r, y, part_chi2);
+            if constexpr (BANDED) {
+                y = ys[spos(k)];
+            } else {
+                const double r = tod_f64(in.d) - in.m.project(pix, c, s);
+                y = r * w;
+                part_chi2 = fma(r, y, part_chi2);
+            }
             if (pix >= 0) {
-                part_psi = fma(y, fma(mm.u, c, -(mm.q * s)), part_psi);
+                part_psi = fma(y, fma(in.m.u, c, -(in.m.q * s)), part_psi);
                 g = -2.0 * y;
             }
         }
@@ -73,7 +90,7 @@ __global__ void __launch_bounds__(FT, 2) chi2_tc_kernel(const Tile *__restrict__
     __syncthreads();
     if (threadIdx.x == 0) {
         double a = 0.0, b = 0.0;
-        for (int i = 0; i < FT / 32; ++i) { a += red[0][i]; b += red[1][i]; }
+        for (int i = 0; i < TT / 32; ++i) { a += red[0][i]; b += red[1][i]; }
         red_add_f64(chi2 + tl.obs, a);
         if (grad_psi) red_add_f64(grad_psi + gdet, -2.0 * b);
     }
@@ -84,9 +101,9 @@ static furax_status run_chi2_tc(const furax_pointing *p, const furax_noise *n, c
                                 double *gm, double *gp, bool f64, cudaStream_t st)
 {
     if (n->kind == FURAX_NOISE_BANDED)
-        return launch_dyn(chi2_tc_kernel<MODE, true, DT>, (unsigned)p->n_tiles, FT, kTcSmem, st, p->d_tiles, p->view(),
+        return launch_dyn(chi2_tc_kernel<MODE, true, DT>, (unsigned)p->n_tiles, TT, kTcSmem, st, p->d_tiles, p->view(),
                           n->view(), d, m, chi2, gm, gp, p->d_err, f64);
-    return launch_dyn(chi2_tc_kernel<MODE, false, DT>, (unsigned)p->n_tiles, FT, 0, st, p->d_tiles, p->view(),
+    return launch_dyn(chi2_tc_kernel<MODE, false, DT>, (unsigned)p->n_tiles, TT, 0, st, p->d_tiles, p->view(),
                       n->view(), d, m, chi2, gm, gp, p->d_err, f64);
 }
 

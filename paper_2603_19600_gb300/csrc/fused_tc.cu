@@ -7,12 +7,14 @@
 // cores (band_tc.cuh) and scatters y (1, cos 2psi, sin 2psi) in time order as whole FP64 pixel records; the
 // pointing is read a second time for the scatter (from L2), which leaves the shared memory to the digits.
 // What bounds it: the L2's FP64 reductions (3 per sample, 18,000 cycles per tile and SM at the rate of
-// furax_probe_l2 kind 5) and the latency of the phases before them (fill, digits 4,000, products 9,000,
-// accumulators to y 6,000-10,000 cycles), which two CTAs per SM overlap in part; then the FP64 pipe (4
-// instructions per sample). Measured (GB300), before (FP64 FMAs; double-FP32 for the right-hand side) and now:
-//   normal operator, 32 x 262,147 samples, nside 256, FP64 cache   2277 -> 324 us
-//   right-hand side, 128 x 524,288 FP32 samples, mixed cache       3437 -> 1730 us
-//   N^-1 alone inside gap filling, 32 x 131,071 samples            1011 -> 60 us
+// furax_probe_l2 kind 5) and the latency of the phases before them (fill 4,000 from data, 21,000 through a map;
+// digits 3,500; products 9,000; accumulators to y 5,000-7,000 cycles), which two CTAs per SM overlap in part.
+// Each CTA has 512 threads at 64 registers: with 256 at 128 the same phases took 5,000 / 26,000, 4,000, 9,000 and
+// 6,000-10,000 cycles and the scatter 33,000 instead of 23,000. Measured (GB300): FP64 FMAs (double-FP32 for the
+// right-hand side), 256 threads, now:
+//   normal operator, 32 x 262,147 samples, nside 256, FP64 cache   2277, 329, 290 us
+//   right-hand side, 128 x 524,288 FP32 samples, mixed cache       3440, 1730, 1419 us
+//   N^-1 alone, 32 x 131,071 samples                               1011, 61, 58 us
 #include "tc_sample.cuh"
 #include "tpl_eval.cuh"
 
@@ -50,7 +52,7 @@ struct TplCorr {
 
 // FROM_TOD: samples d, else P x. TPL (FROM_TOD only): with the template correction.
 template <int MODE, bool FROM_TOD, bool TPL, typename DT>
-__global__ void __launch_bounds__(FT, 2) tc_operator_kernel(const Tile *__restrict__ tiles, PointingView pv, NoiseView nv,
+__global__ void __launch_bounds__(TT, 2) tc_operator_kernel(const Tile *__restrict__ tiles, PointingView pv, NoiseView nv,
                                                             const double4_32a *__restrict__ x, const DT *__restrict__ d,
                                                             double *__restrict__ acc64, unsigned *__restrict__ err,
                                                             bool f64, TplView tv, const unsigned *__restrict__ done, unsigned n_obs)
@@ -74,7 +76,8 @@ __global__ void __launch_bounds__(FT, 2) tc_operator_kernel(const Tile *__restri
     }
     const double *ys = tc_ys(sm);
     double *rec = acc64 + 3 * ob.map_off;
-    tc_each<MODE>(pv, ob, tl, psi, [&](int k, int32_t pix, double c, double s) {
+    tc_each<MODE, TT, 4>(pv, ob, tl, psi, [](int, int32_t) { return TcNone{}; },
+                         [&](int k, int32_t pix, double c, double s, TcNone) {
         double y = pix >= 0 ? ys[spos(k)] : 0.0;
         if constexpr (TPL)
             if (pix >= 0) y = corr.apply(y, nv, tv, tl, ob, gdet, k);
@@ -107,15 +110,20 @@ __global__ void __launch_bounds__(FT) white_operator_kernel(const Tile *__restri
     const DT *row = d + ob.tod_off + (int64_t)tl.det * ob.nsamp + tl.t0;
     double *rec = acc64 + 3 * ob.map_off;
     const int warp = threadIdx.x >> 5;
-    tc_each<MODE>(pv, ob, tl, psi, [&](int k, int32_t pix, double c, double s) {
+    struct In {   // map record or datum
+        TcPix m;
+        DT d;
+    };
+    tc_each<MODE, FT, 4>(pv, ob, tl, psi, [&](int k, int32_t pix) {
+        In in;
+        if constexpr (FROM_TOD) in.d = __ldg(row + k);
+        else in.m.load(x, ob.map_off + max(pix, 0));
+        return in;
+    }, [&](int k, int32_t pix, double c, double s, const In &in) {
         double y = 0.0;
         if (pix >= 0) {
-            if constexpr (FROM_TOD) y = tod_f64(row[k]) * w;
-            else {
-                TcPix m;
-                m.load(x, ob.map_off + pix);
-                y = m.project(pix, c, s) * w;
-            }
+            if constexpr (FROM_TOD) y = tod_f64(in.d) * w;
+            else y = in.m.project(pix, c, s) * w;
             if constexpr (TPL) y = corr.apply(y, nv, tv, tl, ob, gdet, k);
         }
         const double v[3] = {y, y * c, y * s};
@@ -125,7 +133,7 @@ __global__ void __launch_bounds__(FT) white_operator_kernel(const Tile *__restri
 
 // out = N^-1 in on an FP64 TOD, banded.
 template <bool MASKED>
-__global__ void __launch_bounds__(FT, 2) tc_ninv_kernel(const Tile *__restrict__ tiles, const ObsInfo *__restrict__ obs,
+__global__ void __launch_bounds__(TT, 2) tc_ninv_kernel(const Tile *__restrict__ tiles, const ObsInfo *__restrict__ obs,
                                                         NoiseView nv, const double *__restrict__ in,
                                                         double *__restrict__ out, unsigned *__restrict__ err, bool f64)
 {
@@ -140,13 +148,13 @@ __global__ void __launch_bounds__(FT, 2) tc_ninv_kernel(const Tile *__restrict__
     tc_fill_tod(v, sl, in);
     tc_band<MASKED>(sm, v, nv, gdet, err, f64, sl.in0, sl.in1);
     const double *ys = tc_ys(sm);
-    for (int k = threadIdx.x; k < tl.len; k += FT) out[row + tl.t0 + k] = ys[spos(k)];
+    for (int k = threadIdx.x; k < tl.len; k += TT) out[row + tl.t0 + k] = ys[spos(k)];
 }
 
 furax_status launch_ninv_tc(const furax_noise *n, const double *in, double *out, bool masked, bool f64, cudaStream_t st)
 {
     if (n->n_tiles == 0) return FURAX_OK;
-    furax_status rc = launch_dyn(masked ? tc_ninv_kernel<true> : tc_ninv_kernel<false>, (unsigned)n->n_tiles, FT, kTcSmem, st,
+    furax_status rc = launch_dyn(masked ? tc_ninv_kernel<true> : tc_ninv_kernel<false>, (unsigned)n->n_tiles, TT, kTcSmem, st,
                                  n->d_tiles, n->d_obs, n->view(), in, out, n->d_err, f64);
     if (rc) return rc;
     count_launches(1);
@@ -158,7 +166,7 @@ static furax_status run_tc(const furax_pointing *p, const furax_noise *n, const 
                            bool f64, const TplView &tv, const unsigned *done, cudaStream_t st)
 {
     if (n->kind == FURAX_NOISE_BANDED)
-        return launch_dyn(tc_operator_kernel<MODE, FROM_TOD, TPL, DT>, (unsigned)p->n_tiles, FT, kTcSmem, st, p->d_tiles,
+        return launch_dyn(tc_operator_kernel<MODE, FROM_TOD, TPL, DT>, (unsigned)p->n_tiles, TT, kTcSmem, st, p->d_tiles,
                           p->view(), n->view(), x, d, a64, p->d_err, f64, tv, done, (unsigned)p->n_obs);
     white_operator_kernel<MODE, FROM_TOD, TPL, DT><<<tile_grid(p), FT, 0, st>>>(p->d_tiles, p->view(), n->view(), x,
                                                                                          d, a64, tv, done,

@@ -15,8 +15,8 @@ __device__ __forceinline__ double tod_f64(DT v)
 
 // One pixel of an FP64 map padded to 32-byte records (I, Q, U, 0): one 32-byte load and one L2 sector per
 // random gather, where a 24-byte record takes two or three loads and 1.5 sectors (fill phase of the normal
-// operator: 43,600 cycles per tile with three loads, sample by sample; 30,200 with two and the batches below;
-// 25,700 with this; the pass that packs the map costs 8 us at nside 256).
+// operator, 256 threads: 43,600 cycles per tile with three loads, sample by sample; 30,200 with two and the batches
+// below; 25,700 with this, 21,300 with 512 threads; the pass that packs the map costs 8 us at nside 256).
 struct TcPix {
     double i, q, u;
     __device__ __forceinline__ void load(const double4_32a *__restrict__ x4, int64_t gp)
@@ -45,7 +45,7 @@ struct TcSlots {
         : row(ob.tod_off + (int64_t)tl.det * ob.nsamp + tl.t0 - kHalo), in0(tc_in0(tl)), in1(tc_in1(tl, ob))
     {
     }
-    __device__ __forceinline__ int slot(int k) const { return (int)threadIdx.x + k * FT; }
+    __device__ __forceinline__ int slot(int k) const { return (int)threadIdx.x + k * TT; }
     __device__ __forceinline__ bool in(int k) const { return slot(k) >= in0 && slot(k) < in1; }
     __device__ __forceinline__ int64_t index(int k) const { return row + max(in0, min(slot(k), in1 - 1)); }
 };
@@ -87,7 +87,7 @@ __device__ __forceinline__ void tc_fill_map(unsigned char *sm, double (&v)[kTcPe
 #pragma unroll
         for (int k = 0; k < kTcPer; ++k) v[k] = tmp[sl.slot(k)];
     } else {
-        constexpr int B = RESID ? 4 : 5;
+        constexpr int B = 3;
         int32_t pix[kTcPer];
 #pragma unroll
         for (int k = 0; k < kTcPer; ++k) pix[k] = __ldg(pv.pix + sl.index(k));
@@ -119,43 +119,48 @@ __device__ __forceinline__ void tc_fill_map(unsigned char *sm, double (&v)[kTcPe
         }
     }
 }
-static_assert(sizeof(double) * kTcPer * FT <= kTcOffCtl - kTcOffX, "the on-the-fly fill fits the samples' region");
+static_assert(sizeof(double) * kTcPer * TT <= kTcOffCtl - kTcOffX, "the on-the-fly fill fits the samples' region");
 
-// Core samples of the tile in time order, 32 consecutive ones per warp: f(k, pix, c, s) for every lane of
-// a warp together (pix = -1 past the tile or without a pixel). The pointing of eight samples per thread
-// is loaded before the first is used.
-template <int MODE, typename F>
-__device__ __forceinline__ void tc_each(const PointingView &pv, const ObsInfo &ob, const Tile &tl, const DetOffset &psi, F &&f)
+// Core samples of the tile in time order, 32 consecutive ones per warp: f(k, pix, c, s, more(k, pix)) for every
+// lane of a warp together (pix = -1 past the tile or without a pixel). Cached pointing: the loads of B samples per
+// thread (of NT), and what `more` loads for them (k clamped into the tile), are issued before the first is used.
+template <int MODE, int NT, int B, typename G, typename F>
+__device__ __forceinline__ void tc_each(const PointingView &pv, const ObsInfo &ob, const Tile &tl, const DetOffset &psi,
+                                        G &&more, F &&f)
 {
     const int64_t row = ob.tod_off + (int64_t)tl.det * ob.nsamp + tl.t0;
     if constexpr (MODE == 0) {
 #pragma unroll 1
-        for (int k = threadIdx.x; k - (int)(threadIdx.x & 31) < tl.len; k += FT) {
+        for (int k = threadIdx.x; k - (int)(threadIdx.x & 31) < tl.len; k += NT) {
             double c = 0.0, s = 0.0;
             const int32_t pix = k < tl.len ? get_sample<0, double>(pv, ob, tl.det, tl.t0 + k, c, s) : -1;
-            f(k, pix, c, s);
+            f(k, pix, c, s, more(min(k, tl.len - 1), pix));
         }
     } else {
-        constexpr int B = 8;
 #pragma unroll 1
-        for (int k0 = threadIdx.x; k0 - (int)(threadIdx.x & 31) < tl.len; k0 += B * FT) {
+        for (int k0 = threadIdx.x; k0 - (int)(threadIdx.x & 31) < tl.len; k0 += B * NT) {
             int32_t pix[B];
             RawWeights<MODE> w[B];
+            decltype(more(0, 0)) g[B];
+#pragma unroll
+            for (int b = 0; b < B; ++b) pix[b] = __ldg(pv.pix + row + min(k0 + b * NT, tl.len - 1));
 #pragma unroll
             for (int b = 0; b < B; ++b) {
-                const int64_t i = row + min(k0 + b * FT, tl.len - 1);
-                pix[b] = __ldg(pv.pix + i);
-                w[b] = load_weights<MODE>(pv, i);
+                const int k = min(k0 + b * NT, tl.len - 1);
+                w[b] = load_weights<MODE>(pv, row + k);
+                g[b] = more(k, pix[b]);
             }
 #pragma unroll
             for (int b = 0; b < B; ++b) {
-                const int k = k0 + b * FT;
+                const int k = k0 + b * NT;
                 double c, s;
                 widen_weights<MODE>(w[b], psi, c, s);
-                f(k, k < tl.len ? pix[b] : -1, c, s);
+                f(k, k < tl.len ? pix[b] : -1, c, s, g[b]);
             }
         }
     }
 }
+
+struct TcNone {};
 
 }  // namespace fx
