@@ -411,7 +411,7 @@ furax_status furax_mapmaker_cg_deproject(const furax_templates_t *t, const void 
  * FP32 (vectors and scalars stay FP64; the filled values are then good to ~1e-7 relative),
  * FURAX_PREC_F32X2 as FURAX_F64 (the FP64-accurate band product on the tensor cores);
  * iters_out: host int32 [sum ndet] or NULL. The first call allocates TOD-sized workspaces in the
- * handle (3 FP64, plus 1 FP64 for FURAX_F64 / FURAX_PREC_F32X2 or 2 FP32 for FURAX_F32) that later calls reuse and
+ * handle (3 FP64, plus 2 FP64 for FURAX_F64 / FURAX_PREC_F32X2 or 2 FP32 for FURAX_F32) that later calls reuse and
  * furax_noise_destroy frees, so calls on one handle must not run concurrently; synchronises
  * stream. FURAX_ENOTCONVERGED when a detector stopped at maxiter (out is still written). */
 furax_status furax_gapfill(const furax_noise_t *cov, const void *d, const uint8_t *valid, const void *n_real,

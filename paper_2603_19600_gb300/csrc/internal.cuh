@@ -267,7 +267,7 @@ struct furax_noise {
     float *spec32 = nullptr;
     // gap-filling workspaces (TOD-sized), allocated by the first furax_gapfill that needs them and
     // reused by later calls; freed with the handle
-    double *gf_y = nullptr, *gf_r = nullptr, *gf_p = nullptr, *gf_q = nullptr;
+    double *gf_y = nullptr, *gf_r = nullptr, *gf_p = nullptr, *gf_p2 = nullptr, *gf_q = nullptr;
     float *gf_x32 = nullptr, *gf_n32 = nullptr;
     void *gf_sc = nullptr;
     float *band2 = nullptr;     // banded, <= MAXTAPS taps: [ndet][256] band in tap order as duplicated pairs
