@@ -37,7 +37,7 @@ template <int KC> constexpr int tma_threads() { return 32 * (kTmaGather + KC + 1
 constexpr int kRawStages = 2;
 constexpr int kXsStages = 2;
 // Elements of one pointing stream copied per tile: tile + halos, widened to 16-byte boundaries.
-constexpr int kRawN = 4232;
+constexpr int kRawN = kLocalTile;
 static_assert(kRawN % 4 == 0 && kRawN >= TILE + 2 * kHalo + 6, "raw stage must hold an aligned tile + halos");
 constexpr int kGatherPer = (TILE + 2 * kHalo + 32 * kTmaGather - 1) / (32 * kTmaGather);
 constexpr int kKahanBatch = 4;                     // returning atomics in flight per consumer thread
@@ -112,10 +112,11 @@ struct TileSpan {
     int32_t n;
 };
 
-__device__ __forceinline__ TileSpan tile_span(const Tile &tl, const ObsInfo &ob, int halo)
+// local: the tile's pointing is block ti of kLocalTile samples instead.
+__device__ __forceinline__ TileSpan tile_span(const Tile &tl, const ObsInfo &ob, int halo, int64_t ti, bool local)
 {
     TileSpan sp;
-    sp.row = ob.tod_off + (int64_t)tl.det * ob.nsamp;
+    sp.row = local ? ti * kLocalTile - (tl.t0 - kHalo) : ob.tod_off + (int64_t)tl.det * ob.nsamp;
     const int64_t t_lo = tl.t0 - halo > 0 ? tl.t0 - halo : 0;
     const int64_t t_hi = tl.t0 + tl.len + halo < ob.nsamp ? tl.t0 + tl.len + halo : ob.nsamp;
     sp.g0 = (sp.row + t_lo) & ~int64_t(3);
@@ -136,7 +137,7 @@ __global__ void __launch_bounds__(tma_threads<KC>(), 1)
     fused_tma_kernel(const Tile *__restrict__ tiles, int64_t n_tiles, PointingView pv, NoiseView nv,
                      const float4 *__restrict__ x32, float4 *__restrict__ acc_hi, float4 *__restrict__ acc_lo,
                      double *__restrict__ acc64, unsigned *__restrict__ err, FusedTpl tpl, int l2_hint,
-                     const unsigned *__restrict__ done, unsigned n_obs)
+                     const unsigned *__restrict__ done, unsigned n_obs, bool local)
 {
     if (done && *done == n_obs) return;   // a PCG iteration after every observation has converged
     constexpr int kTmaConsumer = KC;
@@ -167,7 +168,7 @@ __global__ void __launch_bounds__(tma_threads<KC>(), 1)
             if (!mbar_wait(&S.raw_empty[r], par ^ 1u, err, budget)) break;
             const Tile tl = tiles[ti];
             const ObsInfo ob = pv.obs[tl.obs];
-            const TileSpan sp = tile_span(tl, ob, halo);
+            const TileSpan sp = tile_span(tl, ob, halo, ti, local);
             const uint32_t bytes = (uint32_t)sp.n * 4u;
             mbar_expect_tx(&S.raw_full[r], 3u * bytes + (TPL == 2 ? (uint32_t)sizeof(float4) : 0u));
             bulk_copy_g2s(S.pix[r], pv.pix + sp.g0, bytes, &S.raw_full[r], hint, pol);
@@ -196,7 +197,7 @@ __global__ void __launch_bounds__(tma_threads<KC>(), 1)
             const Tile tl = tiles[ti];
             const ObsInfo ob = pv.obs[tl.obs];
             const int64_t gdet = ob.det_off + tl.det;
-            const TileSpan sp = tile_span(tl, ob, halo);
+            const TileSpan sp = tile_span(tl, ob, halo, ti, local);
             if (BANDED && tid < kBandPad) {
                 const int k = tid < kHalo ? kHalo - tid : tid - kHalo;
                 const float c = (tid < kBand && k < nv.ntaps) ? nv.p32[gdet * nv.ntaps + k] : 0.f;
@@ -322,7 +323,7 @@ __global__ void __launch_bounds__(tma_threads<KC>(), 1)
         for (int i = 0; i < kConsOut; ++i)
             if (base + i < tl.len) ys[spos(base + i)] = y[i];
         consumers_sync<KC>();
-        const TileSpan sp = tile_span(tl, ob, halo);
+        const TileSpan sp = tile_span(tl, ob, halo, ti, local);
         const int64_t shift = sp.row + tl.t0 - sp.g0;   // stage index of core sample u
         double2 cs = make_double2(1.0, 0.0);
         if (pv.psi_cs) cs = pv.psi_cs[gdet];
@@ -392,48 +393,51 @@ __global__ void __launch_bounds__(tma_threads<KC>(), 1)
 
 template <int ACC, bool BANDED, int TPL, int KC>
 static furax_status run_tma_kc(const furax_pointing *p, const furax_noise *n, const float4 *x32, float4 *hi,
-                               float4 *lo, double *a64, const FusedTpl &ft, const unsigned *done, cudaStream_t st)
+                               float4 *lo, double *a64, const FusedTpl &ft, const unsigned *done, const TmaChunk *local,
+                               cudaStream_t st)
 {
-    const unsigned g = (unsigned)std::min<int64_t>(p->n_tiles, p->n_sm);
-    return launch_dyn(fused_tma_kernel<ACC, BANDED, TPL, KC>, g, tma_threads<KC>(), tma_smem<ACC, KC>(), st, p->d_tiles,
-                      p->n_tiles, p->view(), n->view(), x32, hi, lo, a64, p->d_err, ft, (int)p->sched.l2_evict_first,
-                      done, (unsigned)p->n_obs);
+    const int64_t nt = local ? local->n : p->n_tiles;
+    const unsigned g = (unsigned)std::min<int64_t>(nt, p->n_sm);
+    return launch_dyn(fused_tma_kernel<ACC, BANDED, TPL, KC>, g, tma_threads<KC>(), tma_smem<ACC, KC>(), st,
+                      (const Tile *)p->d_tiles + (local ? local->tile0 : 0), nt, local ? local->pv : p->view(), n->view(), x32,
+                      hi, lo, a64, p->d_err, ft, local ? 0 : (int)p->sched.l2_evict_first, done, (unsigned)p->n_obs,
+                      local != nullptr);
 }
 
 // 16 consumer warps when the schedule asks for them (plain operator only; the template modes keep 8).
 template <int ACC, bool BANDED, int TPL>
 static furax_status run_tma(const furax_pointing *p, const furax_noise *n, const float4 *x32, float4 *hi, float4 *lo,
-                            double *a64, const FusedTpl &ft, const unsigned *done, cudaStream_t st)
+                            double *a64, const FusedTpl &ft, const unsigned *done, const TmaChunk *local, cudaStream_t st)
 {
     if constexpr (TPL == 0)
-        if (p->sched.consumer_warps == 16) return run_tma_kc<ACC, BANDED, TPL, 16>(p, n, x32, hi, lo, a64, ft, done, st);
-    return run_tma_kc<ACC, BANDED, TPL, 8>(p, n, x32, hi, lo, a64, ft, done, st);
+        if (p->sched.consumer_warps == 16) return run_tma_kc<ACC, BANDED, TPL, 16>(p, n, x32, hi, lo, a64, ft, done, local, st);
+    return run_tma_kc<ACC, BANDED, TPL, 8>(p, n, x32, hi, lo, a64, ft, done, local, st);
 }
 
 template <bool BANDED, int TPL>
 static furax_status dispatch_tma(const furax_pointing *p, const furax_noise *n, const float4 *x32, int acc, float4 *hi,
-                                 float4 *lo, double *a64, const FusedTpl &ft, const unsigned *done, cudaStream_t st)
+                                 float4 *lo, double *a64, const FusedTpl &ft, const unsigned *done, const TmaChunk *local, cudaStream_t st)
 {
-    if (acc == FURAX_ACC_F32) return run_tma<FURAX_ACC_F32, BANDED, TPL>(p, n, x32, hi, lo, a64, ft, done, st);
-    if (acc == FURAX_ACC_F32_KAHAN) return run_tma<FURAX_ACC_F32_KAHAN, BANDED, TPL>(p, n, x32, hi, lo, a64, ft, done, st);
-    return run_tma<FURAX_ACC_F64, BANDED, TPL>(p, n, x32, hi, lo, a64, ft, done, st);
+    if (acc == FURAX_ACC_F32) return run_tma<FURAX_ACC_F32, BANDED, TPL>(p, n, x32, hi, lo, a64, ft, done, local, st);
+    if (acc == FURAX_ACC_F32_KAHAN) return run_tma<FURAX_ACC_F32_KAHAN, BANDED, TPL>(p, n, x32, hi, lo, a64, ft, done, local, st);
+    return run_tma<FURAX_ACC_F64, BANDED, TPL>(p, n, x32, hi, lo, a64, ft, done, local, st);
 }
 
 template <int TPL>
 static furax_status dispatch_tma_band(const furax_pointing *p, const furax_noise *n, const float4 *x32, int acc,
-                                      float4 *hi, float4 *lo, double *a64, const FusedTpl &ft, const unsigned *done, cudaStream_t st)
+                                      float4 *hi, float4 *lo, double *a64, const FusedTpl &ft, const unsigned *done, const TmaChunk *local, cudaStream_t st)
 {
-    return n->kind == FURAX_NOISE_BANDED ? dispatch_tma<true, TPL>(p, n, x32, acc, hi, lo, a64, ft, done, st)
-                                         : dispatch_tma<false, TPL>(p, n, x32, acc, hi, lo, a64, ft, done, st);
+    return n->kind == FURAX_NOISE_BANDED ? dispatch_tma<true, TPL>(p, n, x32, acc, hi, lo, a64, ft, done, local, st)
+                                         : dispatch_tma<false, TPL>(p, n, x32, acc, hi, lo, a64, ft, done, local, st);
 }
 
 furax_status launch_fused_tma(const furax_pointing *p, const furax_noise *n, const float4 *x32, int acc, float4 *hi,
-                              float4 *lo, double *a64, cudaStream_t st, const FusedTpl *ft, const unsigned *done)
+                              float4 *lo, double *a64, cudaStream_t st, const FusedTpl *ft, const unsigned *done, const TmaChunk *local)
 {
     const FusedTpl none{0, nullptr, 0, 0};
-    if (!ft || ft->mode == 0) return dispatch_tma_band<0>(p, n, x32, acc, hi, lo, a64, none, done, st);
-    if (ft->mode == 1) return dispatch_tma_band<1>(p, n, x32, acc, hi, lo, a64, *ft, done, st);
-    return dispatch_tma_band<2>(p, n, x32, acc, hi, lo, a64, *ft, done, st);
+    if (!ft || ft->mode == 0) return dispatch_tma_band<0>(p, n, x32, acc, hi, lo, a64, none, done, local, st);
+    if (ft->mode == 1) return dispatch_tma_band<1>(p, n, x32, acc, hi, lo, a64, *ft, done, local, st);
+    return dispatch_tma_band<2>(p, n, x32, acc, hi, lo, a64, *ft, done, local, st);
 }
 
 template <bool BANDED, int TPL, int KC>

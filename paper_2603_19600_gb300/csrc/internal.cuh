@@ -201,6 +201,8 @@ struct furax_pointing {
     void *ws_tod = nullptr;           // [nsamp] scratch TOD (FP64 size)
     void *ws_tod2 = nullptr;
     int32_t *ws_hits = nullptr;       // [npix] hit counts when the caller passes none
+    int32_t *ws_local_pix = nullptr;  // on the fly: pointing of one chunk of tiles (fused_f32.cu)
+    float *ws_local_c = nullptr, *ws_local_s = nullptr;
     float *ws_bore_m = nullptr;       // [nbore][20] boresight rotation matrices (double-FP32, pointing_fast.cuh)
     fx::CgWs *cg = nullptr;           // solver workspace (allocated by the first solve)
     // operator schedule (furax_pointing_set_schedule); pixel-sorted tiles and their permutation
@@ -289,6 +291,13 @@ furax_status launch_set_psi(furax_pointing *p, const double *psi, cudaStream_t s
 furax_status launch_set_hwp(furax_pointing *p, const double *hwp, cudaStream_t st);
 // FP32 cache fill with certified FP32 pixels and exact FP64 fallback (pointing_fast.cu)
 furax_status launch_expand_fast(const furax_pointing *p, unsigned long long *n_invalid, cudaStream_t st);
+// On the fly: the boresight rows, then the same pointing for n tiles from tile0 on with their halos, each in its own
+// block (tile.cuh: kLocalTile).
+furax_status launch_bore_rows(const furax_pointing *p, cudaStream_t st);
+furax_status launch_expand_local(const furax_pointing *p, int64_t tile0, int64_t n, int32_t *pix, float *c, float *s,
+                                 cudaStream_t st);
+// Kernel launches of one FP32 application on the fly.
+int64_t on_the_fly_launches(const furax_pointing *p);
 furax_status launch_P(const furax_pointing *p, const void *map, int map_t, void *tod, int tod_t, cudaStream_t st);
 furax_status launch_PT(const furax_pointing *p, const void *tod, int tod_t, void *map, int map_t, int acc,
                        int32_t *hits, int accumulate, cudaStream_t st);

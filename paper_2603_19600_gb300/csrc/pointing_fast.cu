@@ -27,6 +27,7 @@
 #include "internal.cuh"
 #include "pointing_math.cuh"
 #include "pointing_fast.cuh"
+#include "tile.cuh"
 
 namespace fx {
 
@@ -51,8 +52,8 @@ __global__ void bore_matrix_kernel(const double *__restrict__ q_bore, int64_t n,
         float h[9], l[9];
 #pragma unroll
         for (int k = 0; k < 9; ++k) {
-            h[k] = (float)r[k];
-            l[k] = (float)(r[k] - (double)h[k]);
+            h[k] = f64_to_f32_bits(r[k]);   // conversions off the FP64 pipe, which bounds this kernel
+            l[k] = f64_to_f32_bits(r[k] - f32_to_f64_bits(h[k]));
         }
         o[0] = make_float4(h[0], h[1], h[2], h[3]);
         o[1] = make_float4(h[4], h[5], l[0], l[1]);
@@ -67,6 +68,9 @@ __global__ void bore_matrix_kernel(const double *__restrict__ q_bore, int64_t n,
 // boresight matrices and integer remainders; 537 us packed, with 16-byte loads and without remainders. Smaller
 // blocks (128 threads: 545 us; 64: 681 us) load the detector axes more often. Tighter margins would send fewer samples
 // to the exact recipe, but those would change their weights' rounding.
+// HALO: 0 for the cache (flat time-ordered index), else the halo on both sides of each tile, which is written to
+// its own block of kLocalTile samples (slot u = sample t0 - HALO + u).
+template <int HALO>
 __global__ void __launch_bounds__(256, 4) expand_fast_kernel(const Tile *__restrict__ tiles, const ObsInfo *__restrict__ obs,
                                                           const double *__restrict__ q_bore, const double *__restrict__ q_det,
                                                           const float *__restrict__ bm, const double2 *__restrict__ hwp_cs,
@@ -76,7 +80,7 @@ __global__ void __launch_bounds__(256, 4) expand_fast_kernel(const Tile *__restr
 {
     __shared__ int qn, sdet_ok;
     __shared__ float sdet[12];   // detector axes: d hi, d lo, o hi, o lo
-    __shared__ int32_t queue[TILE];
+    __shared__ int32_t queue[TILE + 2 * HALO];
     const Tile tl = tiles[blockIdx.x];
     const ObsInfo ob = obs[tl.obs];
     const int64_t gdet = ob.det_off + tl.det;
@@ -89,9 +93,10 @@ __global__ void __launch_bounds__(256, 4) expand_fast_kernel(const Tile *__restr
     __syncthreads();
     const DetAxes ax(sdet);
     const bool det_ok = sdet_ok != 0;
-    const int64_t row = ob.tod_off + tl.det * ob.nsamp;
-    for (int k = threadIdx.x; k < tl.len; k += blockDim.x) {
-        const int64_t t = tl.t0 + k;
+    const int64_t row = HALO ? (int64_t)blockIdx.x * kLocalTile - (tl.t0 - HALO) : ob.tod_off + tl.det * ob.nsamp;
+    for (int k = threadIdx.x; k < tl.len + 2 * HALO; k += blockDim.x) {
+        const int64_t t = tl.t0 - HALO + k;
+        if (HALO && (t < 0 || t >= ob.nsamp)) continue;
         int32_t p = -1;
         float c = 1.f, s = 0.f;
         bool ok = det_ok && certified_sample(bm + kBoreRow * (ob.bore_off + t), ax, (int32_t)ob.nside, p, c, s);
@@ -109,7 +114,7 @@ __global__ void __launch_bounds__(256, 4) expand_fast_kernel(const Tile *__restr
     const int nq = qn;
     int bad = 0;
     for (int j = threadIdx.x; j < nq; j += blockDim.x) {
-        const int64_t t = tl.t0 + queue[j];
+        const int64_t t = tl.t0 - HALO + queue[j];
         const SampleF64 r = point_f64(load_quat(q_bore, ob.bore_off + t), qd, ob.nside);
         double c = r.c, s = r.s;
         if (hwp_cs && r.pix >= 0) apply_hwp<double>(c, s, hwp_cs[ob.bore_off + t]);
@@ -124,20 +129,35 @@ __global__ void __launch_bounds__(256, 4) expand_fast_kernel(const Tile *__restr
     }
 }
 
-furax_status launch_expand_fast(const furax_pointing *p, unsigned long long *n_invalid, cudaStream_t st)
+// The boresight rows from the handle's current quaternions.
+furax_status launch_bore_rows(const furax_pointing *p, cudaStream_t st)
 {
     furax_pointing *pm = const_cast<furax_pointing *>(p);
-    furax_status rc;
-    if ((rc = ensure_ws(pm, (void **)&pm->ws_bore_m, sizeof(float) * kBoreRow * std::max<int64_t>(1, p->nbore_total))))
-        return rc;
+    furax_status rc = ensure_ws(pm, (void **)&pm->ws_bore_m, sizeof(float) * kBoreRow * std::max<int64_t>(1, p->nbore_total));
+    if (rc) return rc;
     const unsigned g = (unsigned)std::max<int64_t>(1, std::min<int64_t>((p->nbore_total + 255) / 256, 16LL * p->n_sm));
     bore_matrix_kernel<<<g, 256, 0, st>>>(p->q_bore, p->nbore_total, pm->ws_bore_m);
     count_launches(1);
-    if ((rc = check_launch("boresight matrices"))) return rc;
+    return check_launch("boresight matrices");
+}
+
+furax_status launch_expand_local(const furax_pointing *p, int64_t tile0, int64_t n, int32_t *pix, float *c, float *s,
+                                 cudaStream_t st)
+{
+    expand_fast_kernel<kHalo><<<(unsigned)n, 256, 0, st>>>(p->d_tiles + tile0, p->d_obs, p->q_bore, p->q_det, p->ws_bore_m,
+                                                           p->has_hwp ? p->d_hwp_cs : nullptr, pix, c, s, nullptr);
+    count_launches(1);
+    return check_launch("pointing of a chunk of tiles");
+}
+
+furax_status launch_expand_fast(const furax_pointing *p, unsigned long long *n_invalid, cudaStream_t st)
+{
+    furax_status rc = launch_bore_rows(p, st);
+    if (rc) return rc;
     if (p->n_tiles == 0) return FURAX_OK;
-    expand_fast_kernel<<<(unsigned)p->n_tiles, 256, 0, st>>>(p->d_tiles, p->d_obs, p->q_bore, p->q_det, pm->ws_bore_m,
-                                                             p->has_hwp ? p->d_hwp_cs : nullptr, p->pix, p->c32,
-                                                             p->s32, n_invalid);
+    expand_fast_kernel<0><<<(unsigned)p->n_tiles, 256, 0, st>>>(p->d_tiles, p->d_obs, p->q_bore, p->q_det, p->ws_bore_m,
+                                                                p->has_hwp ? p->d_hwp_cs : nullptr, p->pix, p->c32,
+                                                                p->s32, n_invalid);
     count_launches(1);
     return check_launch("fast pointing expansion");
 }

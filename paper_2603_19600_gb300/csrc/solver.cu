@@ -675,6 +675,8 @@ static furax_status body(const Body &b, cudaStream_t st, cudaEvent_t e0, cudaEve
 
 static int64_t graph_nodes_per_iter(const Body &b)
 {
+    if (b.precision != FURAX_F64 && !long_band(b.n) && b.p->mode == FURAX_POINTING_ON_THE_FLY)
+        return 3 + on_the_fly_launches(b.p) + (b.tp ? 3 : 0);
     if (b.aug) return 4;
     const bool lb = long_band(b.n);
     int64_t k = 3 + (lb ? 3 : 1);

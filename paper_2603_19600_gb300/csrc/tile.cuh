@@ -34,6 +34,10 @@ __device__ __forceinline__ T white_scale(const NoiseView &nv, int64_t gdet)
     else return nv.p64[gdet];
 }
 
+// Pointing of one tile and its halos kept on its own (on the fly): slot u is sample t0 - kHalo + u.
+constexpr int kLocalTile = 4232;
+static_assert(kLocalTile % 4 == 0 && kLocalTile >= TILE + 2 * kHalo + 6, "a tile's block stays 16-byte aligned");
+
 constexpr size_t kF32Smem = sizeof(float) * (XS + MAXTAPS + 2 * XS) + sizeof(int32_t) * XS;
 
 // Kernel shared-memory setup for each translation unit (called once, outside stream capture).
@@ -44,8 +48,13 @@ furax_status prepare_fused_tma();
 // Cached FP32 pointing: persistent TMA-pipelined operator (cache rows must be readable up to the
 // next 16-byte boundary past the last sample).
 // With ft, also does the template work of ft->mode (projection, or the augmented system).
+// local: n tiles from tile0 on, whose pointing lies in pv as blocks of kLocalTile samples.
+struct TmaChunk {
+    int64_t tile0, n;
+    PointingView pv;
+};
 furax_status launch_fused_tma(const furax_pointing *p, const furax_noise *n, const float4 *x32, int acc, float4 *hi,
                               float4 *lo, double *a64, cudaStream_t st, const FusedTpl *ft = nullptr,
-                              const unsigned *done = nullptr);
+                              const unsigned *done = nullptr, const TmaChunk *local = nullptr);
 
 }  // namespace fx
