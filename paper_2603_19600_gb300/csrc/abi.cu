@@ -699,20 +699,25 @@ furax_status furax_rhs(const furax_pointing_t *p, const furax_noise_t *n, const 
     REQUIRE(valid_dtype(d_t), "unknown dtype %d", d_t);
     furax_pointing *pm = const_cast<furax_pointing *>(p);
     cudaStream_t st = (cudaStream_t)stream;
-    if ((rc = ensure_ws(pm, (void **)&pm->ws_acc64, sizeof(double) * 3 * p->npix_total))) return rc;
-    if ((rc = check_cuda(cudaMemsetAsync(pm->ws_acc64, 0, sizeof(double) * 3 * p->npix_total, st), "memset"))) return rc;
+    // Unmasked sums go straight into b (as in ptnp_apply: no copying pass, 67 M samples, nside 512: 1409 -> 1382 us).
+    const size_t bytes = sizeof(double) * 3 * p->npix_total;
+    const bool direct = !valid && apart(d, (d_t == FURAX_F64 ? 8 : 4) * (size_t)p->nsamp_total, b, bytes);
+    if (long_band(n) && (rc = tod_ws(p))) return rc;
+    if (!direct && (rc = ensure_ws(pm, (void **)&pm->ws_acc64, bytes))) return rc;
+    double *sum = direct ? b : pm->ws_acc64;
+    if ((rc = check_cuda(cudaMemsetAsync(sum, 0, bytes, st), "memset"))) return rc;
     const bool prof = prof_on();
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     if (prof) { prof_pair(&e0, &e1); if (e0) cudaEventRecord(e0, st); }
     // FP64-accurate, the band product on the tensor cores.
     // A band longer than the fused kernels hold: overlap-save N^-1 in FP64 with the TOD in HBM.
     if (long_band(n)) {
-        if ((rc = tod_ws(p)) || (rc = launch_rhs_chain(p, n, d, d_t, pm->ws_acc64, st))) return rc;
-    } else if ((rc = launch_rhs_tc(p, n, d, d_t, pm->ws_acc64, false, st))) {
+        if ((rc = launch_rhs_chain(p, n, d, d_t, sum, st))) return rc;
+    } else if ((rc = launch_rhs_tc(p, n, d, d_t, sum, false, st))) {
         return rc;
     }
     if (prof) { if (e1) cudaEventRecord(e1, st); prof_push(2, e0, e1); }
-    return launch_finalize_acc(p, FURAX_ACC_F64, nullptr, nullptr, pm->ws_acc64, valid, b, st);
+    return direct ? FURAX_OK : launch_finalize_acc(p, FURAX_ACC_F64, nullptr, nullptr, sum, valid, b, st);
 }
 
 void furax_cg_default_opts(furax_cg_opts *o)

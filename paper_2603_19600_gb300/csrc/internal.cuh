@@ -346,6 +346,11 @@ furax_status launch_chi2_grad(const furax_pointing *p, const furax_noise *n, con
 // Build (or drop, for the time-ordered kernel) the pixel-sorted tiles of a cached FP32 pointing and
 // sort them; synchronises st. The permutation follows the cache: sort_sorted_tiles after a refresh.
 furax_status set_schedule(furax_pointing *p, const furax_schedule &s, cudaStream_t st);
+// Two buffers share no byte: FP64 reductions may then go straight into the output while the input is read.
+inline bool apart(const void *a, size_t na, const void *b, size_t nb)
+{
+    return (const char *)a + na <= (const char *)b || (const char *)b + nb <= (const char *)a;
+}
 furax_status sort_sorted_tiles(const furax_pointing *p, cudaStream_t st);
 bool sorted_active(const furax_pointing *p);
 void free_sorted(furax_pointing *p);

@@ -219,45 +219,53 @@ furax_status ptnp_apply(const furax_pointing *p, const furax_noise *n, const dou
     furax_pointing *pm = const_cast<furax_pointing *>(p);
     const int64_t np = p->npix_total;
     furax_status rc;
+    // Without a mask or templates the FP64 sums go straight into out, without a pass over the map that copies them
+    // (nside 512: 16.8 M samples on the fly 651 -> 625 us, 268 M cached 3804 -> 3782 us; nside 256: FP64 290 -> 279 us).
+    const bool direct = !valid && !tp && apart(x, sizeof(double) * 3 * np, out, sizeof(double) * 3 * np);
+    double *sum = out;
+    if (!direct && (long_band(n) || precision != FURAX_F32 || acc == FURAX_ACC_F64)) {
+        if ((rc = ensure_ws(pm, (void **)&pm->ws_acc64, sizeof(double) * 3 * np))) return rc;
+        sum = pm->ws_acc64;
+    }
+    auto done = [&] {
+        return direct ? FURAX_OK : launch_finalize_acc(p, FURAX_ACC_F64, nullptr, nullptr, sum, valid, out, st);
+    };
     if (long_band(n)) {
         // the band does not fit the fused kernels: P, overlap-save N^-1 and P^T with the TOD in HBM,
         // FP64 accumulation (FP32 TOD for precision FURAX_F32)
         if ((rc = tod_ws(p))) return rc;
-        if ((rc = ensure_ws(pm, (void **)&pm->ws_acc64, sizeof(double) * 3 * np))) return rc;
         const double *xin = x;
         if (valid) {
             if ((rc = ensure_ws(pm, (void **)&pm->ws_x64, sizeof(double) * 3 * np))) return rc;
             if ((rc = launch_mask_copy(p, x, valid, pm->ws_x64, st))) return rc;
             xin = pm->ws_x64;
         }
-        if ((rc = check_cuda(cudaMemsetAsync(pm->ws_acc64, 0, sizeof(double) * 3 * np, st), "memset"))) return rc;
+        if ((rc = check_cuda(cudaMemsetAsync(sum, 0, sizeof(double) * 3 * np, st), "memset"))) return rc;
         const int tod_t = precision == FURAX_F32 ? FURAX_F32 : FURAX_F64;
-        if ((rc = launch_ata_chain(p, n, xin, tod_t, pm->ws_acc64, st))) return rc;
-        if (tp && (rc = launch_tpl_map(tp, FURAX_F64, FURAX_ACC_F64, nullptr, xin, nullptr, nullptr, pm->ws_acc64, st)))
+        if ((rc = launch_ata_chain(p, n, xin, tod_t, sum, st))) return rc;
+        if (tp && (rc = launch_tpl_map(tp, FURAX_F64, FURAX_ACC_F64, nullptr, xin, nullptr, nullptr, sum, st)))
             return rc;
-        return launch_finalize_acc(p, FURAX_ACC_F64, nullptr, nullptr, pm->ws_acc64, valid, out, st);
+        return done();
     }
     if (precision == FURAX_F64 || precision == FURAX_PREC_F32X2) {
-        if ((rc = ensure_ws(pm, (void **)&pm->ws_acc64, sizeof(double) * 3 * np))) return rc;
         const double *xin = x;   // the templates' pass reads a masked map
         if (valid && tp) {
             if ((rc = ensure_ws(pm, (void **)&pm->ws_x64, sizeof(double) * 3 * np))) return rc;
             if ((rc = launch_mask_copy(p, x, valid, pm->ws_x64, st))) return rc;
             xin = pm->ws_x64;
         }
-        if ((rc = check_cuda(cudaMemsetAsync(pm->ws_acc64, 0, sizeof(double) * 3 * np, st), "memset"))) return rc;
+        if ((rc = check_cuda(cudaMemsetAsync(sum, 0, sizeof(double) * 3 * np, st), "memset"))) return rc;
         const bool f64 = precision == FURAX_F64;
-        if ((rc = timed(f64 ? 1 : 2, st, [&] { return launch_fused_tc(p, n, x, valid, pm->ws_acc64, f64, st); }))) return rc;
-        if (tp && (rc = launch_tpl_map(tp, FURAX_F64, FURAX_ACC_F64, nullptr, xin, nullptr, nullptr, pm->ws_acc64, st)))
+        if ((rc = timed(f64 ? 1 : 2, st, [&] { return launch_fused_tc(p, n, x, valid, sum, f64, st); }))) return rc;
+        if (tp && (rc = launch_tpl_map(tp, FURAX_F64, FURAX_ACC_F64, nullptr, xin, nullptr, nullptr, sum, st)))
             return rc;
-        return launch_finalize_acc(p, FURAX_ACC_F64, nullptr, nullptr, pm->ws_acc64, valid, out, st);
+        return done();
     }
     if ((rc = ensure_ws(pm, (void **)&pm->ws_map32, sizeof(float4) * np))) return rc;
     float4 *hi = nullptr, *lo = nullptr;
     double *a64 = nullptr;
     if (acc == FURAX_ACC_F64) {
-        if ((rc = ensure_ws(pm, (void **)&pm->ws_acc64, sizeof(double) * 3 * np))) return rc;
-        a64 = pm->ws_acc64;
+        a64 = sum;
         if ((rc = check_cuda(cudaMemsetAsync(a64, 0, sizeof(double) * 3 * np, st), "memset"))) return rc;
     } else {
         if ((rc = ensure_ws(pm, (void **)&pm->ws_acc_hi, sizeof(float4) * kKahanStride * np))) return rc;
@@ -272,7 +280,7 @@ furax_status ptnp_apply(const furax_pointing *p, const furax_noise *n, const dou
         return rc;
     if (tp && (rc = launch_tpl_map(tp, FURAX_F32, acc, pm->ws_map32, nullptr, hi, lo, a64, st, tpl_a != nullptr)))
         return rc;
-    return launch_finalize_acc(p, acc, hi, lo, a64, valid, out, st);
+    return acc == FURAX_ACC_F64 ? done() : launch_finalize_acc(p, acc, hi, lo, nullptr, valid, out, st);
 }
 
 // ------------------------------------------------------------------------------------
