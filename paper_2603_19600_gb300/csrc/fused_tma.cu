@@ -132,12 +132,14 @@ __device__ __forceinline__ TileSpan tile_span(const Tile &tl, const ObsInfo &ob,
 //   TPL 2: the augmented system [m; a]: u_t = (P m)_t + sum_l a_l P_l(tau_t) with the detector's
 //          amplitudes a (l <= 2) read from x32[tpl.base + det], and T^T z (l <= tpl.order)
 //          accumulated into the amplitude pseudo-pixel tpl.base + det like a pixel.
-template <int ACC, bool BANDED, int TPL, int KC>
+// LOCAL: the tiles' pointing lies in blocks of its own (a compile-time switch: as an argument it cost the augmented kernel,
+// which uses every register, 4.14 -> 4.45 ms per 268 M samples).
+template <int ACC, bool BANDED, int TPL, int KC, bool LOCAL>
 __global__ void __launch_bounds__(tma_threads<KC>(), 1)
     fused_tma_kernel(const Tile *__restrict__ tiles, int64_t n_tiles, PointingView pv, NoiseView nv,
                      const float4 *__restrict__ x32, float4 *__restrict__ acc_hi, float4 *__restrict__ acc_lo,
                      double *__restrict__ acc64, unsigned *__restrict__ err, FusedTpl tpl, int l2_hint,
-                     const unsigned *__restrict__ done, unsigned n_obs, bool local)
+                     const unsigned *__restrict__ done, unsigned n_obs)
 {
     if (done && *done == n_obs) return;   // a PCG iteration after every observation has converged
     constexpr int kTmaConsumer = KC;
@@ -168,7 +170,7 @@ __global__ void __launch_bounds__(tma_threads<KC>(), 1)
             if (!mbar_wait(&S.raw_empty[r], par ^ 1u, err, budget)) break;
             const Tile tl = tiles[ti];
             const ObsInfo ob = pv.obs[tl.obs];
-            const TileSpan sp = tile_span(tl, ob, halo, ti, local);
+            const TileSpan sp = tile_span(tl, ob, halo, ti, LOCAL);
             const uint32_t bytes = (uint32_t)sp.n * 4u;
             mbar_expect_tx(&S.raw_full[r], 3u * bytes + (TPL == 2 ? (uint32_t)sizeof(float4) : 0u));
             bulk_copy_g2s(S.pix[r], pv.pix + sp.g0, bytes, &S.raw_full[r], hint, pol);
@@ -197,7 +199,7 @@ __global__ void __launch_bounds__(tma_threads<KC>(), 1)
             const Tile tl = tiles[ti];
             const ObsInfo ob = pv.obs[tl.obs];
             const int64_t gdet = ob.det_off + tl.det;
-            const TileSpan sp = tile_span(tl, ob, halo, ti, local);
+            const TileSpan sp = tile_span(tl, ob, halo, ti, LOCAL);
             if (BANDED && tid < kBandPad) {
                 const int k = tid < kHalo ? kHalo - tid : tid - kHalo;
                 const float c = (tid < kBand && k < nv.ntaps) ? nv.p32[gdet * nv.ntaps + k] : 0.f;
@@ -323,7 +325,7 @@ __global__ void __launch_bounds__(tma_threads<KC>(), 1)
         for (int i = 0; i < kConsOut; ++i)
             if (base + i < tl.len) ys[spos(base + i)] = y[i];
         consumers_sync<KC>();
-        const TileSpan sp = tile_span(tl, ob, halo, ti, local);
+        const TileSpan sp = tile_span(tl, ob, halo, ti, LOCAL);
         const int64_t shift = sp.row + tl.t0 - sp.g0;   // stage index of core sample u
         double2 cs = make_double2(1.0, 0.0);
         if (pv.psi_cs) cs = pv.psi_cs[gdet];
@@ -391,17 +393,16 @@ __global__ void __launch_bounds__(tma_threads<KC>(), 1)
     }
 }
 
-template <int ACC, bool BANDED, int TPL, int KC>
+template <int ACC, bool BANDED, int TPL, int KC, bool LOCAL = false>
 static furax_status run_tma_kc(const furax_pointing *p, const furax_noise *n, const float4 *x32, float4 *hi,
                                float4 *lo, double *a64, const FusedTpl &ft, const unsigned *done, const TmaChunk *local,
                                cudaStream_t st)
 {
     const int64_t nt = local ? local->n : p->n_tiles;
     const unsigned g = (unsigned)std::min<int64_t>(nt, p->n_sm);
-    return launch_dyn(fused_tma_kernel<ACC, BANDED, TPL, KC>, g, tma_threads<KC>(), tma_smem<ACC, KC>(), st,
+    return launch_dyn(fused_tma_kernel<ACC, BANDED, TPL, KC, LOCAL>, g, tma_threads<KC>(), tma_smem<ACC, KC>(), st,
                       (const Tile *)p->d_tiles + (local ? local->tile0 : 0), nt, local ? local->pv : p->view(), n->view(), x32,
-                      hi, lo, a64, p->d_err, ft, local ? 0 : (int)p->sched.l2_evict_first, done, (unsigned)p->n_obs,
-                      local != nullptr);
+                      hi, lo, a64, p->d_err, ft, local ? 0 : (int)p->sched.l2_evict_first, done, (unsigned)p->n_obs);
 }
 
 // 16 consumer warps when the schedule asks for them (plain operator only; the template modes keep 8).
@@ -409,8 +410,10 @@ template <int ACC, bool BANDED, int TPL>
 static furax_status run_tma(const furax_pointing *p, const furax_noise *n, const float4 *x32, float4 *hi, float4 *lo,
                             double *a64, const FusedTpl &ft, const unsigned *done, const TmaChunk *local, cudaStream_t st)
 {
-    if constexpr (TPL == 0)
+    if constexpr (TPL == 0) {
+        if (local) return run_tma_kc<ACC, BANDED, TPL, 8, true>(p, n, x32, hi, lo, a64, ft, done, local, st);
         if (p->sched.consumer_warps == 16) return run_tma_kc<ACC, BANDED, TPL, 16>(p, n, x32, hi, lo, a64, ft, done, local, st);
+    }
     return run_tma_kc<ACC, BANDED, TPL, 8>(p, n, x32, hi, lo, a64, ft, done, local, st);
 }
 
@@ -440,13 +443,13 @@ furax_status launch_fused_tma(const furax_pointing *p, const furax_noise *n, con
     return dispatch_tma_band<2>(p, n, x32, acc, hi, lo, a64, *ft, done, local, st);
 }
 
-template <bool BANDED, int TPL, int KC>
+template <bool BANDED, int TPL, int KC, bool LOCAL = false>
 static furax_status prepare_tma_band()
 {
     furax_status rc = FURAX_OK;
-    if (!rc) rc = allow_smem((const void *)fused_tma_kernel<FURAX_ACC_F32, BANDED, TPL, KC>, tma_smem<FURAX_ACC_F32, KC>());
-    if (!rc) rc = allow_smem((const void *)fused_tma_kernel<FURAX_ACC_F32_KAHAN, BANDED, TPL, KC>, tma_smem<FURAX_ACC_F32_KAHAN, KC>());
-    if (!rc) rc = allow_smem((const void *)fused_tma_kernel<FURAX_ACC_F64, BANDED, TPL, KC>, tma_smem<FURAX_ACC_F64, KC>());
+    if (!rc) rc = allow_smem((const void *)fused_tma_kernel<FURAX_ACC_F32, BANDED, TPL, KC, LOCAL>, tma_smem<FURAX_ACC_F32, KC>());
+    if (!rc) rc = allow_smem((const void *)fused_tma_kernel<FURAX_ACC_F32_KAHAN, BANDED, TPL, KC, LOCAL>, tma_smem<FURAX_ACC_F32_KAHAN, KC>());
+    if (!rc) rc = allow_smem((const void *)fused_tma_kernel<FURAX_ACC_F64, BANDED, TPL, KC, LOCAL>, tma_smem<FURAX_ACC_F64, KC>());
     return rc;
 }
 
@@ -455,6 +458,8 @@ furax_status prepare_fused_tma()
     furax_status rc = FURAX_OK;
     if (!rc) rc = prepare_tma_band<true, 0, 8>();
     if (!rc) rc = prepare_tma_band<false, 0, 8>();
+    if (!rc) rc = prepare_tma_band<true, 0, 8, true>();
+    if (!rc) rc = prepare_tma_band<false, 0, 8, true>();
     if (!rc) rc = prepare_tma_band<true, 0, 16>();
     if (!rc) rc = prepare_tma_band<false, 0, 16>();
     if (!rc) rc = prepare_tma_band<true, 1, 8>();
