@@ -53,7 +53,7 @@ __global__ void __launch_bounds__(TT, 2) chi2_tc_kernel(const Tile *__restrict__
         TcPix m;
         DT d;
     };
-    tc_each<MODE, TT, 2>(pv, ob, tl, psi, [&](int k, int32_t pix) {
+    tc_each<MODE == 0 && BANDED ? kTcKept : MODE, TT, 2>(pv, ob, tl, psi, [&](int k, int32_t pix) {
         In in;
         in.m.load(m, ob.map_off + max(pix, 0));
         if constexpr (!BANDED) in.d = __ldg(row + tl.t0 + k);
@@ -100,6 +100,13 @@ template <int MODE, typename DT>
 static furax_status run_chi2_tc(const furax_pointing *p, const furax_noise *n, const DT *d, const double4_32a *m, double *chi2,
                                 double *gm, double *gp, bool f64, cudaStream_t st)
 {
+    if constexpr (MODE == 0) {
+        if (n->kind == FURAX_NOISE_BANDED)
+            return each_kept_chunk(p, [&](const Tile *tiles, unsigned g, const PointingView &pv) {
+                return launch_dyn(chi2_tc_kernel<MODE, true, DT>, g, TT, kTcSmem, st, tiles, pv, n->view(), d, m, chi2, gm, gp,
+                                  p->d_err, f64);
+            });
+    }
     if (n->kind == FURAX_NOISE_BANDED)
         return launch_dyn(chi2_tc_kernel<MODE, true, DT>, (unsigned)p->n_tiles, TT, kTcSmem, st, p->d_tiles, p->view(),
                           n->view(), d, m, chi2, gm, gp, p->d_err, f64);

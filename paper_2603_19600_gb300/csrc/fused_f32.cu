@@ -119,6 +119,20 @@ static furax_status dispatch_fused_f32(const furax_pointing *p, const furax_nois
 // bytes per sample through memory. The workspace (250 MB) is all that on-the-fly pointing ever holds.
 static int64_t chunk_tiles(const furax_pointing *p) { return std::min<int64_t>(p->n_tiles, 32LL * p->n_sm); }
 
+// The same workspace holds the FP64 pointing of half as many tiles (fused_tc.cu, chi2_tc.cu).
+int64_t kept_tiles(const furax_pointing *p) { return std::min<int64_t>(p->n_tiles, 16LL * p->n_sm); }
+
+furax_status ensure_local_ws(const furax_pointing *p)
+{
+    furax_pointing *pm = const_cast<furax_pointing *>(p);
+    const size_t pix = sizeof(float) * kLocalTile * (size_t)chunk_tiles(p);
+    const size_t w = std::max(pix, sizeof(double) * TILE * (size_t)kept_tiles(p));
+    furax_status rc = ensure_ws(pm, (void **)&pm->ws_local_pix, pix);
+    if (!rc) rc = ensure_ws(pm, (void **)&pm->ws_local_c, w);
+    if (!rc) rc = ensure_ws(pm, (void **)&pm->ws_local_s, w);
+    return rc;
+}
+
 int64_t on_the_fly_launches(const furax_pointing *p)
 {
     const int64_t c = chunk_tiles(p);
@@ -130,11 +144,8 @@ static furax_status apply_on_the_fly(const furax_pointing *p, const furax_noise 
 {
     furax_pointing *pm = const_cast<furax_pointing *>(p);
     const int64_t c = chunk_tiles(p);
-    const size_t bytes = sizeof(float) * kLocalTile * (size_t)c;
     furax_status rc;
-    if ((rc = ensure_ws(pm, (void **)&pm->ws_local_pix, bytes)) || (rc = ensure_ws(pm, (void **)&pm->ws_local_c, bytes)) ||
-        (rc = ensure_ws(pm, (void **)&pm->ws_local_s, bytes)) || (rc = launch_bore_rows(p, st)))
-        return rc;
+    if ((rc = ensure_local_ws(p)) || (rc = launch_bore_rows(p, st))) return rc;
     TmaChunk chunk{0, 0, p->view()};
     chunk.pv.pix = p->ws_local_pix;
     chunk.pv.c32 = p->ws_local_c;

@@ -76,7 +76,7 @@ __global__ void __launch_bounds__(TT, 2) tc_operator_kernel(const Tile *__restri
     }
     const double *ys = tc_ys(sm);
     double *rec = acc64 + 3 * ob.map_off;
-    tc_each<MODE, TT, 4>(pv, ob, tl, psi, [](int, int32_t) { return TcNone{}; },
+    tc_each<MODE == 0 && !FROM_TOD ? kTcKept : MODE, TT, 4>(pv, ob, tl, psi, [](int, int32_t) { return TcNone{}; },
                          [&](int k, int32_t pix, double c, double s, TcNone) {
         double y = pix >= 0 ? ys[spos(k)] : 0.0;
         if constexpr (TPL)
@@ -165,6 +165,13 @@ template <int MODE, bool FROM_TOD, bool TPL, typename DT>
 static furax_status run_tc(const furax_pointing *p, const furax_noise *n, const double4_32a *x, const DT *d, double *a64,
                            bool f64, const TplView &tv, const unsigned *done, cudaStream_t st)
 {
+    if constexpr (MODE == 0 && !FROM_TOD) {
+        if (n->kind == FURAX_NOISE_BANDED)
+            return each_kept_chunk(p, [&](const Tile *tiles, unsigned g, const PointingView &pv) {
+                return launch_dyn(tc_operator_kernel<MODE, FROM_TOD, TPL, DT>, g, TT, kTcSmem, st, tiles, pv, n->view(), x, d, a64,
+                                  p->d_err, f64, tv, done, (unsigned)p->n_obs);
+            });
+    }
     if (n->kind == FURAX_NOISE_BANDED)
         return launch_dyn(tc_operator_kernel<MODE, FROM_TOD, TPL, DT>, (unsigned)p->n_tiles, TT, kTcSmem, st, p->d_tiles,
                           p->view(), n->view(), x, d, a64, p->d_err, f64, tv, done, (unsigned)p->n_obs);

@@ -201,7 +201,7 @@ struct furax_pointing {
     void *ws_tod = nullptr;           // [nsamp] scratch TOD (FP64 size)
     void *ws_tod2 = nullptr;
     int32_t *ws_hits = nullptr;       // [npix] hit counts when the caller passes none
-    int32_t *ws_local_pix = nullptr;  // on the fly: pointing of one chunk of tiles (fused_f32.cu)
+    int32_t *ws_local_pix = nullptr;  // on the fly: pointing of one chunk of tiles (fused_f32.cu; FP64: tc_sample.cuh)
     float *ws_local_c = nullptr, *ws_local_s = nullptr;
     float *ws_bore_m = nullptr;       // [nbore][20] boresight rotation matrices (double-FP32, pointing_fast.cuh)
     fx::CgWs *cg = nullptr;           // solver workspace (allocated by the first solve)
@@ -298,6 +298,9 @@ furax_status launch_expand_local(const furax_pointing *p, int64_t tile0, int64_t
                                  cudaStream_t st);
 // Kernel launches of one FP32 application on the fly.
 int64_t on_the_fly_launches(const furax_pointing *p);
+// Workspace of on-the-fly pointing, and how many tiles of FP64 pointing (TILE samples each) it holds.
+furax_status ensure_local_ws(const furax_pointing *p);
+int64_t kept_tiles(const furax_pointing *p);
 furax_status launch_P(const furax_pointing *p, const void *map, int map_t, void *tod, int tod_t, cudaStream_t st);
 furax_status launch_PT(const furax_pointing *p, const void *tod, int tod_t, void *map, int map_t, int acc,
                        int32_t *hits, int accumulate, cudaStream_t st);

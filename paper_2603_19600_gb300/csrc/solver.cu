@@ -687,7 +687,11 @@ static int64_t graph_nodes_per_iter(const Body &b)
         return 3 + on_the_fly_launches(b.p) + (b.tp ? 3 : 0);
     if (b.aug) return 4;
     const bool lb = long_band(b.n);
-    int64_t k = 3 + (lb ? 3 : 1);
+    int64_t op = 1;   // launches of the operator
+    if (lb) op = 3;
+    else if (b.precision == FURAX_F64 && b.p->mode == FURAX_POINTING_ON_THE_FLY && b.n->kind == FURAX_NOISE_BANDED && b.p->n_tiles)
+        op = (b.p->n_tiles + kept_tiles(b.p) - 1) / kept_tiles(b.p);
+    int64_t k = 3 + op;
     if (b.tp) k += (!lb && b.precision != FURAX_F64 && tpl_fused_target(b.tp, b.p)) ? 2 : 3;
     return k;
 }

@@ -63,7 +63,9 @@ __device__ __forceinline__ void tc_fill_tod(double (&v)[kTcPer], const TcSlots &
 
 // v[k] = (P x)_t, or d_t - (P x)_t with RESID, of this thread's slots. Cached pointing: every pixel index is
 // loaded first, then weights, data and map records a few samples at a time (registers). On the fly: one
-// sample at a time (the FP64 recipe is too long to unroll), through shared memory.
+// sample at a time (the FP64 recipe is too long to unroll), through shared memory; the recipe's results of the tile's own
+// samples are kept for the scatter in this CTA's block of pv.pix, c64, s64 (tc_each<kTcKept>), which stay in L2
+// until then.
 template <int MODE, bool RESID, typename DT>
 __device__ __forceinline__ void tc_fill_map(unsigned char *sm, double (&v)[kTcPer], const TcSlots &sl, const PointingView &pv,
                                             const ObsInfo &ob, const Tile &tl, const DetOffset &psi,
@@ -77,6 +79,13 @@ __device__ __forceinline__ void tc_fill_map(unsigned char *sm, double (&v)[kTcPe
             if (sl.in(k)) {
                 double c, s;
                 const int32_t pix = get_sample<0, double>(pv, ob, tl.det, tl.t0 - kHalo + sl.slot(k), c, s);
+                const int t = sl.slot(k) - kHalo;
+                if (t >= 0 && t < tl.len) {
+                    const int64_t i = (int64_t)blockIdx.x * TILE + t;
+                    __stcg(const_cast<int32_t *>(pv.pix) + i, pix);
+                    __stcg(const_cast<double *>(pv.c64) + i, c);
+                    __stcg(const_cast<double *>(pv.s64) + i, s);
+                }
                 TcPix m;
                 m.load(x, ob.map_off + max(pix, 0));
                 r = m.project(pix, c, s);
@@ -124,6 +133,9 @@ static_assert(sizeof(double) * kTcPer * TT <= kTcOffCtl - kTcOffX, "the on-the-f
 // Core samples of the tile in time order, 32 consecutive ones per warp: f(k, pix, c, s, more(k, pix)) for every
 // lane of a warp together (pix = -1 past the tile or without a pixel). Cached pointing: the loads of B samples per
 // thread (of NT), and what `more` loads for them (k clamped into the tile), are issued before the first is used.
+// kTcKept: as left by tc_fill_map<0> of the same CTA, offsets applied.
+constexpr int kTcKept = 4;
+
 template <int MODE, int NT, int B, typename G, typename F>
 __device__ __forceinline__ void tc_each(const PointingView &pv, const ObsInfo &ob, const Tile &tl, const DetOffset &psi,
                                         G &&more, F &&f)
@@ -135,6 +147,15 @@ __device__ __forceinline__ void tc_each(const PointingView &pv, const ObsInfo &o
             double c = 0.0, s = 0.0;
             const int32_t pix = k < tl.len ? get_sample<0, double>(pv, ob, tl.det, tl.t0 + k, c, s) : -1;
             f(k, pix, c, s, more(min(k, tl.len - 1), pix));
+        }
+    } else if constexpr (MODE == kTcKept) {
+        const int64_t at = (int64_t)blockIdx.x * TILE;
+#pragma unroll 1
+        for (int k = threadIdx.x; k - (int)(threadIdx.x & 31) < tl.len; k += NT) {
+            const int64_t i = at + min(k, tl.len - 1);
+            const int32_t pix = __ldcg(pv.pix + i);
+            const double c = __ldcg(pv.c64 + i), s = __ldcg(pv.s64 + i);
+            f(k, k < tl.len ? pix : -1, c, s, more(min(k, tl.len - 1), pix));
         }
     } else {
 #pragma unroll 1
@@ -162,5 +183,22 @@ __device__ __forceinline__ void tc_each(const PointingView &pv, const ObsInfo &o
 }
 
 struct TcNone {};
+
+// Launches f(tiles, number, view) for chunks of tiles whose FP64 pointing is kept in the on-the-fly workspace.
+template <typename F>
+furax_status each_kept_chunk(const furax_pointing *p, F &&f)
+{
+    furax_status rc = ensure_local_ws(p);
+    PointingView pv = p->view();
+    pv.pix = p->ws_local_pix;
+    pv.c64 = reinterpret_cast<const double *>(p->ws_local_c);
+    pv.s64 = reinterpret_cast<const double *>(p->ws_local_s);
+    const int64_t c = kept_tiles(p);
+    for (int64_t t = 0; !rc && t < p->n_tiles; t += c) {
+        rc = f((const Tile *)p->d_tiles + t, (unsigned)std::min(c, p->n_tiles - t), pv);
+        if (t > 0) count_launches(1);   // the caller counts one
+    }
+    return rc;
+}
 
 }  // namespace fx
