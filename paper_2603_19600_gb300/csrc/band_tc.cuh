@@ -199,6 +199,8 @@ __device__ __forceinline__ void tc_put2(unsigned char *p, uint32_t w, uint32_t s
     *reinterpret_cast<__half *>(p + 2 * kTcPitch) = __high2half(h);
 }
 
+constexpr int kTcChainTaps = 16;   // bands up to this long take the chain in either precision
+
 // The FP64 FMA chain over the skewed samples xs, taps from global memory, y over the samples: tiles the
 // digits do not take.
 // With finite samples the zeros past the band's last tap add nothing and are skipped.
@@ -434,7 +436,9 @@ __device__ __forceinline__ void tc_band(unsigned char *sm, const double (&v)[kTc
         asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
         __syncthreads();
     } else {
-        const bool dot2 = !f64 && emax > 1023 - 80 && emax < 1023 + 100;   // well inside FP32's range
+        // Dot2 well inside FP32's range, and for bands of which the chain's 2 ntaps - 1 FP64 FMAs cost more than its
+        // 127 x 10 FP32 operations (right-hand side of 2.1 M samples and 4 taps: 219 us with Dot2, 72 us with the chain)
+        const bool dot2 = !f64 && emax > 1023 - 80 && emax < 1023 + 100 && nv.ntaps > kTcChainTaps;
         double *xs = tc_ys(sm);
         float *xh = reinterpret_cast<float *>(xs);
 #pragma unroll

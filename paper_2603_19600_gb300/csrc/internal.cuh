@@ -221,10 +221,14 @@ struct furax_pointing {
 
 namespace fx {
 // Four blocks per tile below two tiles per SM, one above (block-Jacobi blocks of 4 x 65,536 samples: 25 us on
-// 64 blocks, 20 us on 256; with more tiles than that the SMs are full either way).
+// 64 blocks, 20 us on 256; with more tiles than that the SMs are full either way), if the tiles are mostly long:
+// quarters of 1000-sample tiles would be three empty blocks beside a full one, which lands on the SMs unevenly (P on the
+// fly of 300 x 1000 samples: 152 us, 105 us on whole tiles; quarters of the own length: 35 us instead of 29 us for a
+// white FP64 operator, whose threads take four samples at a time).
 inline dim3 tile_grid(const furax_pointing *p)
 {
-    return dim3((unsigned)p->n_tiles, p->n_tiles < 2LL * p->n_sm ? 4u : 1u);
+    const bool split = p->n_tiles < 2LL * p->n_sm && p->nsamp_total > p->n_tiles * (TILE / 2);
+    return dim3((unsigned)p->n_tiles, split ? 4u : 1u);
 }
 }  // namespace fx
 

@@ -119,10 +119,11 @@ __global__ void __launch_bounds__(256) P_kernel(const Tile *__restrict__ tiles, 
     const Tile tl = tile_part(tiles[blockIdx.x]);
     const ObsInfo ob = pv.obs[tl.obs];
     const int64_t row = ob.tod_off + (int64_t)tl.det * ob.nsamp + tl.t0;
-    if constexpr (MODE != 0 && sizeof(T) == 8) {
+    if constexpr ((MODE == 1 || MODE == 2) && sizeof(T) == 8) {
         // FP64 from a cache: four samples per thread, each stage's loads in flight together (widening is
         // branch-free): 12.6 M samples at nside 256 99 -> 85 us, 148 G random gathers/s of the 166 G/s that
-        // furax_probe_l2 measures (padding the map to one 32-byte load per sample: 87 us; eight samples: 102 us)
+        // furax_probe_l2 measures (padding the map to one 32-byte load per sample: 87 us; eight samples: 102 us). The
+        // mixed cache's four words per weight pair leave too few registers for that: 43 us of 2.1 M samples against 27.
         constexpr int B = 4;
         const DetOffset psi(pv, ob.det_off + tl.det);
         for (int k0 = threadIdx.x; k0 < tl.len; k0 += 256 * B) {

@@ -95,3 +95,28 @@ def test_solution_does_not_depend_on_the_pixel_tiles(fx, dev, precision):
         assert info.converged
         maps.append(m[:small.npix].clone())
     assert float((maps[0] - maps[1]).norm()) <= 2e-6 * float(maps[0].norm())
+
+
+@pytest.mark.parametrize("ntaps", [4, 16, 17, 64])
+def test_short_bands_agree_in_either_precision(fx, dev, ntaps):
+    """Bands on both sides of the rules that choose among digits, FMA chain and compensated product, to the 1e-12
+    that the FP64-accurate paths are held to elsewhere."""
+    P, N, x, d = _problem(fx, dev, "cache_mixed", ntaps=ntaps)
+    f64 = fx.ptnp_apply(P, N, x, precision="f64")
+    assert float((fx.ptnp_apply(P, N, x, precision="f32x2") - f64).norm()) <= 1e-12 * float(f64.norm())
+    ref = P.transpose(N.inv_apply(d))
+    assert float((fx.rhs(P, N, d) - ref).norm()) <= 1e-12 * float(ref.norm())
+
+
+@pytest.mark.parametrize("per_sm,ns", [(17, 150), (0, 9001)])
+def test_on_the_fly_fp64_pointing_is_kept_for_the_scatter(fx, dev, per_sm, ns):
+    """Several chunks (16 tiles per SM), and tiles of full length with both halos."""
+    nd = per_sm * torch.cuda.get_device_properties(dev).multi_processor_count + 3
+    P, N, x, d = _problem(fx, dev, "on_the_fly", nd=nd, ns=ns)
+    C, M, _, _ = _problem(fx, dev, "cache_f64", nd=nd, ns=ns)
+    tol = _reorder_bound(C, 1.01 * M.inv_apply(C.apply(x)))
+    got, ref = (fx.ptnp_apply(p, n, x, precision="f64") for p, n in ((P, N), (C, M)))
+    assert float((got - ref).abs().max()) <= tol
+    got, ref = (fx.chi2_grad(p, n, d, x) for p, n in ((P, N), (C, M)))
+    tol = 2 * _reorder_bound(C, 1.01 * M.inv_apply(d - C.apply(x)))
+    assert float((got[1] - ref[1]).abs().max()) <= tol
