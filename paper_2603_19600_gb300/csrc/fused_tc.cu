@@ -12,8 +12,8 @@
 // Each CTA has 512 threads at 64 registers: with 256 at 128 the same phases took 5,000 / 26,000, 4,000, 9,000 and
 // 6,000-10,000 cycles and the scatter 33,000 instead of 23,000. Measured (GB300): FP64 FMAs (double-FP32 for the
 // right-hand side), 256 threads, now:
-//   normal operator, 32 x 262,147 samples, nside 256, FP64 cache   2277, 329, 290 us
-//   right-hand side, 128 x 524,288 FP32 samples, mixed cache       3440, 1730, 1419 us
+//   normal operator, 32 x 262,147 samples, nside 256, FP64 cache   2277, 329, 277 us
+//   right-hand side, 128 x 524,288 FP32 samples, mixed cache       3440, 1730, 1387 us
 //   N^-1 alone, 32 x 131,071 samples                               1011, 61, 58 us
 #include "tc_sample.cuh"
 #include "tpl_eval.cuh"
