@@ -587,7 +587,6 @@ static furax_status get_ws(furax_pointing *p, int hist_cap, CgWs **out)
     if (!rc) rc = alloc((void **)&w->partial, sizeof(double) * KD * (size_t)nparts);
     if (!rc) rc = alloc((void **)&w->sc, sizeof(CgScalars) * p->n_obs);
     if (!rc) rc = alloc((void **)&w->count, sizeof(unsigned) * (p->n_obs + 1));
-    if (!rc) rc = check_cuda(cudaMemset(w->count, 0, sizeof(unsigned) * (p->n_obs + 1)), "memset");
     if (!rc) rc = alloc((void **)&w->norms, sizeof(double) * 2 * p->n_obs);
     w->hist_cap = std::max(hist_cap, 1);
     if (!rc) rc = alloc((void **)&w->hist, sizeof(double) * w->hist_cap);
@@ -829,6 +828,8 @@ furax_status mapmaker_cg(const furax_pointing *p, const furax_noise *n, const vo
     CgWs *w = nullptr;
     furax_status rc;
     if ((rc = get_ws(pm, o->maxiter + 1, &w))) return rc;
+    // on the solve's own stream: nothing orders the legacy default stream with it
+    if ((rc = check_cuda(cudaMemsetAsync(w->count, 0, sizeof(unsigned) * (p->n_obs + 1), st), "memset"))) return rc;
     const int64_t np = p->npix_total;
     if ((rc = ensure_ws(pm, (void **)&pm->ws_x4, sizeof(double4_32a) * (size_t)np))) return rc;   // written by cg_init
     const unsigned pg = (unsigned)std::max<int64_t>(1, p->n_ptiles);
