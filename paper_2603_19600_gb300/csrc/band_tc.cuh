@@ -59,7 +59,6 @@ constexpr int kTcDetBytes = kTcCDig * kTcCores * 128;   // per detector in globa
 constexpr int kTcOffX = kTcCDig * 2 * kTcRun;           // shared memory: taps, then sample digits
 constexpr int kTcOffCtl = kTcOffX + kTcXDig * 2 * kTcPitch;
 constexpr int kTcRange = 6, kTcRangeDot2 = 8;           // log2 of the largest range taken (see above)
-constexpr int kTcRangeMasked = 20;                      // masked vectors: see tc_band
 constexpr int kTcNoTaps = -(1 << 20);                   // exponent of taps that have no digits
 constexpr int kTcMinTaps = 8;                           // shorter bands take the chain (see above)
 constexpr unsigned kTcTmemCols = 256;                   // 2 row blocks x 8 weights x 16 columns
@@ -354,8 +353,7 @@ static_assert((2 * XS + 4) % 4 == 0 && sizeof(float) * (2 * XS + 4) + (16 + 8) *
 // tc_begin; on return the results are visible to the CTA and no TMEM is held. Slots [in0, in1) lie in the
 // stream. f64: FP64 accuracy of every output (else that of the compensated product). MASKED: zero
 // samples are masked ones whose own outputs are not used (the vectors of gap filling): all-zero groups do not
-// count as quiet, and groups with few observed samples may be small by chance; a range of 2^20 keeps the
-// error of any output below 2^-36 of its neighbourhood and 2^-56 of the tile.
+// count as quiet.
 template <bool MASKED>
 __device__ __forceinline__ void tc_band(unsigned char *sm, const double (&v)[kTcPer], const NoiseView &nv, int64_t gdet,
                                         unsigned *err, bool f64, int in0, int in1)
@@ -377,7 +375,7 @@ __device__ __forceinline__ void tc_band(unsigned char *sm, const double (&v)[kTc
     for (int w = 0; w < TT / 32; ++w) { gmax = max(gmax, C.wmax[w]); gmin = min(gmin, C.wmin[w]); }
     const int emax = (int)(gmax >> 20), ec = nv.tc_exp[gdet];
     const int ey = emax - 1022 + ec - 69;   // y = (H 2^32 + L) 2^ey
-    const int range = MASKED ? kTcRangeMasked : f64 ? kTcRange : kTcRangeDot2;
+    const int range = f64 ? kTcRange : kTcRangeDot2;
     const bool digits = emax >= 123 && emax < 2047 && emax - (int)(gmin >> 20) <= range && ec > -900 && ec < 900 && ey > -900 && ey < 900;
     const uint32_t tmem = C.tmem;
     if (digits) {

@@ -132,7 +132,6 @@ __global__ void __launch_bounds__(FT) white_operator_kernel(const Tile *__restri
 }
 
 // out = N^-1 in on an FP64 TOD, banded.
-template <bool MASKED>
 __global__ void __launch_bounds__(TT, 2) tc_ninv_kernel(const Tile *__restrict__ tiles, const ObsInfo *__restrict__ obs,
                                                         NoiseView nv, const double *__restrict__ in,
                                                         double *__restrict__ out, unsigned *__restrict__ err, bool f64)
@@ -146,16 +145,16 @@ __global__ void __launch_bounds__(TT, 2) tc_ninv_kernel(const Tile *__restrict__
     double v[kTcPer];
     const TcSlots sl(tl, ob);
     tc_fill_tod(v, sl, in);
-    tc_band<MASKED>(sm, v, nv, gdet, err, f64, sl.in0, sl.in1);
+    tc_band<false>(sm, v, nv, gdet, err, f64, sl.in0, sl.in1);
     const double *ys = tc_ys(sm);
     for (int k = threadIdx.x; k < tl.len; k += TT) out[row + tl.t0 + k] = ys[spos(k)];
 }
 
-furax_status launch_ninv_tc(const furax_noise *n, const double *in, double *out, bool masked, bool f64, cudaStream_t st)
+furax_status launch_ninv_tc(const furax_noise *n, const double *in, double *out, bool f64, cudaStream_t st)
 {
     if (n->n_tiles == 0) return FURAX_OK;
-    furax_status rc = launch_dyn(masked ? tc_ninv_kernel<true> : tc_ninv_kernel<false>, (unsigned)n->n_tiles, TT, kTcSmem, st,
-                                 n->d_tiles, n->d_obs, n->view(), in, out, n->d_err, f64);
+    furax_status rc = launch_dyn(tc_ninv_kernel, (unsigned)n->n_tiles, TT, kTcSmem, st, n->d_tiles, n->d_obs, n->view(), in, out,
+                                 n->d_err, f64);
     if (rc) return rc;
     count_launches(1);
     return check_launch("N^-1 apply (FP64, banded)");
@@ -286,8 +285,7 @@ furax_status prepare_noise_tc(furax_noise *n, cudaStream_t st)
 {
     furax_status rc;
     const size_t nd = (size_t)n->ndet_total;
-    if ((rc = allow_smem((const void *)tc_ninv_kernel<false>, kTcSmem))) return rc;
-    if ((rc = allow_smem((const void *)tc_ninv_kernel<true>, kTcSmem))) return rc;
+    if ((rc = allow_smem((const void *)tc_ninv_kernel, kTcSmem))) return rc;
     tap_digits_kernel<<<(unsigned)nd, 128, 0, st>>>(n->p64, n->ntaps, n->tc_taps, n->tc_exp);
     count_launches(1);
     return check_launch("tap digits");

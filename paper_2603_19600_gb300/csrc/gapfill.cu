@@ -321,11 +321,10 @@ furax_status gapfill(const furax_noise *n, const void *d, const uint8_t *valid, 
                      int maxiter, double tol, int precision, int32_t *iters_out, cudaStream_t st)
 {
     const bool f32 = precision == FURAX_F32;   // band product in FP32, vectors and scalars in FP64
-    // N on masked vectors (zero in the gaps): short bands on the tensor cores, FURAX_PREC_F32X2 with the
+    // N y, of which the gaps' outputs are used: short bands on the tensor cores, FURAX_PREC_F32X2 with the
     // compensated product for tiles outside the digits' range
     auto ninv64 = [&](const double *in, double *o) {
-        return long_band(n) ? launch_ninv(n, in, o, FURAX_F64, st)
-                            : launch_ninv_tc(n, in, o, true, precision == FURAX_F64, st);
+        return long_band(n) ? launch_ninv(n, in, o, FURAX_F64, st) : launch_ninv_tc(n, in, o, precision == FURAX_F64, st);
     };
     const int64_t ns = n->nsamp_total, nd = n->ndet_total;
     if (ns == 0 || nd == 0) return FURAX_OK;

@@ -313,9 +313,8 @@ furax_status launch_bj(const furax_pointing *p, const furax_noise *n, double rco
 
 // ---- launchers (noise.cu)
 furax_status launch_ninv(const furax_noise *n, const void *in, void *out, int dtype, cudaStream_t st);
-// FP64 in, FP64 out, bands of up to MAXTAPS taps on the tensor cores (fused_tc.cu). masked: zero samples of
-// `in` are masked ones; f64 as below.
-furax_status launch_ninv_tc(const furax_noise *n, const double *in, double *out, bool masked, bool f64, cudaStream_t st);
+// FP64 in, FP64 out, bands of up to MAXTAPS taps on the tensor cores (fused_tc.cu); f64 as below.
+furax_status launch_ninv_tc(const furax_noise *n, const double *in, double *out, bool f64, cudaStream_t st);
 // Digits of the taps of a short band (fused_tc.cu).
 furax_status prepare_noise_tc(furax_noise *n, cudaStream_t st);
 size_t tc_taps_bytes(int64_t ndet);
