@@ -590,7 +590,7 @@ furax_status furax_noise_create(int32_t kind, const double *params, int32_t ntap
                  o_err = part(sizeof(unsigned) * kCtlWords),
                  o_band2 = part(short_band ? sizeof(float) * kBandPairs * 2 * (size_t)ndet : 0),
                  o_exp = part(short_band ? sizeof(int32_t) * (size_t)ndet : 0),
-                 o_taps = part(short_band ? tc_taps_bytes(ndet) : 0);
+                 o_w = part(short_band ? tc_weights_bytes(ndet) : 0), o_taps = part(short_band ? tc_taps_bytes(ndet) : 0);
     if (cudaMalloc((void **)&n->slab, bytes) != cudaSuccess) {
         cudaGetLastError();
         delete n;
@@ -605,6 +605,7 @@ furax_status furax_noise_create(int32_t kind, const double *params, int32_t ntap
     if (short_band) {
         n->band2 = (float *)(n->slab + o_band2);
         n->tc_exp = (int32_t *)(n->slab + o_exp);
+        n->tc_w = (float *)(n->slab + o_w);
         n->tc_taps = n->slab + o_taps;
     }
     if (cudaMemcpyAsync(n->d_obs, L.obs.data(), sizeof(ObsInfo) * L.obs.size(), cudaMemcpyHostToDevice,

@@ -7,16 +7,12 @@
 // rate, so it is computed without rounding (Ozaki, Ogita, Oishi & Rump 2012, error-free splitting;
 // integer digits in FP16 with FP32 accumulators):
 //   * the tile's samples become 62-bit integers relative to the tile's largest magnitude, and those
-//     eight balanced base-256 digits (values in [-128, 128], exact in FP16); the taps, once per noise
-//     handle, 55-bit integers relative to the largest tap and seven digits;
+//     eight balanced base-256 digits (values in [-128, 127], exact in FP16); the taps, once per noise
+//     handle, 63-bit integers relative to the largest tap and eight digits;
 //   * y is a sum over digit pairs (i, j) of weight 256^-(i+j); all pairs of one weight d = i + j share
-//     one FP32 accumulator per output: at most 7 pairs x 127 taps x 2^14 < 2^24, so every partial sum
-//     is an integer that FP32 holds exactly, in any order. Weights d <= 7 are kept (35 pairs);
+//     one FP32 accumulator per output: at most 8 pairs x 127 taps x 2^14 < 2^24, so every partial sum
+//     is an integer that FP32 holds exactly, in any order. Weights d <= 7 are kept (36 pairs);
 //   * the eight accumulators are combined as an 82-bit integer and rounded to FP64 once.
-// Error: the dropped weights d >= 8 are ~2^-57 and the taps' rounding ~2^-52.6 of a typical output, and
-// the samples are kept to 2^-62 of the tile's maximum. Measured against extended precision (Gaussian
-// samples, the 1/f band): N^-1 1.5e-16 relative where the FP64 FMA chain is at 3.8e-16; the normal operator
-// 1.3e-16 - 2.2e-16 (chain 1.7e-16 - 2.9e-16, double-FP32 1.3e-14 - 3.9e-14).
 //
 // As a matrix product: D[m][n] = sum_k A[m][k] B[n][k], row m = outputs 16 m .. 16 m + 15, A[m][k] =
 // digit of x[16 m + k] (k < 144: 16 outputs + 126 halo, padded), B[n][k] = digit of c_|k - n - 63|. Both
@@ -30,13 +26,21 @@
 // x multiplies the digits 0 .. min(6, 7 - i) of c in one instruction: their columns stand side by side
 // (16 per digit), and so do the accumulators of the weights i, i + 1, ... in TMEM.
 //
-// Integers relative to the tile's maximum do not resolve outputs that are far smaller than it. Tiles that
-// hold such outputs take a floating-point product instead, decided per tile inside the kernel: the FP64
-// FMA chain, or, where the caller asked for no more, the compensated double-FP32 dot product. These are
-// tiles where a 32-sample group of the stream is zero or more than 2^6 (2^8) below the tile's maximum (up to
-// there the digits' error stays below that of the product they replace, relative to the quiet samples),
-// tiles with infinities, NaNs or extreme exponents, and all tiles of bands with fewer than 8 taps or almost
-// without weight off the diagonal, where an output can be as small as one sample.
+// Error: with X and C the powers of two above the tile's largest sample and the detector's largest tap, an
+// output is off by the dropped weights d >= 8, at most 2^-53.2 X C and in practice 2^-59.7 X C (rms; they are sums
+// of some 700 digit products of either sign), and by its one rounding. Small beside |c| * |x|, the scale of an FP64 FMA
+// chain's error, only where the band reaches samples that are not too far below X. So every block of 8
+// outputs is checked: sums of |x| over blocks of 8 samples, weighted with the smallest |tap| that joins the
+// two blocks, bound |c| * |x| of its outputs from below (within a factor of 2 for the 1/f band), and blocks for
+// which that is under 2^-kTcRange X C are formed again by the FP64 FMA chain, a warp per block. Up to there the
+// digits' error is at most 6 u |c| * |x| in emulation (u = 2^-53; rms 0.3 u on Gaussian samples), that of the chain up to 13 u
+// (rms 2 u). An output whose band holds only zeros is exact in digits too. Where the caller asked for no more
+// than the compensated double-FP32 product, the line is kTcRangeDot2, and many blocks take that product.
+// A few loud samples (glitches, a planet, infinities and NaNs) are left out of the digits, and every block whose band
+// reaches one is formed again (tc_band). Tiles with extreme exponents, tiles mostly below the line, and bands whose
+// small or missing taps would send ordinary noise to the chain (tap_digits_kernel) form every block that way.
+// Measured (FP64 data, 32 x 131,071 samples, N^-1 alone, all tiles alike): 65 us in digits (58 without sums and check), 126 us
+// with a glitch per tile (895 with the chain for the whole tile), 524 us with half of each tile 2^16 louder.
 #pragma once
 #include <cuda_fp16.h>
 #include "tile.cuh"
@@ -44,7 +48,7 @@
 
 namespace fx {
 
-constexpr int kTcXDig = 8, kTcCDig = 7;                 // digits of the samples and of the taps
+constexpr int kTcXDig = 8, kTcCDig = 8;                 // digits of the samples and of the taps
 constexpr int kTcDiag = 8;                              // weights kept
 constexpr int kTcOut = 16;                              // outputs per row (columns per weight)
 constexpr int kTcSteps = 9;                             // K = 144 in steps of 16
@@ -58,20 +62,36 @@ constexpr int kTcCores = 19;                            // distinct core matrice
 constexpr int kTcDetBytes = kTcCDig * kTcCores * 128;   // per detector in global memory
 constexpr int kTcOffX = kTcCDig * 2 * kTcRun;           // shared memory: taps, then sample digits
 constexpr int kTcOffCtl = kTcOffX + kTcXDig * 2 * kTcPitch;
-constexpr int kTcRange = 6, kTcRangeDot2 = 8;           // log2 of the largest range taken (see above)
-constexpr int kTcNoTaps = -(1 << 20);                   // exponent of taps that have no digits
-constexpr int kTcMinTaps = 8;                           // shorter bands take the chain (see above)
+constexpr int kTcRange = 9, kTcRangeDot2 = 12;          // -log2 of the smallest |c| * |x| / (X C) taken (see above)
+constexpr int kTcNoTaps = -(1 << 20);                   // "exponent" of taps that are not used in digits,
+constexpr int kTcBadTaps = -(1 << 21);                  // of taps that are not finite
+constexpr int kTcBlocks = kTcSlots / 8;                 // blocks of 8 samples
+constexpr int kTcReach = 17;                            // blocks that the band joins to a block of 8 outputs
+constexpr int kTcWeights = 16;                          // floats per detector: weights of the first 16 (the last is 0)
+constexpr int kTcSumRows = 64 + kTcReach - 1;
+constexpr uint32_t kTcOut28 = 1u << 28;                 // marks a sample above the cut in a sum of 25-bit magnitudes
+constexpr int kTcChainTaps = 16;                        // bands up to this long take the chain in either precision
+constexpr int kTcLoud = 12;                             // groups of 32 samples that may lie above the cut
 constexpr unsigned kTcTmemCols = 256;                   // 2 row blocks x 8 weights x 16 columns
 static_assert(TT == 512 && TR == 8 && kTcOut == 2 * TR, "each of 16 warps owns half of 32 rows");
 static_assert(kTcOffX % 128 == 0 && kTcPitch % 16 == 0 && kTcRun % 16 == 0, "16-byte units");
-static_assert(7 * 127 * 128 * 128 < (1 << 24), "accumulators must stay exact in FP32");
+static_assert(kTcDiag * 127 * 128 * 128 < (1 << 24), "accumulators must stay exact in FP32");
+static_assert(kTcDiag == kTcCDig, "the first digit's instruction writes every weight");
+static_assert(TILE / 8 == TT, "one block of outputs per thread");
+static_assert(sizeof(double) * XS <= kTcOffX, "the taps' region also holds the samples afterwards");
 static_assert(sizeof(double) * XS + (sizeof(double) * 96 + 128) * (TT / 32) <= kTcOffCtl - kTcOffX,
               "the samples' region also holds y and the record staging afterwards");
 
 struct TcCtl {
     uint64_t taps_full, mma_done;
     uint32_t tmem;
-    unsigned wmax[TT / 32], wmin[TT / 32];
+    unsigned nlist;
+    unsigned gmax[kTcPer * (TT / 32)];   // largest |x| (high word) of each 32 samples
+    __align__(16) float w[kTcWeights];   // the detector's weights
+    union {
+        float sum[kTcSumRows][9];        // sum of |x| over 8 samples (tc_put_sum)
+        uint16_t list[TILE / 8];         // blocks of outputs that are formed again
+    };
 };
 constexpr size_t kTcSmem = kTcOffCtl + sizeof(TcCtl);
 // Two CTAs per SM (one loads and scatters while the other multiplies) and no more: each holds half of TMEM.
@@ -95,7 +115,9 @@ __device__ __forceinline__ void tc_begin(unsigned char *sm, const NoiseView &nv,
                      : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
     }
+    if (threadIdx.x < kTcWeights) C.w[threadIdx.x] = __ldg(nv.tc_w + gdet * kTcWeights + threadIdx.x);
     if (threadIdx.x == 0) {
+        C.nlist = 0u;
         mbar_init(&C.taps_full, 1);
         mbar_init(&C.mma_done, 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -141,13 +163,7 @@ __device__ __forceinline__ void tc_issue(unsigned char *sm, uint32_t tmem)
 #pragma unroll
             for (int i = 0; i < kTcXDig; ++i) {
                 const uint64_t a = tc_desc(x0 + 2 * i * kTcPitch + 16 * (128 * mt + q), kTcPitch, 128);
-                const int nj = i == 0 ? kTcCDig : kTcDiag - i;
-                if (i == 1 && q == 0) {   // weight 7 starts here: the others add to what digit 0 wrote
-                    tc_mma(d + 16, a, b, 6, true);
-                    tc_mma(d + 112, a, tc_desc(t0 + 12 * kTcRun, 128, kTcRun), 1, false);
-                } else {
-                    tc_mma(d + 16 * i, a, b, nj, !(q == 0 && i == 0));
-                }
+                tc_mma(d + 16 * i, a, b, kTcDiag - i, !(q == 0 && i == 0));
             }
         }
     }
@@ -196,30 +212,6 @@ __device__ __forceinline__ void tc_put2(unsigned char *p, uint32_t w, uint32_t s
     const __half2 h = __hsub2(*reinterpret_cast<const __half2 *>(&r), __half2half2(__ushort_as_half(0x6480)));
     *reinterpret_cast<__half *>(p) = __low2half(h);
     *reinterpret_cast<__half *>(p + 2 * kTcPitch) = __high2half(h);
-}
-
-constexpr int kTcChainTaps = 16;   // bands up to this long take the chain in either precision
-
-// The FP64 FMA chain over the skewed samples xs, taps from global memory, y over the samples: tiles the
-// digits do not take.
-// With finite samples the zeros past the band's last tap add nothing and are skipped.
-static __device__ __noinline__ void tc_chain(double *xs, const double *__restrict__ c, int ntaps, bool finite)
-{
-    const int base = threadIdx.x * TR;
-    double y[TR];
-#pragma unroll
-    for (int r = 0; r < TR; ++r) y[r] = 0.0;
-    const int skip = finite ? kHalo + 1 - ntaps : 0;
-#pragma unroll 1
-    for (int j = skip; j < kBand - skip; ++j) {
-        const int k = j < kHalo ? kHalo - j : j - kHalo;
-        const double t = k < ntaps ? c[k] : 0.0;
-#pragma unroll
-        for (int r = 0; r < TR; ++r) y[r] = fma(t, xs[spos(base + r + j)], y[r]);
-    }
-    __syncthreads();
-#pragma unroll
-    for (int r = 0; r < TR; ++r) xs[spos(base + r)] = y[r];
 }
 
 // Compensated dot product in double-FP32 on output pairs (y_i, y_{i+4}) (Ogita, Rump & Oishi 2005,
@@ -322,13 +314,51 @@ __device__ __forceinline__ void band_product_dfx2(const float *__restrict__ xs, 
     }
 }
 
-// The compensated product over the samples in the digits' region (high words, then low words, skewed),
-// y over them in FP64.
-static __device__ __noinline__ void tc_dot2(float *xh, const double *__restrict__ c, int ntaps)
+// Outputs of the n blocks in C.list again, from the samples in the taps' region (skewed; see tc_put_samples).
+
+// FP64 FMA chain. Few blocks: a warp each, four lanes to the band of an output (2,000 cycles where a thread per block
+// takes 20,000). Many: a thread each, whose eight outputs share the loads (normal operator with 4 taps: 178 us, with warps 316).
+static __device__ __noinline__ void tc_redo_chain(unsigned char *sm, int n, const double *__restrict__ c, int ntaps)
 {
-    float *xl = xh + XS + 1;
-    float4 *C4 = reinterpret_cast<float4 *>(xh + 2 * XS + 4);
-    float2 *CL2 = reinterpret_cast<float2 *>(C4 + kBandPad);
+    const TcCtl &C = *reinterpret_cast<const TcCtl *>(sm + kTcOffCtl);
+    const double *xs = reinterpret_cast<const double *>(sm);
+    const int lane = threadIdx.x & 31, part = lane & 3, skip = kHalo + 1 - ntaps;
+    if (n > TT / 4) {
+        if ((int)threadIdx.x >= n) return;
+        const int base = 8 * (int)C.list[threadIdx.x];
+        double y[TR];
+#pragma unroll
+        for (int r = 0; r < TR; ++r) y[r] = 0.0;
+#pragma unroll 1
+        for (int j = skip; j < kBand - skip; ++j) {
+            const double t = __ldg(c + (j < kHalo ? kHalo - j : j - kHalo));
+#pragma unroll
+            for (int r = 0; r < TR; ++r) y[r] = fma(t, xs[spos(base + r + j)], y[r]);
+        }
+#pragma unroll
+        for (int r = 0; r < TR; ++r) tc_ys(sm)[spos(base + r)] = y[r];
+        return;
+    }
+#pragma unroll 1
+    for (int i = threadIdx.x >> 5; i < n; i += TT / 32) {
+        const int t = 8 * (int)C.list[i] + (lane >> 2);
+        double y = 0.0;
+#pragma unroll 4
+        for (int j = skip + part; j < kBand - skip; j += 4)
+            y = fma(__ldg(c + (j < kHalo ? kHalo - j : j - kHalo)), xs[spos(t + j)], y);
+        y += __shfl_xor_sync(0xffffffffu, y, 1);
+        y += __shfl_xor_sync(0xffffffffu, y, 2);
+        if (part == 0) tc_ys(sm)[spos(t)] = y;
+    }
+}
+
+// The compensated product, a thread per block.
+static __device__ __noinline__ void tc_redo_dot2(unsigned char *sm, int n, const double *__restrict__ c, int ntaps)
+{
+    const TcCtl &C = *reinterpret_cast<const TcCtl *>(sm + kTcOffCtl);
+    const float *xh = reinterpret_cast<const float *>(sm), *xl = xh + XS + 1;
+    float4 *C4 = reinterpret_cast<float4 *>(sm + kTcOffCtl) - kBandPad;   // behind y and the staging
+    float2 *CL2 = reinterpret_cast<float2 *>(C4) - kBandPad;
     if (threadIdx.x < kBandPad) {
         const int j = threadIdx.x, k = j < kHalo ? kHalo - j : j - kHalo;
         const double t = j < kBand && k < ntaps ? c[k] : 0.0;
@@ -337,58 +367,159 @@ static __device__ __noinline__ void tc_dot2(float *xh, const double *__restrict_
         CL2[j] = make_float2(l, l);
     }
     __syncthreads();
+    if ((int)threadIdx.x >= n) return;
     float S[TR], E[TR];
-    const int base = threadIdx.x * TR;
+    const int base = 8 * (int)C.list[threadIdx.x];
     band_product_dfx2<TR>(xh, xl, C4, CL2, base, S, E);
-    __syncthreads();
-    double *ys = reinterpret_cast<double *>(xh);
+    double *ys = tc_ys(sm);
 #pragma unroll
     for (int r = 0; r < TR; ++r) ys[spos(base + r)] = (double)S[r] + (double)E[r];
 }
-static_assert((2 * XS + 4) % 4 == 0 && sizeof(float) * (2 * XS + 4) + (16 + 8) * kBandPad <= kTcOffCtl - kTcOffX,
-              "the compensated product fits the samples' region");
+static_assert(TR == 8 && sizeof(float) * 2 * (XS + 1) <= kTcOffX && kTcOffCtl % 16 == 0 &&
+                  sizeof(double) * XS + (sizeof(double) * 96 + 128) * (TT / 32) + (16 + 8) * kBandPad <= kTcOffCtl - kTcOffX,
+              "samples in the taps' region, the compensated product's taps behind y and the staging");
 
-// tc_ys(sm)[spos(t)] = sum_k c_|k| x_{t+k} for the tile's outputs t. v[k]: the sample of slot u = threadIdx.x +
-// 512 k (slot 63 is the tile's first output; zero past the loaded samples). Every thread calls it after
-// tc_begin; on return the results are visible to the CTA and no TMEM is held. Slots [in0, in1) lie in the
-// stream. f64: FP64 accuracy of every output (else that of the compensated product). MASKED: zero
-// samples are masked ones whose own outputs are not used (the vectors of gap filling): all-zero groups do not
-// count as quiet.
-template <bool MASKED>
+// This thread's samples into the taps' region: FP64, or high and low words for the compensated product.
+__device__ __forceinline__ void tc_put_samples(unsigned char *sm, const double (&v)[kTcPer], bool dot2)
+{
+    float *xh = reinterpret_cast<float *>(sm);
+    double *xs = reinterpret_cast<double *>(sm);
+#pragma unroll
+    for (int k = 0; k < kTcPer; ++k) {
+        const int u = threadIdx.x + k * TT;
+        if (u < TILE + 2 * kHalo) {
+            if (dot2) {
+                const float h = (float)v[k];
+                xh[spos(u)] = h;
+                xh[XS + 1 + spos(u)] = (float)(v[k] - (double)h);
+            } else {
+                xs[spos(u)] = v[k];
+            }
+        }
+    }
+}
+
+// Sum over the 8 lanes of an aligned group of a[0] .. a[7]: lane l gets that of a[l & 7] (7 exchanges instead of 24).
+__device__ __forceinline__ uint32_t tc_sum8(const uint32_t (&a)[kTcPer])
+{
+    const int lane = threadIdx.x & 31;
+    uint32_t b[4], c[2];
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+        b[i] = (lane & 4 ? a[i + 4] : a[i]) + __shfl_xor_sync(0xffffffffu, lane & 4 ? a[i] : a[i + 4], 4);
+#pragma unroll
+    for (int i = 0; i < 2; ++i)
+        c[i] = (lane & 2 ? b[i + 2] : b[i]) + __shfl_xor_sync(0xffffffffu, lane & 2 ? b[i] : b[i + 2], 2);
+    return (lane & 1 ? c[1] : c[0]) + __shfl_xor_sync(0xffffffffu, lane & 1 ? c[0] : c[1], 1);
+}
+
+// Sum of block 64 k + at: row `at`, so that neither the writing lanes (four rows, eight k) nor the reading ones (a row each)
+// share a bank, and once more behind the last row, so that a block's successors are the rows that follow.
+__device__ __forceinline__ void tc_put_sum(TcCtl &C, int at, int k, uint32_t s)
+{
+    const float f = s >= kTcOut28 ? __int_as_float(0x7f800000) : (float)s;
+    C.sum[at][k] = f;
+    if (at < kTcReach - 1 && k > 0) C.sum[64 + at][k - 1] = f;
+}
+
+// True if the band may reach too little for block o of 8 outputs to keep its accuracy in digits (see above), or reaches
+// a sample above the cut.
+__device__ __forceinline__ bool tc_quiet(const TcCtl &C, int o, float line)
+{
+    const float *x = &C.sum[o & 63][o >> 6];
+    float s = 0.f, any = 0.f;
+#pragma unroll
+    for (int m = 0; m < kTcReach; ++m) {
+        any = fmaxf(any, x[9 * m]);
+        if (m < kTcWeights) s = fmaf(C.w[m], x[9 * m], s);
+    }
+    return any > 0.f && (s < line || any > 1e30f);
+}
+static_assert(TILE / 8 + kTcReach - 1 == kTcBlocks, "every sample of the band belongs to a block");
+
+struct TcKeep {   // for a caller that needs its samples afterwards
+    const double (&v)[kTcPer];
+    __device__ __forceinline__ void operator()(double (&w)[kTcPer]) const
+    {
+#pragma unroll
+        for (int k = 0; k < kTcPer; ++k) w[k] = v[k];
+    }
+};
+
+struct TcAll {   // every output is used
+    __device__ __forceinline__ bool operator()(int) const { return true; }
+};
+
+// tc_ys(sm)[spos(t)] = sum_k c_|k| x_{t+k} for the tile's len outputs t. v[k]: the sample of slot u = threadIdx.x +
+// 512 k (slot 63 is the tile's first output; zero outside the stream and past the loaded samples). Every thread
+// calls it after tc_begin; on return the results are visible to the CTA and no TMEM is held. f64: FP64 accuracy of
+// every output (else that of the compensated product). again(w): w = v once more, for outputs that are formed again
+// (to keep v in registers past the products cost N^-1 alone 109 -> 121 us of 8.4 M samples). used(t): false if outputs
+// t .. t + 7 are not used.
+template <class Again, class Used = TcAll>
 __device__ __forceinline__ void tc_band(unsigned char *sm, const double (&v)[kTcPer], const NoiseView &nv, int64_t gdet,
-                                        unsigned *err, bool f64, int in0, int in1)
+                                        unsigned *err, bool f64, int len, Again &&again, Used &&used = Used{})
 {
     TcCtl &C = *reinterpret_cast<TcCtl *>(sm + kTcOffCtl);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    // largest and smallest nonzero 32-sample group maximum (high words of |x| order like the values)
-    unsigned gmax = 0u, gmin = 0xffffffffu;
+    // largest magnitude of each 32 samples (high words of |x| order like the values)
 #pragma unroll
     for (int k = 0; k < kTcPer; ++k) {
         const unsigned m = __reduce_max_sync(0xffffffffu, (unsigned)__double2hiint(v[k]) & 0x7fffffffu);
-        gmax = max(gmax, m);
-        const int u0 = 32 * warp + k * TT;
-        if (MASKED ? m != 0u : u0 >= in0 && u0 + 32 <= in1) gmin = min(gmin, m);   // whole groups of the stream
+        if (lane == 0) C.gmax[k * (TT / 32) + warp] = m;
     }
-    if (lane == 0) { C.wmax[warp] = gmax; C.wmin[warp] = gmin; }
     __syncthreads();
+    const int range = f64 ? kTcRange : kTcRangeDot2, ec = nv.tc_exp[gdet];
+    constexpr int G = (kTcPer * (TT / 32) + 31) / 32;
+    unsigned g[G], gmax = 0u;
 #pragma unroll
-    for (int w = 0; w < TT / 32; ++w) { gmax = max(gmax, C.wmax[w]); gmin = min(gmin, C.wmin[w]); }
-    const int emax = (int)(gmax >> 20), ec = nv.tc_exp[gdet];
+    for (int i = 0; i < G; ++i) {
+        g[i] = lane + 32 * i < kTcPer * (TT / 32) ? C.gmax[lane + 32 * i] : 0u;
+        gmax = max(gmax, g[i]);
+    }
+    gmax = __reduce_max_sync(0xffffffffu, gmax);
+    auto groups = [&](auto &&f) {   // groups with f(their exponent)
+        int n = 0;
+#pragma unroll
+        for (int i = 0; i < G; ++i) n += __popc(__ballot_sync(0xffffffffu, g[i] != 0u && f((int)(g[i] >> 20))));
+        return n;
+    };
+    int emax = (int)(gmax >> 20);   // exponent of the largest sample in digits
+    bool digits = true;
+    // Much of the tile is far below its largest sample. If that is up to kTcLoud groups' doing (glitches, a planet, NaNs),
+    // these groups' loud samples stay out of the digits and all that the band joins to them is formed again. If the tile is
+    // below the line all the same, the products are not worth forming.
+    if (emax == 2047 || groups([&](int e) { return e + range - 5 < emax; }) > kTcLoud) {
+        int lo = 0, hi = 2047;   // smallest exponent with no more than kTcLoud groups above it
+        while (lo < hi) {
+            const int mid = (lo + hi) >> 1;
+            if (groups([&](int e) { return e > mid; }) <= kTcLoud) hi = mid;
+            else lo = mid + 1;
+        }
+        if (lo + 4 <= emax) emax = lo;
+        digits = groups([&](int e) { return e + range < emax; }) <= 100;
+    }
     const int ey = emax - 1022 + ec - 69;   // y = (H 2^32 + L) 2^ey
-    const int range = f64 ? kTcRange : kTcRangeDot2;
-    const bool digits = emax >= 123 && emax < 2047 && emax - (int)(gmin >> 20) <= range && ec > -900 && ec < 900 && ey > -900 && ey < 900;
+    digits = digits && emax >= 123 && emax < 2047 && ec > -900 && ec < 900 && ey > -900 && ey < 900;
+    // the compensated product, well inside FP32's range
+    const bool may_dot2 = !f64 && emax > 1023 - 80 && (int)(gmax >> 20) < 1023 + 100;
     const uint32_t tmem = C.tmem;
+    int nredo = 0;
     if (digits) {
         unsigned char *px = sm + kTcOffX;
+        const int top = (emax + 1) << 20;   // high words from here on stay out
+        uint32_t a[kTcPer];   // 2^25 |x| / X rounded down, at least 1 unless x is zero
 #pragma unroll
         for (int k = 0; k < kTcPer; ++k) {
             const int u = threadIdx.x + k * TT;
+            const uint32_t hi = (uint32_t)__double2hiint(v[k]), lo = (uint32_t)__double2loint(v[k]);
+            const int ah = (int)(hi & 0x7fffffffu);
+            // 62-bit integer x 2^(62 - ex) with |x| < 2^ex, then offset digits (byte = digit + 128)
+            const int e = ah >> 20;
+            uint64_t m = (((uint64_t)((hi & 0xfffffu) | (e ? 0x100000u : 0u)) << 32) | lo) << 9;
+            m = ah >= top ? 0ull : m >> min(emax - e, 63);
+            a[k] = ah >= top ? kTcOut28 : (uint32_t)(m >> 32) >> 5 | (uint32_t)((ah | lo) != 0);
             if (u < kTcSlots) {
-                // 62-bit integer x 2^(62 - ex) with |x| < 2^ex, then offset digits (byte = digit + 128)
-                const uint32_t hi = (uint32_t)__double2hiint(v[k]), lo = (uint32_t)__double2loint(v[k]);
-                const int e = (int)(hi >> 20) & 0x7ff;
-                uint64_t m = (((uint64_t)((hi & 0xfffffu) | (e ? 0x100000u : 0u)) << 32) | lo) << 9;
-                m >>= min(emax - e, 63);
                 const uint64_t w = ((int32_t)hi < 0 ? 0ull - m : m) + 0x8080808080808080ull;
                 unsigned char *p = px + ((u >> 3) & 1) * kTcPitch + (u >> 4) * 16 + (u & 7) * 2;
                 const uint32_t wh = (uint32_t)(w >> 32), wl = (uint32_t)w;
@@ -397,6 +528,15 @@ __device__ __forceinline__ void tc_band(unsigned char *sm, const double (&v)[kTc
                 tc_put2(p + 8 * kTcPitch, wl, 0x4243);
                 tc_put2(p + 12 * kTcPitch, wl, 0x4041);
             }
+        }
+        // sums over blocks: slot u = threadIdx.x + 512 k is of block 64 k + threadIdx.x / 8
+        static_assert(kTcPer == 9 && TT == 512, "eight samples at once, then the ninth");
+        const int at = threadIdx.x >> 3;
+        tc_put_sum(C, at, lane & 7, tc_sum8(a));
+        if (512 + at < kTcBlocks) {   // whole warps
+#pragma unroll
+            for (int o = 1; o < 8; o <<= 1) a[8] += __shfl_xor_sync(0xffffffffu, a[8], o);
+            if ((lane & 7) == 0) tc_put_sum(C, at, 8, a[8]);
         }
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // the digits, for the tensor core's reads
         __syncthreads();
@@ -409,8 +549,41 @@ __device__ __forceinline__ void tc_band(unsigned char *sm, const double (&v)[kTc
                          : "memory");
         }
         __syncwarp();
+        // while the products run: which blocks of outputs the digits do not resolve
+        const int t8 = 8 * threadIdx.x;
+        const bool redo = t8 < len && tc_quiet(C, threadIdx.x, ldexpf(1.f, 25 - range)) && used(t8);
+        nredo = __syncthreads_count(redo);
+        if (redo) C.list[atomicAdd(&C.nlist, 1u)] = (uint16_t)threadIdx.x;
         mbar_wait(&C.mma_done, 0, err, budget);
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    } else {
+        if (threadIdx.x == 0) mbar_wait(&C.taps_full, 0, err, wait_budget(err));   // their region is written over
+        C.list[threadIdx.x] = (uint16_t)threadIdx.x;
+        nredo = (len + 7) / 8;
+        bool zero = gmax == 0u && ec != kTcBadTaps;
+        if (zero) {   // no sample, no output
+            bool any = false;
+#pragma unroll
+            for (int k = 0; k < kTcPer; ++k) any = any || __double2loint(v[k]) != 0;
+            zero = !__syncthreads_or(any);
+        }
+        if (zero) {
+            nredo = 0;
+#pragma unroll
+            for (int r = 0; r < TR; ++r) tc_ys(sm)[spos(TR * threadIdx.x + r)] = 0.0;
+        }
+        __syncthreads();
+    }
+    // The chain takes 565 cycles a block with 64 taps, the compensated product, which walks 127 taps whatever their number,
+    // 15,000 for any few and 150 a block for many (normal operator with 8 taps: 282 us with the chain, 459 us).
+    const bool dot2 = may_dot2 && nredo > 32 && nv.ntaps > kTcChainTaps;
+    if (nredo) {
+        double w[kTcPer];
+        again(w);
+        tc_put_samples(sm, w, dot2);
+        __syncthreads();   // `again` may use the region of y
+    }
+    if (digits) {
         // warps 4 b .. 4 b + 3 hold the 128 rows of block b & 1, one lane each, and half b >> 1 of their columns
         const int half = warp >> 3, r0 = 128 * ((warp >> 2) & 1) + 32 * (warp & 3) + lane;
         const uint32_t at = tmem + ((uint32_t)(warp & 3) << 21) + 128u * ((warp >> 2) & 1) + 8u * half;
@@ -431,31 +604,13 @@ __device__ __forceinline__ void tc_band(unsigned char *sm, const double (&v)[kTc
                 ys[8 * (1 - half) + 4 * h + r] = tc_value(H, L, ey);
             }
         }
-        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-        __syncthreads();
-    } else {
-        // Dot2 well inside FP32's range, and for bands of which the chain's 2 ntaps - 1 FP64 FMAs cost more than its
-        // 127 x 10 FP32 operations (right-hand side of 2.1 M samples and 4 taps: 219 us with Dot2, 72 us with the chain)
-        const bool dot2 = !f64 && emax > 1023 - 80 && emax < 1023 + 100 && nv.ntaps > kTcChainTaps;
-        double *xs = tc_ys(sm);
-        float *xh = reinterpret_cast<float *>(xs);
-#pragma unroll
-        for (int k = 0; k < kTcPer; ++k) {
-            const int u = threadIdx.x + k * TT;
-            if (u < TILE + 2 * kHalo) {
-                if (dot2) {
-                    const float h = (float)v[k];
-                    xh[spos(u)] = h;
-                    xh[XS + 1 + spos(u)] = (float)(v[k] - (double)h);
-                } else {
-                    xs[spos(u)] = v[k];
-                }
-            }
-        }
-        if (threadIdx.x == 0) mbar_wait(&C.taps_full, 0, err, wait_budget(err));   // no copy in flight at exit
-        __syncthreads();
-        if (dot2) tc_dot2(xh, nv.p64 + gdet * nv.ntaps, nv.ntaps);
-        else tc_chain(xs, nv.p64 + gdet * nv.ntaps, nv.ntaps, emax < 2047);
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    if (nredo) {
+        const double *c = nv.p64 + gdet * nv.ntaps;
+        if (dot2) tc_redo_dot2(sm, nredo, c, nv.ntaps);
+        else tc_redo_chain(sm, nredo, c, nv.ntaps);
         __syncthreads();
     }
     if (warp == 0)

@@ -34,7 +34,7 @@ __global__ void __launch_bounds__(TT, 2) chi2_tc_kernel(const Tile *__restrict__
         double v[kTcPer];
         const TcSlots sl(tl, ob);
         tc_fill_map<MODE, true>(sm, v, sl, pv, ob, tl, psi, m, d);
-        tc_band<false>(sm, v, nv, gdet, err, f64, sl.in0, sl.in1);
+        tc_band(sm, v, nv, gdet, err, f64, tl.len, TcKeep{v});
         // r^T N^-1 r over this thread's own slots: r is still at hand
 #pragma unroll
         for (int k = 0; k < kTcPer; ++k) {

@@ -70,9 +70,12 @@ __global__ void __launch_bounds__(TT, 2) tc_operator_kernel(const Tile *__restri
     {
         double v[kTcPer];
         const TcSlots sl(tl, ob);
-        if constexpr (FROM_TOD) tc_fill_tod(v, sl, d);
-        else tc_fill_map<MODE, false>(sm, v, sl, pv, ob, tl, psi, x, d);
-        tc_band<false>(sm, v, nv, gdet, err, f64, sl.in0, sl.in1);
+        auto fill = [&](double (&w)[kTcPer]) {
+            if constexpr (FROM_TOD) tc_fill_tod(w, sl, d);
+            else tc_fill_map<MODE, false>(sm, w, sl, pv, ob, tl, psi, x, d);
+        };
+        fill(v);
+        tc_band(sm, v, nv, gdet, err, f64, tl.len, fill);
     }
     const double *ys = tc_ys(sm);
     double *rec = acc64 + 3 * ob.map_off;
@@ -145,7 +148,7 @@ __global__ void __launch_bounds__(TT, 2) tc_ninv_kernel(const Tile *__restrict__
     double v[kTcPer];
     const TcSlots sl(tl, ob);
     tc_fill_tod(v, sl, in);
-    tc_band<false>(sm, v, nv, gdet, err, f64, sl.in0, sl.in1);
+    tc_band(sm, v, nv, gdet, err, f64, tl.len, [&](double (&w)[kTcPer]) { tc_fill_tod(w, sl, in); });
     const double *ys = tc_ys(sm);
     for (int k = threadIdx.x; k < tl.len; k += TT) out[row + tl.t0 + k] = ys[spos(k)];
 }
@@ -246,47 +249,63 @@ furax_status launch_rhs_tc(const furax_pointing *p, const furax_noise *n, const 
                             : dispatch_tc<true, false, float>(p, n, nullptr, d32, a64, f64, TplView{}, nullptr, st);
 }
 
-// Digits of a detector's taps (one CTA each): integers relative to 2^ec, balanced base-256
+// Digits of a detector's taps (one CTA each): 63-bit integers relative to 2^ec, balanced base-256
 // digits, stored as the distinct core matrices of the operand (band_tc.cuh): [digit][matrix h][row r][column e]
 // is the tap of lag index 8 h - 8 + e - r (0 .. 126).
 __global__ void __launch_bounds__(128) tap_digits_kernel(const double *__restrict__ taps, int ntaps,
-                                                         unsigned char *__restrict__ out, int32_t *__restrict__ exps)
+                                                         unsigned char *__restrict__ out, int32_t *__restrict__ exps,
+                                                         float *__restrict__ weights)
 {
     __shared__ double c[MAXTAPS];
     const int64_t det = blockIdx.x;
     if (threadIdx.x < MAXTAPS) c[threadIdx.x] = threadIdx.x < ntaps ? taps[det * ntaps + threadIdx.x] : 0.0;
     __syncthreads();
-    double m = 0.0, off = 0.0;   // largest tap, weight off the diagonal
+    double m = 0.0;   // largest tap
     bool finite = true;
     for (int k = 0; k < MAXTAPS; ++k) {
         m = fmax(m, fabs(c[k]));
-        if (k > 0) off += 2.0 * fabs(c[k]);
         finite = finite && isfinite(c[k]);
     }
-    const bool ok = finite && ntaps >= kTcMinTaps && off >= m / 16 && m > 0.0;
-    // |c| 2^(55 - ec) <= 0x7f7f7f7f7f7f7f, the largest integer of seven balanced digits
+    bool ok = finite && m > 0.0;
+    // |c| 2^(63 - ec) <= 0x7f7f7f7f7f7f7f7f, the largest integer of eight balanced digits
     int ec = ok ? ilogb(m) + 1 : 0;
     if (scalbn(m, -ec) > 0.99) ++ec;
-    if (threadIdx.x == 0) exps[det] = ok ? ec : kTcNoTaps;
+    // Weight m: the smallest tap between sample block o + m and output block o (tap index 8 m - 7 .. 8 m + 7).
+    __shared__ float w[kTcWeights];
+    if (threadIdx.x < kTcWeights) {
+        double v = m;
+        for (int j = 8 * (int)threadIdx.x - 7; j <= 8 * (int)threadIdx.x + 7; ++j)
+            v = j < 0 || j >= kBand ? 0.0 : fmin(v, fabs(c[j < kHalo ? kHalo - j : j - kHalo]));
+        w[threadIdx.x] = ok ? (float)scalbn(v, -ec) : 0.f;
+        weights[det * kTcWeights + threadIdx.x] = w[threadIdx.x];
+    }
+    __syncthreads();
+    // Gaussian samples have sums of 6.4 sigma = 1.6 X where X = 4 sigma; twice that over the line on average leaves few
+    // blocks of ordinary noise below it.
+    float sum = 0.f;
+    for (int i = 0; i < kTcWeights; ++i) sum += w[i];
+    ok = ok && 1.6f * sum >= ldexpf(2.f, -kTcRange);
+    if (threadIdx.x == 0) exps[det] = ok ? ec : finite ? kTcNoTaps : kTcBadTaps;
     __half *o = reinterpret_cast<__half *>(out + det * kTcDetBytes);
     for (int i = threadIdx.x; i < kTcCores * 64; i += 128) {
         const int j = 8 * (i >> 6) - 8 + (i & 7) - ((i >> 3) & 7);
         const int lag = j < kHalo ? kHalo - j : j - kHalo;
-        const double v = ok && j >= 0 && j < kBand ? scalbn(c[lag], 55 - ec) : 0.0;
-        const uint64_t w = (uint64_t)__double2ll_rn(v) + 0x80808080808080ull;
+        const double v = ok && j >= 0 && j < kBand ? scalbn(c[lag], 63 - ec) : 0.0;
+        const uint64_t d = (uint64_t)__double2ll_rn(v) + 0x8080808080808080ull;
         for (int g = 0; g < kTcCDig; ++g)
-            o[g * kTcCores * 64 + i] = __int2half_rn((int)((w >> (8 * (kTcCDig - 1 - g))) & 0xff) - 128);
+            o[g * kTcCores * 64 + i] = __int2half_rn((int)((d >> (8 * (kTcCDig - 1 - g))) & 0xff) - 128);
     }
 }
 
 size_t tc_taps_bytes(int64_t ndet) { return (size_t)kTcDetBytes * (size_t)ndet; }
+size_t tc_weights_bytes(int64_t ndet) { return sizeof(float) * kTcWeights * (size_t)ndet; }
 
 furax_status prepare_noise_tc(furax_noise *n, cudaStream_t st)
 {
     furax_status rc;
     const size_t nd = (size_t)n->ndet_total;
     if ((rc = allow_smem((const void *)tc_ninv_kernel, kTcSmem))) return rc;
-    tap_digits_kernel<<<(unsigned)nd, 128, 0, st>>>(n->p64, n->ntaps, n->tc_taps, n->tc_exp);
+    tap_digits_kernel<<<(unsigned)nd, 128, 0, st>>>(n->p64, n->ntaps, n->tc_taps, n->tc_exp, n->tc_w);
     count_launches(1);
     return check_launch("tap digits");
 }

@@ -239,7 +239,12 @@ __global__ void __launch_bounds__(TT, 2) gf_apply_tc_kernel(const Tile *__restri
 #pragma unroll
     for (int k = 0; k < kTcPer; ++k)
         if (!sl.in(k)) v[k] = 0.0;
-    tc_band<true>(sm, v, nv, gdet, err, f64, sl.in0, sl.in1);
+    const int64_t row = sl.row + kHalo;
+    tc_band(sm, v, nv, gdet, err, f64, tl.len, TcKeep{v}, [&](int t) {   // outputs in gaps are not used
+        bool any = false;
+        for (int k = t; k < min(t + 8, tl.len); ++k) any = any || valid[row + k];
+        return any;
+    });
     const double *ys = tc_ys(sm);
     double acc = 0.0;
 #pragma unroll

@@ -95,6 +95,7 @@ struct NoiseView {
     const double *diag;     // diagonal of N^-1 per detector [ndet] (FP64)
     const unsigned char *tc_taps;  // banded (<= MAXTAPS taps): tap digits per detector (band_tc.cuh)
     const int32_t *tc_exp;         // [ndet] exponent of the tap digits
+    const float *tc_w;             // [ndet][kTcWeights] what the band joins blocks of samples with
     const float *band2;     // banded (<= MAXTAPS taps): [ndet][2 kBandPad] band in tap order as duplicated pairs
 };
 
@@ -279,8 +280,9 @@ struct furax_noise {
     float *band2 = nullptr;     // banded, <= MAXTAPS taps: [ndet][256] band in tap order as duplicated pairs
     unsigned char *tc_taps = nullptr;   // banded, <= MAXTAPS taps: digits of the taps for the tensor cores
     int32_t *tc_exp = nullptr;          // [ndet]
+    float *tc_w = nullptr;              // [ndet][kTcWeights]
     unsigned *d_err = nullptr;          // device control block (kCtlWords) of the kernels run on this handle alone
-    fx::NoiseView view() const { return fx::NoiseView{kind, ntaps, p64, p32, diag, tc_taps, tc_exp, band2}; }
+    fx::NoiseView view() const { return fx::NoiseView{kind, ntaps, p64, p32, diag, tc_taps, tc_exp, tc_w, band2}; }
 };
 
 namespace fx {
@@ -318,6 +320,7 @@ furax_status launch_ninv_tc(const furax_noise *n, const double *in, double *out,
 // Digits of the taps of a short band (fused_tc.cu).
 furax_status prepare_noise_tc(furax_noise *n, cudaStream_t st);
 size_t tc_taps_bytes(int64_t ndet);
+size_t tc_weights_bytes(int64_t ndet);
 // Bands longer than the fused kernels hold go through the TOD in HBM (overlap-save N^-1).
 inline bool long_band(const furax_noise *n) { return n->kind == FURAX_NOISE_BANDED && n->ntaps > MAXTAPS; }
 // noise_fft.cu: blocks, twiddles and spectra of a long band (synchronises st); the N^-1 apply.
