@@ -441,20 +441,31 @@ furax_status furax_chi2_grad(const furax_pointing_t *p, const furax_noise_t *n, 
  * furax_mapmaker_cg checks this itself at its synchronisation points. */
 furax_status furax_device_status(furax_pointing_t *p, void *stream);
 
+/* The same for the kernels that run on a noise handle alone: FURAX_ETIMEOUT once if a wait of furax_noise_inv_apply
+ * (FP64, short band) has given up since the last call, and the word is cleared. The outputs of a tile whose wait gave up
+ * are NaN. furax_gapfill reports its own waits itself and leaves this word alone. */
+furax_status furax_noise_status(furax_noise_t *n, void *stream);
+
 /* Budget of every bounded device-side wait of this handle's pipelined kernels (the mbarrier
- * hand-offs between the roles of the cached FP32 operator), in SM clock cycles; 0 restores the
+ * hand-offs between the roles of the cached FP32 operator, and between the copies, the tensor cores and the
+ * other threads of the FP64-accurate kernels), in SM clock cycles; 0 restores the
  * default of 2^32 cycles (about 2 s). A wait that runs out sets the error word that
  * furax_device_status reports (FURAX_ETIMEOUT) and its role leaves its loop, so the kernel
- * returns; the output of that launch is then incomplete. Ordered on `stream`; synchronises it.
+ * returns; the output of that launch is then incomplete. Tensor-core kernels wait once more as long for what is in
+ * flight. Ordered on `stream`; synchronises it.
  * Errors: FURAX_EINVAL for a NULL handle or a negative budget. The paper has no counterpart:
  * this is a property of the GPU pipeline. */
 furax_status furax_set_wait_budget(furax_pointing_t *p, int64_t cycles, void *stream);
+/* The same for the waits on a noise handle (furax_noise_inv_apply, furax_gapfill). */
+furax_status furax_noise_set_wait_budget(furax_noise_t *n, int64_t cycles, void *stream);
 
 /* Test hook for the bounded waits: with hold != 0 the loader role of the cached FP32 operator
- * issues no copies in this handle's later launches, so the other roles' waits run out after the
- * wait budget (no copy is ever left in flight). hold = 0 restores normal operation. Ordered on
+ * issues no copies, and the tensor-core kernels issue no products, in this handle's later launches, so the other
+ * waits run out after the wait budget (nothing is ever left in flight). hold = 0 restores normal operation. Ordered on
  * `stream`; synchronises it. The paper has no counterpart. */
 furax_status furax_debug_hold_loader(furax_pointing_t *p, int32_t hold, void *stream);
+/* The same for a noise handle (furax_noise_inv_apply, furax_gapfill). */
+furax_status furax_debug_hold_noise(furax_noise_t *n, int32_t hold, void *stream);
 
 /* ---------------------------------------------------------------------------------------
  * Device probes (measurement instruments; the paper has no counterpart). They give the

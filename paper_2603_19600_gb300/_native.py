@@ -96,7 +96,9 @@ _SIGS = {
     "furax_pointing_refresh": [_V, _V],
     "furax_pointing_cache": [_V, _V, _V, _V, _V],
     "furax_device_status": [_V, _V],
+    "furax_noise_status": [_V, _V],
     "furax_set_wait_budget": [_V, _I64, _V],
+    "furax_noise_set_wait_budget": [_V, _I64, _V],
     "furax_pointing_set_schedule": [_V, ctypes.POINTER(Schedule), _V],
     "furax_pointing_get_schedule": [_V, ctypes.POINTER(Schedule)],
     "furax_autotune": [_V, _V, _I32, ctypes.POINTER(Schedule), _I32, _I32, ctypes.POINTER(_D),
@@ -106,6 +108,7 @@ _SIGS = {
     "furax_probe_fma": [_I32, _I64, _V, ctypes.POINTER(_D), _V],
     "furax_probe_l2": [_I32, _V, _I64, _V, _I64, _V, _V],
     "furax_debug_hold_loader": [_V, _I32, _V],
+    "furax_debug_hold_noise": [_V, _I32, _V],
     "furax_pointing_set_psi_offset": [_V, _V, _V],
     "furax_profile_read": [_I32, ctypes.POINTER(_D), ctypes.POINTER(_I64)],
     "furax_pointing_expand": [_V, _V, _V, _V, _I32, _V],
@@ -258,6 +261,11 @@ def furax_device_status(h, stream=None) -> None:
     _call("furax_device_status", h, _stream(stream))
 
 
+def furax_noise_status(h, stream=None) -> None:
+    """The same for a noise handle (FP64 furax_noise_inv_apply)."""
+    _call("furax_noise_status", h, _stream(stream))
+
+
 def furax_pointing_set_schedule(h, kernel: int, tile_len: int = 0, max_rows: int = 12, group_tol: float = 2.0,
                                 l2_evict_first: int = 0, consumer_warps: int = 0, stream=None) -> None:
     sch = Schedule(int(kernel), int(tile_len), int(max_rows), float(group_tol), int(l2_evict_first),
@@ -297,9 +305,19 @@ def furax_set_wait_budget(h, cycles: int, stream=None) -> None:
     _call("furax_set_wait_budget", h, int(cycles), _stream(stream))
 
 
+def furax_noise_set_wait_budget(h, cycles: int, stream=None) -> None:
+    """The same for the waits on a noise handle."""
+    _call("furax_noise_set_wait_budget", h, int(cycles), _stream(stream))
+
+
 def furax_debug_hold_loader(h, hold: bool, stream=None) -> None:
     """Test hook: hold the cached FP32 operator's loader so that its other roles' waits run out."""
     _call("furax_debug_hold_loader", h, int(bool(hold)), _stream(stream))
+
+
+def furax_debug_hold_noise(h, hold: bool, stream=None) -> None:
+    """The same for a noise handle."""
+    _call("furax_debug_hold_noise", h, int(bool(hold)), _stream(stream))
 
 
 def furax_probe_convert(in64=None, out32=None, in32=None, out64=None, stream=None) -> None:

@@ -232,40 +232,73 @@ void furax_profile_reset(void)
     g_prof_cnt[0] = g_prof_cnt[1] = g_prof_cnt[2] = 0;
 }
 
-furax_status furax_device_status(furax_pointing_t *p, void *stream)
+// The control block of a handle (mbarrier.cuh). A kernel reads it at its start: writes are ordered on the stream like
+// a launch.
+static furax_status take_status(unsigned *ctl, cudaStream_t st)
 {
-    REQUIRE(p, "pointing handle is NULL");
-    cudaStream_t st = (cudaStream_t)stream;
     unsigned h = 0;
-    furax_status rc = check_cuda(cudaMemcpyAsync(&h, p->d_err, sizeof h, cudaMemcpyDeviceToHost, st), "read status");
+    furax_status rc = check_cuda(cudaMemcpyAsync(&h, ctl, sizeof h, cudaMemcpyDeviceToHost, st), "read status");
     if (!rc) rc = check_cuda(cudaStreamSynchronize(st), "status sync");
     if (rc) return rc;
     if (h) {
-        cudaMemsetAsync(p->d_err, 0, sizeof(unsigned), st);
+        cudaMemsetAsync(ctl, 0, sizeof(unsigned), st);
         cudaStreamSynchronize(st);
         return set_error(FURAX_ETIMEOUT, "a bounded device-side wait gave up (error word %u)", h);
     }
     return FURAX_OK;
 }
 
+static furax_status put_budget(unsigned *ctl, int64_t cycles, cudaStream_t st)
+{
+    REQUIRE(cycles >= 0, "the wait budget must be >= 0 cycles (0 selects the default)");
+    furax_status rc = check_cuda(cudaMemcpyAsync(ctl + 2, &cycles, sizeof cycles, cudaMemcpyHostToDevice, st),
+                                 "set wait budget");
+    return rc ? rc : check_cuda(cudaStreamSynchronize(st), "wait budget sync");
+}
+
+static furax_status put_hold(unsigned *ctl, int32_t hold, cudaStream_t st)
+{
+    const unsigned h = hold ? 1u : 0u;
+    furax_status rc = check_cuda(cudaMemcpyAsync(ctl + 1, &h, sizeof h, cudaMemcpyHostToDevice, st), "hold");
+    return rc ? rc : check_cuda(cudaStreamSynchronize(st), "hold sync");
+}
+
+furax_status furax_device_status(furax_pointing_t *p, void *stream)
+{
+    REQUIRE(p, "pointing handle is NULL");
+    return take_status(p->d_err, (cudaStream_t)stream);
+}
+
+furax_status furax_noise_status(furax_noise_t *n, void *stream)
+{
+    REQUIRE(n, "noise handle is NULL");
+    return take_status(n->d_err, (cudaStream_t)stream);
+}
+
 furax_status furax_set_wait_budget(furax_pointing_t *p, int64_t cycles, void *stream)
 {
     REQUIRE(p, "pointing handle is NULL");
-    REQUIRE(cycles >= 0, "the wait budget must be >= 0 cycles (0 selects the default)");
-    cudaStream_t st = (cudaStream_t)stream;
-    // a kernel reads the budget at its start: the write is ordered on the stream like a launch
-    furax_status rc = check_cuda(cudaMemcpyAsync(p->d_err + 2, &cycles, sizeof cycles, cudaMemcpyHostToDevice, st),
-                                 "set wait budget");
-    return rc ? rc : check_cuda(cudaStreamSynchronize(st), "wait budget sync");
+    return put_budget(p->d_err, cycles, (cudaStream_t)stream);
+}
+
+furax_status furax_noise_set_wait_budget(furax_noise_t *n, int64_t cycles, void *stream)
+{
+    REQUIRE(n, "noise handle is NULL");
+    furax_status rc = put_budget(n->d_err, cycles, (cudaStream_t)stream);
+    return rc ? rc : put_budget(n->gf_err(), cycles, (cudaStream_t)stream);
 }
 
 furax_status furax_debug_hold_loader(furax_pointing_t *p, int32_t hold, void *stream)
 {
     REQUIRE(p, "pointing handle is NULL");
-    cudaStream_t st = (cudaStream_t)stream;
-    const unsigned h = hold ? 1u : 0u;
-    furax_status rc = check_cuda(cudaMemcpyAsync(p->d_err + 1, &h, sizeof h, cudaMemcpyHostToDevice, st), "hold loader");
-    return rc ? rc : check_cuda(cudaStreamSynchronize(st), "hold loader sync");
+    return put_hold(p->d_err, hold, (cudaStream_t)stream);
+}
+
+furax_status furax_debug_hold_noise(furax_noise_t *n, int32_t hold, void *stream)
+{
+    REQUIRE(n, "noise handle is NULL");
+    furax_status rc = put_hold(n->d_err, hold, (cudaStream_t)stream);
+    return rc ? rc : put_hold(n->gf_err(), hold, (cudaStream_t)stream);
 }
 
 furax_status furax_pointing_cache(const furax_pointing_t *p, int32_t *pix, float *c, float *s, void *stream)
@@ -587,7 +620,7 @@ furax_status furax_noise_create(int32_t kind, const double *params, int32_t ntap
     auto part = [&](size_t b) { const size_t at = bytes; bytes += (b + 255) & ~size_t(255); return at; };
     const size_t o_obs = part(sizeof(ObsInfo) * L.obs.size()), o_tiles = part(sizeof(Tile) * L.tiles.size()),
                  o_p64 = part(sizeof(double) * cnt), o_diag = part(sizeof(double) * ndet), o_p32 = part(sizeof(float) * cnt),
-                 o_err = part(sizeof(unsigned) * kCtlWords),
+                 o_err = part(sizeof(unsigned) * 2 * kCtlWords),
                  o_band2 = part(short_band ? sizeof(float) * kBandPairs * 2 * (size_t)ndet : 0),
                  o_exp = part(short_band ? sizeof(int32_t) * (size_t)ndet : 0),
                  o_w = part(short_band ? tc_weights_bytes(ndet) : 0), o_taps = part(short_band ? tc_taps_bytes(ndet) : 0);
@@ -612,7 +645,7 @@ furax_status furax_noise_create(int32_t kind, const double *params, int32_t ntap
                         (cudaStream_t)stream) != cudaSuccess ||
         cudaMemcpyAsync(n->d_tiles, L.tiles.data(), sizeof(Tile) * L.tiles.size(), cudaMemcpyHostToDevice,
                         (cudaStream_t)stream) != cudaSuccess ||
-        cudaMemsetAsync(n->d_err, 0, sizeof(unsigned) * kCtlWords, (cudaStream_t)stream) != cudaSuccess ||
+        cudaMemsetAsync(n->d_err, 0, sizeof(unsigned) * 2 * kCtlWords, (cudaStream_t)stream) != cudaSuccess ||
         cudaStreamSynchronize((cudaStream_t)stream) != cudaSuccess) {
         cudaGetLastError();
         cudaFree(n->slab);

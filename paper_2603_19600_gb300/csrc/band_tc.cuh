@@ -85,7 +85,8 @@ static_assert(sizeof(double) * XS + (sizeof(double) * 96 + 128) * (TT / 32) <= k
 struct TcCtl {
     uint64_t taps_full, mma_done;
     uint32_t tmem;
-    unsigned nlist;
+    unsigned nlist, gave_up, held;
+    __align__(16) unsigned ctl[kCtlWords];   // the handle's control block, copied with the taps
     unsigned gmax[kTcPer * (TT / 32)];   // largest |x| (high word) of each 32 samples
     __align__(16) float w[kTcWeights];   // the detector's weights
     union {
@@ -106,7 +107,7 @@ __device__ __forceinline__ double *tc_stage(unsigned char *sm)
 __device__ __forceinline__ int32_t *tc_stage_pix(unsigned char *sm) { return reinterpret_cast<int32_t *>(tc_stage(sm) + 96); }
 
 // Start of the CTA: TMEM, barriers and the copy of the detector's tap digits. Every thread calls it.
-__device__ __forceinline__ void tc_begin(unsigned char *sm, const NoiseView &nv, int64_t gdet)
+__device__ __forceinline__ void tc_begin(unsigned char *sm, const NoiseView &nv, int64_t gdet, const unsigned *err)
 {
     TcCtl &C = *reinterpret_cast<TcCtl *>(sm + kTcOffCtl);
     if (threadIdx.x < 32) {
@@ -117,14 +118,15 @@ __device__ __forceinline__ void tc_begin(unsigned char *sm, const NoiseView &nv,
     }
     if (threadIdx.x < kTcWeights) C.w[threadIdx.x] = __ldg(nv.tc_w + gdet * kTcWeights + threadIdx.x);
     if (threadIdx.x == 0) {
-        C.nlist = 0u;
+        C.nlist = C.gave_up = C.held = 0u;
         mbar_init(&C.taps_full, 1);
         mbar_init(&C.mma_done, 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(&C.taps_full)),
-                     "r"(kTcCDig * 2 * kTcRun)
+                     "r"(kTcCDig * 2 * kTcRun + (int)sizeof C.ctl)
                      : "memory");
+        bulk_copy_g2s(C.ctl, err, sizeof C.ctl, &C.taps_full, false, 0);
         const unsigned char *src = nv.tc_taps + gdet * kTcDetBytes;
         for (int j = 0; j < kTcCDig; ++j)
             for (int h = 0; h < 2; ++h)
@@ -453,11 +455,12 @@ struct TcAll {   // every output is used
 // tc_ys(sm)[spos(t)] = sum_k c_|k| x_{t+k} for the tile's len outputs t. v[k]: the sample of slot u = threadIdx.x +
 // 512 k (slot 63 is the tile's first output; zero outside the stream and past the loaded samples). Every thread
 // calls it after tc_begin; on return the results are visible to the CTA and no TMEM is held. f64: FP64 accuracy of
-// every output (else that of the compensated product). again(w): w = v once more, for outputs that are formed again
+// every output (else that of the compensated product). False if a wait gave up: there are no results then, and the error
+// word is set. again(w): w = v once more, for outputs that are formed again
 // (to keep v in registers past the products cost N^-1 alone 109 -> 121 us of 8.4 M samples). used(t): false if outputs
 // t .. t + 7 are not used.
 template <class Again, class Used = TcAll>
-__device__ __forceinline__ void tc_band(unsigned char *sm, const double (&v)[kTcPer], const NoiseView &nv, int64_t gdet,
+__device__ __forceinline__ bool tc_band(unsigned char *sm, const double (&v)[kTcPer], const NoiseView &nv, int64_t gdet,
                                         unsigned *err, bool f64, int len, Again &&again, Used &&used = Used{})
 {
     TcCtl &C = *reinterpret_cast<TcCtl *>(sm + kTcOffCtl);
@@ -543,10 +546,16 @@ __device__ __forceinline__ void tc_band(unsigned char *sm, const double (&v)[kTc
         const long long budget = wait_budget(err);
         if (threadIdx.x == 0) {
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            if (mbar_wait(&C.taps_full, 0, err, budget)) tc_issue(sm, tmem);
-            asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-                             smem_u32(&C.mma_done))
-                         : "memory");
+            const bool taps = mbar_wait(&C.taps_full, 0, err, budget);
+            if (taps && C.ctl[1]) {
+                C.held = 1u;   // nothing is issued, and the waits run out
+            } else {
+                if (taps) tc_issue(sm, tmem);
+                else C.gave_up = 1u;
+                asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
+                                 smem_u32(&C.mma_done))
+                             : "memory");
+            }
         }
         __syncwarp();
         // while the products run: which blocks of outputs the digits do not resolve
@@ -554,10 +563,10 @@ __device__ __forceinline__ void tc_band(unsigned char *sm, const double (&v)[kTc
         const bool redo = t8 < len && tc_quiet(C, threadIdx.x, ldexpf(1.f, 25 - range)) && used(t8);
         nredo = __syncthreads_count(redo);
         if (redo) C.list[atomicAdd(&C.nlist, 1u)] = (uint16_t)threadIdx.x;
-        mbar_wait(&C.mma_done, 0, err, budget);
+        if (!mbar_wait(&C.mma_done, 0, err, budget)) C.gave_up = 1u;
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     } else {
-        if (threadIdx.x == 0) mbar_wait(&C.taps_full, 0, err, wait_budget(err));   // their region is written over
+        if (threadIdx.x == 0 && !mbar_wait(&C.taps_full, 0, err, wait_budget(err))) C.gave_up = 1u;   // written over below
         C.list[threadIdx.x] = (uint16_t)threadIdx.x;
         nredo = (len + 7) / 8;
         bool zero = gmax == 0u && ec != kTcBadTaps;
@@ -583,7 +592,7 @@ __device__ __forceinline__ void tc_band(unsigned char *sm, const double (&v)[kTc
         tc_put_samples(sm, w, dot2);
         __syncthreads();   // `again` may use the region of y
     }
-    if (digits) {
+    if (digits) {   // sums that are not complete are dropped below
         // warps 4 b .. 4 b + 3 hold the 128 rows of block b & 1, one lane each, and half b >> 1 of their columns
         const int half = warp >> 3, r0 = 128 * ((warp >> 2) & 1) + 32 * (warp & 3) + lane;
         const uint32_t at = tmem + ((uint32_t)(warp & 3) << 21) + 128u * ((warp >> 2) & 1) + 8u * half;
@@ -607,7 +616,14 @@ __device__ __forceinline__ void tc_band(unsigned char *sm, const double (&v)[kTc
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
-    if (nredo) {
+    const bool bad = C.gave_up != 0u;
+    if (bad) {   // what is in flight gets as long again to end before its memory is given back
+        if (threadIdx.x == 0) {
+            mbar_wait(&C.taps_full, 0, err, wait_budget(err));
+            if (digits && !C.held) mbar_wait(&C.mma_done, 0, err, wait_budget(err));
+        }
+        __syncthreads();
+    } else if (nredo) {
         const double *c = nv.p64 + gdet * nv.ntaps;
         if (dot2) tc_redo_dot2(sm, nredo, c, nv.ntaps);
         else tc_redo_chain(sm, nredo, c, nv.ntaps);
@@ -615,6 +631,7 @@ __device__ __forceinline__ void tc_band(unsigned char *sm, const double (&v)[kTc
     }
     if (warp == 0)
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kTcTmemCols));
+    return !bad;
 }
 
 }  // namespace fx

@@ -30,11 +30,11 @@ __global__ void __launch_bounds__(TT, 2) chi2_tc_kernel(const Tile *__restrict__
     if constexpr (BANDED) {
         stage = tc_stage(sm);
         spix = tc_stage_pix(sm);
-        tc_begin(sm, nv, gdet);
+        tc_begin(sm, nv, gdet, err);
         double v[kTcPer];
         const TcSlots sl(tl, ob);
         tc_fill_map<MODE, true>(sm, v, sl, pv, ob, tl, psi, m, d);
-        tc_band(sm, v, nv, gdet, err, f64, tl.len, TcKeep{v});
+        if (!tc_band(sm, v, nv, gdet, err, f64, tl.len, TcKeep{v})) return;
         // r^T N^-1 r over this thread's own slots: r is still at hand
 #pragma unroll
         for (int k = 0; k < kTcPer; ++k) {

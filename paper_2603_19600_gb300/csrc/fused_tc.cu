@@ -64,7 +64,7 @@ __global__ void __launch_bounds__(TT, 2) tc_operator_kernel(const Tile *__restri
     const ObsInfo ob = pv.obs[tl.obs];
     const int64_t gdet = ob.det_off + tl.det;
     const DetOffset psi(pv, gdet);
-    tc_begin(sm, nv, gdet);
+    tc_begin(sm, nv, gdet, err);
     if constexpr (TPL)
         if (threadIdx.x == 0) corr.init(tv, tl, ob, gdet);
     {
@@ -75,7 +75,7 @@ __global__ void __launch_bounds__(TT, 2) tc_operator_kernel(const Tile *__restri
             else tc_fill_map<MODE, false>(sm, w, sl, pv, ob, tl, psi, x, d);
         };
         fill(v);
-        tc_band(sm, v, nv, gdet, err, f64, tl.len, fill);
+        if (!tc_band(sm, v, nv, gdet, err, f64, tl.len, fill)) return;
     }
     const double *ys = tc_ys(sm);
     double *rec = acc64 + 3 * ob.map_off;
@@ -144,20 +144,20 @@ __global__ void __launch_bounds__(TT, 2) tc_ninv_kernel(const Tile *__restrict__
     const ObsInfo ob = obs[tl.obs];
     const int64_t gdet = ob.det_off + tl.det;
     const int64_t row = ob.tod_off + (int64_t)tl.det * ob.nsamp;
-    tc_begin(sm, nv, gdet);
+    tc_begin(sm, nv, gdet, err);
     double v[kTcPer];
     const TcSlots sl(tl, ob);
     tc_fill_tod(v, sl, in);
-    tc_band(sm, v, nv, gdet, err, f64, tl.len, [&](double (&w)[kTcPer]) { tc_fill_tod(w, sl, in); });
-    const double *ys = tc_ys(sm);
-    for (int k = threadIdx.x; k < tl.len; k += TT) out[row + tl.t0 + k] = ys[spos(k)];
+    const bool ok = tc_band(sm, v, nv, gdet, err, f64, tl.len, [&](double (&w)[kTcPer]) { tc_fill_tod(w, sl, in); });
+    const double *ys = tc_ys(sm);   // NaN where there are no results: this handle's status may never be asked for
+    for (int k = threadIdx.x; k < tl.len; k += TT) out[row + tl.t0 + k] = ok ? ys[spos(k)] : __longlong_as_double(-1LL);
 }
 
-furax_status launch_ninv_tc(const furax_noise *n, const double *in, double *out, bool f64, cudaStream_t st)
+furax_status launch_ninv_tc(const furax_noise *n, const double *in, double *out, bool f64, unsigned *err, cudaStream_t st)
 {
     if (n->n_tiles == 0) return FURAX_OK;
     furax_status rc = launch_dyn(tc_ninv_kernel, (unsigned)n->n_tiles, TT, kTcSmem, st, n->d_tiles, n->d_obs, n->view(), in, out,
-                                 n->d_err, f64);
+                                 err, f64);
     if (rc) return rc;
     count_launches(1);
     return check_launch("N^-1 apply (FP64, banded)");

@@ -224,7 +224,7 @@ __global__ void __launch_bounds__(TT, 2) gf_apply_tc_kernel(const Tile *__restri
     GfDet &s = sc[gdet];
     if (s.done) return;
     const double beta = s.beta;
-    tc_begin(sm, nv, gdet);
+    tc_begin(sm, nv, gdet, err);
     double v[kTcPer];
     const TcSlots sl(tl, ob);
 #pragma unroll
@@ -240,11 +240,12 @@ __global__ void __launch_bounds__(TT, 2) gf_apply_tc_kernel(const Tile *__restri
     for (int k = 0; k < kTcPer; ++k)
         if (!sl.in(k)) v[k] = 0.0;
     const int64_t row = sl.row + kHalo;
-    tc_band(sm, v, nv, gdet, err, f64, tl.len, TcKeep{v}, [&](int t) {   // outputs in gaps are not used
+    const bool ok = tc_band(sm, v, nv, gdet, err, f64, tl.len, TcKeep{v}, [&](int t) {   // outputs in gaps are not used
         bool any = false;
         for (int k = t; k < min(t + 8, tl.len); ++k) any = any || valid[row + k];
         return any;
     });
+    if (!ok) return;   // the host sees the error word
     const double *ys = tc_ys(sm);
     double acc = 0.0;
 #pragma unroll
@@ -329,7 +330,7 @@ furax_status gapfill(const furax_noise *n, const void *d, const uint8_t *valid, 
     // N y, of which the gaps' outputs are used: short bands on the tensor cores, FURAX_PREC_F32X2 with the
     // compensated product for tiles outside the digits' range
     auto ninv64 = [&](const double *in, double *o) {
-        return long_band(n) ? launch_ninv(n, in, o, FURAX_F64, st) : launch_ninv_tc(n, in, o, precision == FURAX_F64, st);
+        return long_band(n) ? launch_ninv(n, in, o, FURAX_F64, st) : launch_ninv_tc(n, in, o, precision == FURAX_F64, n->gf_err(), st);
     };
     const int64_t ns = n->nsamp_total, nd = n->ndet_total;
     if (ns == 0 || nd == 0) return FURAX_OK;
@@ -356,7 +357,9 @@ furax_status gapfill(const furax_noise *n, const void *d, const uint8_t *valid, 
     float *x32 = nm->gf_x32, *n32 = nm->gf_n32;
     std::vector<GfDet> h(nd);
     bool all_done = false;
+    unsigned gave_up = 0;
     if (!rc) rc = check_cuda(cudaMemsetAsync(sc, 0, sizeof(GfDet) * nd, st), "memset");
+    if (!rc) rc = check_cuda(cudaMemsetAsync(n->gf_err(), 0, sizeof gave_up, st), "clear");
     if (!rc) {
         if (dtype == FURAX_F64)
             gf_init_kernel<double><<<g, FT, 0, st>>>(n->d_tiles, n->d_obs, (const double *)d, (const double *)nr, valid,
@@ -372,7 +375,7 @@ furax_status gapfill(const furax_noise *n, const void *d, const uint8_t *valid, 
         }
         rc = check_launch("gap filling (start)");
     }
-    for (int it = 0; !rc && it < maxiter && !all_done; ++it) {
+    for (int it = 0; !rc && it < maxiter && !all_done && !gave_up; ++it) {
         if (f32) {   // N p in FP32
             if ((rc = launch_ninv(n, x32, n32, FURAX_F32, st))) break;
             gf_pq_kernel<float><<<g, FT, 0, st>>>(n->d_tiles, n->d_obs, valid, p, n32, nullptr, sc);
@@ -380,7 +383,7 @@ furax_status gapfill(const furax_noise *n, const void *d, const uint8_t *valid, 
             gf_update_kernel<float><<<g, FT, 0, st>>>(n->d_tiles, n->d_obs, valid, p, n32, y, r, sc);
         } else if (fused) {
             if ((rc = launch_dyn(gf_apply_tc_kernel, g, TT, kTcSmem, st, n->d_tiles, n->d_obs, n->view(), valid, r,
-                                 it % 2 ? p : nm->gf_p2, it % 2 ? nm->gf_p2 : p, q, sc, n->d_err, precision == FURAX_F64)))
+                                 it % 2 ? p : nm->gf_p2, it % 2 ? nm->gf_p2 : p, q, sc, n->gf_err(), precision == FURAX_F64)))
                 break;
             gf_step_kernel<<<g, FT, 0, st>>>(n->d_tiles, n->d_obs, it % 2 ? nm->gf_p2 : p, q, y, r, sc, tol * tol);
             count_launches(2);
@@ -398,6 +401,8 @@ furax_status gapfill(const furax_noise *n, const void *d, const uint8_t *valid, 
         if ((rc = check_launch("gap filling (iteration)"))) break;
         if ((it + 1) % 16 == 0 || it + 1 == maxiter) {
             if ((rc = check_cuda(cudaMemcpyAsync(h.data(), sc, sizeof(GfDet) * nd, cudaMemcpyDeviceToHost, st), "read")))
+                break;
+            if ((rc = check_cuda(cudaMemcpyAsync(&gave_up, n->gf_err(), sizeof gave_up, cudaMemcpyDeviceToHost, st), "read")))
                 break;
             if ((rc = check_cuda(cudaStreamSynchronize(st), "gap filling"))) break;
             all_done = true;
@@ -427,10 +432,8 @@ furax_status gapfill(const furax_noise *n, const void *d, const uint8_t *valid, 
         count_launches(1);
         rc = check_launch("gap filling (fill)");
     }
-    unsigned gave_up = 0;
     if (!rc) rc = check_cuda(cudaMemcpyAsync(h.data(), sc, sizeof(GfDet) * nd, cudaMemcpyDeviceToHost, st), "read");
-    if (!rc) rc = check_cuda(cudaMemcpyAsync(&gave_up, n->d_err, sizeof gave_up, cudaMemcpyDeviceToHost, st), "read");
-    if (!rc) rc = check_cuda(cudaMemsetAsync(n->d_err, 0, sizeof gave_up, st), "clear");
+    if (!rc) rc = check_cuda(cudaMemcpyAsync(&gave_up, n->gf_err(), sizeof gave_up, cudaMemcpyDeviceToHost, st), "read");
     if (!rc) rc = check_cuda(cudaStreamSynchronize(st), "gap filling");
     if (rc) return rc;
     if (gave_up) return set_error(FURAX_ETIMEOUT, "a bounded device-side wait gave up during gap filling");

@@ -19,7 +19,7 @@ constexpr int TILE = 4096;      // samples per work tile (one detector, contiguo
 inline int pixel_tile(int64_t npix_total) { return npix_total <= (1 << 18) ? 256 : 1024; }
 constexpr int MAXTAPS = 64;     // longest band of the fused kernels (c_0..c_63)
 constexpr int kLongTaps = 2048; // longest band of the overlap-save N^-1 (TOD in HBM)
-constexpr int kCtlWords = 4;    // device control block of a pointing handle (error, hold, wait budget)
+constexpr int kCtlWords = 4;    // device control block of a handle (error, hold, wait budget)
 constexpr int kBandPairs = 128; // band of the fused kernels in tap order (127 taps + one zero), as FP32 pairs
 
 struct ObsInfo {
@@ -281,7 +281,9 @@ struct furax_noise {
     unsigned char *tc_taps = nullptr;   // banded, <= MAXTAPS taps: digits of the taps for the tensor cores
     int32_t *tc_exp = nullptr;          // [ndet]
     float *tc_w = nullptr;              // [ndet][kTcWeights]
-    unsigned *d_err = nullptr;          // device control block (kCtlWords) of the kernels run on this handle alone
+    // device control blocks (kCtlWords each) of the kernels run on this handle alone: N^-1, then gap filling
+    unsigned *d_err = nullptr;
+    unsigned *gf_err() const { return d_err + fx::kCtlWords; }
     fx::NoiseView view() const { return fx::NoiseView{kind, ntaps, p64, p32, diag, tc_taps, tc_exp, tc_w, band2}; }
 };
 
@@ -315,8 +317,9 @@ furax_status launch_bj(const furax_pointing *p, const furax_noise *n, double rco
 
 // ---- launchers (noise.cu)
 furax_status launch_ninv(const furax_noise *n, const void *in, void *out, int dtype, cudaStream_t st);
-// FP64 in, FP64 out, bands of up to MAXTAPS taps on the tensor cores (fused_tc.cu); f64 as below.
-furax_status launch_ninv_tc(const furax_noise *n, const double *in, double *out, bool f64, cudaStream_t st);
+// FP64 in, FP64 out, bands of up to MAXTAPS taps on the tensor cores (fused_tc.cu); f64 as below. err: control block.
+furax_status launch_ninv_tc(const furax_noise *n, const double *in, double *out, bool f64, unsigned *err,
+                            cudaStream_t st);
 // Digits of the taps of a short band (fused_tc.cu).
 furax_status prepare_noise_tc(furax_noise *n, cudaStream_t st);
 size_t tc_taps_bytes(int64_t ndet);

@@ -2,10 +2,11 @@
 // A wait that has not completed within its budget of SM cycles records an error word in global
 // memory and returns false; the caller then leaves its loop, so a kernel always terminates.
 //
-// The handle's device control block (kCtlWords 32-bit words, furax_pointing::d_err):
-//   [0]    error word (kErrWaitTimeout once a wait gave up; cleared by furax_device_status)
-//   [1]    hold flag: the loader of the cached FP32 operator issues no copies while it is set
-//          (furax_debug_hold_loader), so that the other roles' waits run out
+// A handle's device control block (kCtlWords 32-bit words, furax_pointing::d_err, furax_noise::d_err and gf_err()):
+//   [0]    error word (kErrWaitTimeout once a wait gave up; cleared by furax_device_status, furax_noise_status
+//          and the next gap filling)
+//   [1]    hold flag: while it is set, the loader of the cached FP32 operator issues no copies and the tensor-core
+//          kernels no products (furax_debug_hold_loader, furax_debug_hold_noise), so that the other waits run out
 //   [2..3] wait budget in SM cycles (int64; 0 selects kWaitCycles)
 #pragma once
 #include <cstdint>

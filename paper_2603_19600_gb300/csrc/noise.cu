@@ -50,7 +50,7 @@ furax_status launch_ninv(const furax_noise *n, const void *in, void *out, int dt
     const NoiseView nv = n->view();
     const bool b = n->kind == FURAX_NOISE_BANDED;
     if (dtype == FURAX_F64) {
-        if (b) return launch_ninv_tc(n, (const double *)in, (double *)out, true, st);
+        if (b) return launch_ninv_tc(n, (const double *)in, (double *)out, true, n->d_err, st);
         ninv_kernel<double, false><<<g, FT, 0, st>>>(n->d_tiles, n->d_obs, nv, (const double *)in, (double *)out);
     } else {
         if (b) ninv_kernel<float, true><<<g, FT, 0, st>>>(n->d_tiles, n->d_obs, nv, (const float *)in, (float *)out);
