@@ -318,14 +318,15 @@ __device__ __forceinline__ void band_product_dfx2(const float *__restrict__ xs, 
 
 // Outputs of the n blocks in C.list again, from the samples in the taps' region (skewed; see tc_put_samples).
 
-// FP64 FMA chain. Few blocks: a warp each, four lanes to the band of an output (2,000 cycles where a thread per block
-// takes 20,000). Many: a thread each, whose eight outputs share the loads (normal operator with 4 taps: 178 us, with warps 316).
+// FP64 FMA chain. A warp per block, four lanes to the band of an output, or a thread per block, whose eight outputs share
+// the loads: whichever takes fewer FP64 instructions of a warp (17 blocks of 64 taps: 578 against 1016; 512 blocks of 4 taps:
+// 2048 against 896, which is 316 against 178 us of a normal operator).
 static __device__ __noinline__ void tc_redo_chain(unsigned char *sm, int n, const double *__restrict__ c, int ntaps)
 {
     const TcCtl &C = *reinterpret_cast<const TcCtl *>(sm + kTcOffCtl);
     const double *xs = reinterpret_cast<const double *>(sm);
     const int lane = threadIdx.x & 31, part = lane & 3, skip = kHalo + 1 - ntaps;
-    if (n > TT / 4) {
+    if ((n + 31) / 32 * 8 * (2 * ntaps - 1) <= n * ((2 * ntaps + 2) / 4 + 2)) {
         if ((int)threadIdx.x >= n) return;
         const int base = 8 * (int)C.list[threadIdx.x];
         double y[TR];

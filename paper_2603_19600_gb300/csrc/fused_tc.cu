@@ -75,7 +75,12 @@ __global__ void __launch_bounds__(TT, 2) tc_operator_kernel(const Tile *__restri
             else tc_fill_map<MODE, false>(sm, w, sl, pv, ob, tl, psi, x, d);
         };
         fill(v);
-        if (!tc_band(sm, v, nv, gdet, err, f64, tl.len, fill)) return;
+        bool ok;
+        if constexpr (MODE == 0 && !FROM_TOD)   // the recipe costs more than the registers
+            ok = tc_band(sm, v, nv, gdet, err, f64, tl.len, TcKeep{v});
+        else
+            ok = tc_band(sm, v, nv, gdet, err, f64, tl.len, fill);
+        if (!ok) return;
     }
     const double *ys = tc_ys(sm);
     double *rec = acc64 + 3 * ob.map_off;
