@@ -116,7 +116,9 @@ static furax_status dispatch_fused_f32(const furax_pointing *p, const furax_nois
 // had to be 72 KB of shared memory and 80 registers wide and ran its phases (pointing, exact recipe, gather, band,
 // scatter) one after the other. 64 x 262,144 samples, nside 512: 768 us that way, 648 us this way (626 us since the sums go straight into the output) with 32 tiles per SM
 // and chunk; with 16 some 60 us more, with 8, which stay in L2, 130 us more: the last round of every launch costs more than the 24
-// bytes per sample through memory. The workspace (250 MB) is all that on-the-fly pointing ever holds.
+// bytes per sample through memory. The workspace (250 MB) is all that on-the-fly pointing ever holds. The three kernels
+// of a chunk are dependent launches, each placed while the one before ends: 3 x 9001 samples with FP32 sums take 60 us in one kernel,
+// 64 us in ordinary launches and 58 us so (300 x 1000: 45, 50, 43 us).
 static int64_t chunk_tiles(const furax_pointing *p) { return std::min<int64_t>(p->n_tiles, 32LL * p->n_sm); }
 
 // The same workspace holds the FP64 pointing of half as many tiles (fused_tc.cu, chi2_tc.cu).

@@ -141,6 +141,7 @@ __global__ void __launch_bounds__(tma_threads<KC>(), 1)
                      double *__restrict__ acc64, unsigned *__restrict__ err, FusedTpl tpl, int l2_hint,
                      const unsigned *__restrict__ done, unsigned n_obs)
 {
+    if constexpr (LOCAL) prior_done();   // the pointing is written
     if (done && *done == n_obs) return;   // a PCG iteration after every observation has converged
     constexpr int kTmaConsumer = KC;
     constexpr int kConsOut = cons_out<KC>();
@@ -400,9 +401,13 @@ static furax_status run_tma_kc(const furax_pointing *p, const furax_noise *n, co
 {
     const int64_t nt = local ? local->n : p->n_tiles;
     const unsigned g = (unsigned)std::min<int64_t>(nt, p->n_sm);
-    return launch_dyn(fused_tma_kernel<ACC, BANDED, TPL, KC, LOCAL>, g, tma_threads<KC>(), tma_smem<ACC, KC>(), st,
-                      (const Tile *)p->d_tiles + (local ? local->tile0 : 0), nt, local ? local->pv : p->view(), n->view(), x32,
-                      hi, lo, a64, p->d_err, ft, local ? 0 : (int)p->sched.l2_evict_first, done, (unsigned)p->n_obs);
+    auto launch = [&](auto &&how) {
+        return how(fused_tma_kernel<ACC, BANDED, TPL, KC, LOCAL>, g, tma_threads<KC>(), tma_smem<ACC, KC>(), st,
+                   (const Tile *)p->d_tiles + (local ? local->tile0 : 0), nt, local ? local->pv : p->view(), n->view(), x32,
+                   hi, lo, a64, p->d_err, ft, local ? 0 : (int)p->sched.l2_evict_first, done, (unsigned)p->n_obs);
+    };
+    if constexpr (LOCAL) return launch([](auto &&...a) { return launch_behind(a...); });
+    return launch([](auto &&...a) { return launch_dyn(a...); });
 }
 
 // 16 consumer warps when the schedule asks for them (plain operator only; the template modes keep 8).

@@ -151,6 +151,31 @@ furax_status launch_dyn(void (*kern)(KArgs...), unsigned grid, unsigned block, s
     return FURAX_OK;
 }
 
+// A launch whose blocks may be placed while the kernel before it still runs (programmatic dependent launch). Both
+// kernels call prior_done() before they touch what an earlier one writes or reads; the one before may call let_next_start().
+template <typename... KArgs, typename... Args>
+furax_status launch_behind(void (*kern)(KArgs...), unsigned grid, unsigned block, size_t smem, cudaStream_t st,
+                           Args... args)
+{
+    if (smem > 48 * 1024) {
+        furax_status rc = allow_smem((const void *)kern, smem);
+        if (rc) return rc;
+    }
+    cudaLaunchAttribute attr{};
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(block);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    return check_cuda(cudaLaunchKernelEx(&cfg, kern, KArgs(args)...), "launch");
+}
+__device__ __forceinline__ void prior_done() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void let_next_start() { asm volatile("griddepcontrol.launch_dependents;"); }
+
 // Kernels without neighbours (no band) split a tile over gridDim.y blocks when there are few tiles
 // (tile_grid), so that a small observation still fills the GPU: this block's part of the tile (len may be <= 0).
 __device__ __forceinline__ Tile tile_part(Tile t)

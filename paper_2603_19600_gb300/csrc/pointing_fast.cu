@@ -35,6 +35,7 @@ namespace fx {
 // that must take the exact path (not finite, or |q|^2 not within 4u of 1).
 __global__ void bore_matrix_kernel(const double *__restrict__ q_bore, int64_t n, float *__restrict__ m)
 {
+    let_next_start();
     for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < n; t += (int64_t)gridDim.x * blockDim.x) {
         const Quat q = load_quat(q_bore, t);
         const double off = fabs(q.w * q.w + q.x * q.x + q.y * q.y + q.z * q.z - 1.0);
@@ -91,6 +92,10 @@ __global__ void __launch_bounds__(256, 4) expand_fast_kernel(const Tile *__restr
         qn = 0;
     }
     __syncthreads();
+    if constexpr (HALO > 0) {
+        let_next_start();
+        prior_done();   // the boresight rows are written; the operator is done with the previous chunk
+    }
     const DetAxes ax(sdet);
     const bool det_ok = sdet_ok != 0;
     const int64_t row = HALO ? (int64_t)blockIdx.x * kLocalTile - (tl.t0 - HALO) : ob.tod_off + tl.det * ob.nsamp;
@@ -144,8 +149,9 @@ furax_status launch_bore_rows(const furax_pointing *p, cudaStream_t st)
 furax_status launch_expand_local(const furax_pointing *p, int64_t tile0, int64_t n, int32_t *pix, float *c, float *s,
                                  cudaStream_t st)
 {
-    expand_fast_kernel<kHalo><<<(unsigned)n, 256, 0, st>>>(p->d_tiles + tile0, p->d_obs, p->q_bore, p->q_det, p->ws_bore_m,
-                                                           p->has_hwp ? p->d_hwp_cs : nullptr, pix, c, s, nullptr);
+    furax_status rc = launch_behind(expand_fast_kernel<kHalo>, (unsigned)n, 256, 0, st, p->d_tiles + tile0, p->d_obs, p->q_bore,
+                                    p->q_det, p->ws_bore_m, p->has_hwp ? p->d_hwp_cs : nullptr, pix, c, s, nullptr);
+    if (rc) return rc;
     count_launches(1);
     return check_launch("pointing of a chunk of tiles");
 }
