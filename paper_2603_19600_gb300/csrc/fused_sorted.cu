@@ -483,8 +483,9 @@ furax_status set_schedule(furax_pointing *p, const furax_schedule &s, cudaStream
 
     // detector lines of sight in the boresight frame
     std::vector<double> qd(4 * (size_t)p->ndet_total);
-    if ((rc = check_cuda(cudaMemcpy(qd.data(), p->q_det, sizeof(double) * qd.size(), cudaMemcpyDeviceToHost),
-                         "read detector quaternions")))
+    if ((rc = check_cuda(cudaMemcpyAsync(qd.data(), p->q_det, sizeof(double) * qd.size(), cudaMemcpyDeviceToHost, st),
+                         "read detector quaternions")) ||
+        (rc = check_cuda(cudaStreamSynchronize(st), "read detector quaternions")))
         return rc;
     std::vector<STile> tiles;
     std::vector<int32_t> sdet;
@@ -496,14 +497,17 @@ furax_status set_schedule(furax_pointing *p, const furax_schedule &s, cudaStream
         // mean rotation axis of the scan over 16 sample pairs spread over the observation
         double ax[3] = {0.0, 0.0, 0.0};
         if (ob.nsamp >= 2) {
-            std::vector<double> qb(8);
+            std::vector<double> qb(8 * 16);
             for (int k = 0; k < 16; ++k) {
                 const int64_t t = std::min<int64_t>(ob.nsamp - 2, (int64_t)((k + 0.5) * (double)ob.nsamp / 16.0));
-                if ((rc = check_cuda(cudaMemcpy(qb.data(), p->q_bore + 4 * (ob.bore_off + t), sizeof(double) * 8,
-                                                cudaMemcpyDeviceToHost), "read boresight")))
+                if ((rc = check_cuda(cudaMemcpyAsync(&qb[8 * k], p->q_bore + 4 * (ob.bore_off + t), sizeof(double) * 8,
+                                                     cudaMemcpyDeviceToHost, st), "read boresight")))
                     return rc;
+            }
+            if ((rc = check_cuda(cudaStreamSynchronize(st), "read boresight"))) return rc;
+            for (int k = 0; k < 16; ++k) {
                 double a[3];
-                if (rotation_axis(qb.data(), qb.data() + 4, a)) {
+                if (rotation_axis(&qb[8 * k], &qb[8 * k + 4], a)) {
                     const double sg = (a[0] * ax[0] + a[1] * ax[1] + a[2] * ax[2]) < 0.0 ? -1.0 : 1.0;
                     for (int c = 0; c < 3; ++c) ax[c] += sg * a[c];
                 }
@@ -607,9 +611,10 @@ furax_status set_schedule(furax_pointing *p, const furax_schedule &s, cudaStream
     }
     p->n_stiles = (int64_t)tiles.size();
     p->perm_cap = cap;
-    if ((rc = check_cuda(cudaMemcpy(p->d_stiles, tiles.data(), sizeof(STile) * tiles.size(), cudaMemcpyHostToDevice),
+    // on the stream that sorts: a copy on the legacy stream may still be under way when it returns
+    if ((rc = check_cuda(cudaMemcpyAsync(p->d_stiles, tiles.data(), sizeof(STile) * tiles.size(), cudaMemcpyHostToDevice, st),
                          "upload sorted tiles")) ||
-        (rc = check_cuda(cudaMemcpy(p->d_sdet, sdet.data(), sizeof(int32_t) * sdet.size(), cudaMemcpyHostToDevice),
+        (rc = check_cuda(cudaMemcpyAsync(p->d_sdet, sdet.data(), sizeof(int32_t) * sdet.size(), cudaMemcpyHostToDevice, st),
                          "upload tile rows"))) {
         free_sorted(p);
         p->sched.kernel = FURAX_SCHED_TIME_ORDERED;

@@ -20,6 +20,13 @@ def test_no_clear_on_the_default_stream():
         assert not re.search(r"\bcudaMemset\s*\(", code), path
 
 
+def test_no_copy_on_the_default_stream():
+    """cudaMemcpy from pageable memory may return before the copy has reached the device, on that stream."""
+    for path in glob.glob(os.path.join(CSRC, "*.cu*")):
+        code = re.sub(r"//[^\n]*", "", open(path).read())
+        assert not re.search(r"\bcudaMemcpy\s*\(", code), path
+
+
 @pytest.mark.gpu
 @pytest.mark.parametrize("kw", [{"tol": 1e-10}, {"tol": 1e-10, "binned_only": True},
                                 {"tol": 1e-8, "precision": "f32", "acc": "f64"}])
