@@ -16,7 +16,8 @@ namespace fx {
 // ------------------------------------------------------------------------------------
 // FP32 fused apply: acc += P^T N^-1 P x32  (x32: padded FP32 map, zero on masked pixels)
 // ------------------------------------------------------------------------------------
-template <int MODE, int ACC, bool BANDED>
+// On the FP64 cache (FP32 weights are read by the pipelined kernels).
+template <int ACC, bool BANDED>
 __global__ void __launch_bounds__(FT, 3) fused_f32_kernel(const Tile *__restrict__ tiles, PointingView pv, NoiseView nv,
                                                           const float4 *__restrict__ x32, float4 *__restrict__ acc_hi,
                                                           float4 *__restrict__ acc_lo, double *__restrict__ acc64)
@@ -41,7 +42,7 @@ __global__ void __launch_bounds__(FT, 3) fused_f32_kernel(const Tile *__restrict
         float v = 0.f, c = 0.f, s = 0.f;
         int32_t pix = -1;
         if (t >= 0 && t < ob.nsamp) {
-            pix = get_sample<MODE, float>(pv, ob, tl.det, t, c, s);
+            pix = get_sample<FURAX_POINTING_CACHE_F64, float>(pv, ob, tl.det, t, c, s);
             if (pix >= 0) {
                 const float4 m = __ldg(x32 + ob.map_off + pix);
                 v = fmaf(m.z, s, fmaf(m.y, c, m.x));
@@ -86,7 +87,7 @@ __global__ void __launch_bounds__(FT, 3) fused_f32_kernel(const Tile *__restrict
     }
 }
 
-template <int MODE, bool BANDED>
+template <bool BANDED>
 static furax_status dispatch_fused_f32_acc(const furax_pointing *p, const furax_noise *n, const float4 *x32, int acc,
                                            float4 *hi, float4 *lo, double *a64, cudaStream_t st)
 {
@@ -94,21 +95,20 @@ static furax_status dispatch_fused_f32_acc(const furax_pointing *p, const furax_
     const PointingView pv = p->view();
     const NoiseView nv = n->view();
     if (acc == FURAX_ACC_F32)
-        return launch_dyn(fused_f32_kernel<MODE, FURAX_ACC_F32, BANDED>, g, FT, kF32Smem, st, p->d_tiles, pv, nv, x32,
+        return launch_dyn(fused_f32_kernel<FURAX_ACC_F32, BANDED>, g, FT, kF32Smem, st, p->d_tiles, pv, nv, x32,
                           hi, lo, a64);
     if (acc == FURAX_ACC_F32_KAHAN)
-        return launch_dyn(fused_f32_kernel<MODE, FURAX_ACC_F32_KAHAN, BANDED>, g, FT, kF32Smem, st, p->d_tiles, pv, nv,
+        return launch_dyn(fused_f32_kernel<FURAX_ACC_F32_KAHAN, BANDED>, g, FT, kF32Smem, st, p->d_tiles, pv, nv,
                           x32, hi, lo, a64);
-    return launch_dyn(fused_f32_kernel<MODE, FURAX_ACC_F64, BANDED>, g, FT, kF32Smem, st, p->d_tiles, pv, nv, x32, hi,
+    return launch_dyn(fused_f32_kernel<FURAX_ACC_F64, BANDED>, g, FT, kF32Smem, st, p->d_tiles, pv, nv, x32, hi,
                       lo, a64);
 }
 
-template <int MODE>
 static furax_status dispatch_fused_f32(const furax_pointing *p, const furax_noise *n, const float4 *x32, int acc,
                                        float4 *hi, float4 *lo, double *a64, cudaStream_t st)
 {
-    if (n->kind == FURAX_NOISE_BANDED) return dispatch_fused_f32_acc<MODE, true>(p, n, x32, acc, hi, lo, a64, st);
-    return dispatch_fused_f32_acc<MODE, false>(p, n, x32, acc, hi, lo, a64, st);
+    if (n->kind == FURAX_NOISE_BANDED) return dispatch_fused_f32_acc<true>(p, n, x32, acc, hi, lo, a64, st);
+    return dispatch_fused_f32_acc<false>(p, n, x32, acc, hi, lo, a64, st);
 }
 
 // On the fly: the certified pointing (pointing_fast.cu) of a chunk of tiles goes to a workspace, and the
@@ -180,19 +180,19 @@ furax_status launch_fused_f32(const furax_pointing *p, const furax_noise *n, con
         rc = launch_fused_sorted(p, n, x32, acc, hi, lo, a64, st);   // pixel-sorted schedule
     else if (p->mode == FURAX_POINTING_CACHE_F32 || p->mode == FURAX_POINTING_CACHE_MIXED)  // FP32 weights: hi
         rc = launch_fused_tma(p, n, x32, acc, hi, lo, a64, st, ft, done);
-    else rc = dispatch_fused_f32<2>(p, n, x32, acc, hi, lo, a64, st);
+    else rc = dispatch_fused_f32(p, n, x32, acc, hi, lo, a64, st);
     if (rc) return rc;
     count_launches(1);
     return check_launch("fused P^T N^-1 P (FP32)");
 }
 
-template <int MODE, bool B>
-static furax_status prep_f32_mode_band()
+template <bool B>
+static furax_status prep_f32_band()
 {
     furax_status rc = FURAX_OK;
-    if (!rc) rc = allow_smem((const void *)fused_f32_kernel<MODE, FURAX_ACC_F32, B>, kF32Smem);
-    if (!rc) rc = allow_smem((const void *)fused_f32_kernel<MODE, FURAX_ACC_F32_KAHAN, B>, kF32Smem);
-    if (!rc) rc = allow_smem((const void *)fused_f32_kernel<MODE, FURAX_ACC_F64, B>, kF32Smem);
+    if (!rc) rc = allow_smem((const void *)fused_f32_kernel<FURAX_ACC_F32, B>, kF32Smem);
+    if (!rc) rc = allow_smem((const void *)fused_f32_kernel<FURAX_ACC_F32_KAHAN, B>, kF32Smem);
+    if (!rc) rc = allow_smem((const void *)fused_f32_kernel<FURAX_ACC_F64, B>, kF32Smem);
     return rc;
 }
 
@@ -200,8 +200,8 @@ furax_status prepare_fused_f32()
 {
     furax_status rc = prepare_fused_tma();
     if (!rc) rc = prepare_fused_sorted();
-    if (!rc) rc = prep_f32_mode_band<2, true>();
-    if (!rc) rc = prep_f32_mode_band<2, false>();
+    if (!rc) rc = prep_f32_band<true>();
+    if (!rc) rc = prep_f32_band<false>();
     return rc;
 }
 

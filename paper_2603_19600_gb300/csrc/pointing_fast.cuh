@@ -17,49 +17,24 @@ constexpr int kBoreRow = 20;
 constexpr double kUnitTol = 4.0 * 5.9604644775390625e-8;       // |q|^2 within this of 1: FP32 path
 
 __device__ __forceinline__ unsigned long long f2_neg(unsigned long long a) { return a ^ 0x8000000080000000ull; }
-__device__ __forceinline__ unsigned long long f2_add_rn(unsigned long long a, unsigned long long b)
-{
-    unsigned long long d;
-    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-    return d;
-}
-__device__ __forceinline__ unsigned long long f2_sub_rn(unsigned long long a, unsigned long long b)
-{
-    unsigned long long d;
-    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-    return d;
-}
-__device__ __forceinline__ unsigned long long f2_mul_rn(unsigned long long a, unsigned long long b)
-{
-    unsigned long long d;
-    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-    return d;
-}
-__device__ __forceinline__ unsigned long long f2_fma_rn(unsigned long long a, unsigned long long b, unsigned long long c)
-{
-    unsigned long long d;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
-    return d;
-}
-
 // Two dot products of three terms in double-FP32 (exact products of the hi parts, two-sums), rounded to
 // FP32: packed, so that the six of a sample are three of these (half the instructions, the same roundings).
 __device__ __forceinline__ unsigned long long dot3_df_x2(const unsigned long long (&mh)[3], const unsigned long long (&ml)[3],
                                                          const unsigned long long (&vh)[3], const unsigned long long (&vl)[3])
 {
-    unsigned long long s = f2_mul_rn(mh[0], vh[0]);
-    unsigned long long err = f2_fma_rn(mh[0], vl[0], f2_fma_rn(ml[0], vh[0], f2_fma_rn(mh[0], vh[0], f2_neg(s))));
+    unsigned long long s = f2_mul(mh[0], vh[0]);
+    unsigned long long err = f2_fma(mh[0], vl[0], f2_fma(ml[0], vh[0], f2_fma(mh[0], vh[0], f2_neg(s))));
 #pragma unroll
     for (int j = 1; j < 3; ++j) {
-        const unsigned long long p = f2_mul_rn(mh[j], vh[j]);
-        const unsigned long long e = f2_fma_rn(mh[j], vh[j], f2_neg(p));
-        const unsigned long long t = f2_add_rn(s, p);
-        const unsigned long long bv = f2_sub_rn(t, s);
-        const unsigned long long te = f2_add_rn(f2_sub_rn(s, f2_sub_rn(t, bv)), f2_sub_rn(p, bv));
+        const unsigned long long p = f2_mul(mh[j], vh[j]);
+        const unsigned long long e = f2_fma(mh[j], vh[j], f2_neg(p));
+        const unsigned long long t = f2_add(s, p);
+        const unsigned long long bv = f2_sub(t, s);
+        const unsigned long long te = f2_add(f2_sub(s, f2_sub(t, bv)), f2_sub(p, bv));
         s = t;
-        err = f2_fma_rn(mh[j], vl[j], f2_fma_rn(ml[j], vh[j], f2_add_rn(err, f2_add_rn(te, e))));
+        err = f2_fma(mh[j], vl[j], f2_fma(ml[j], vh[j], f2_add(err, f2_add(te, e))));
     }
-    return f2_add_rn(s, err);
+    return f2_add(s, err);
 }
 
 __device__ __forceinline__ float frac_dist(float v)
