@@ -32,17 +32,19 @@
 // chain's error, only where the band reaches samples that are not too far below X. So every block of 8
 // outputs is checked: sums of |x| over blocks of 8 samples, weighted with the smallest |tap| that joins the
 // two blocks, bound |c| * |x| of its outputs from below (within a factor of 2 for the 1/f band), and blocks for
-// which that is under 2^-kTcRange X C are formed again by the FP64 FMA chain, a warp per block. Up to there the
-// digits' error is at most 6 u |c| * |x| in emulation (u = 2^-53; rms 0.3 u on Gaussian samples), that of the chain up to 13 u
+// which that is under 2^-kTcRange X C are formed again by the FP64 FMA chain. (Ordinary noise passes by a coarser bound of the
+// same kind, over groups of 32 samples, without the blocks: right-hand side of 67 M samples 1456 -> 1426 us.) Up to the line the
+// digits' error is at most 9 u |c| * |x| in emulation (u = 2^-53; rms 0.3 u on Gaussian samples), that of the chain up to 14 u
 // (rms 2 u). An output whose band holds only zeros is exact in digits too. Where the caller asked for no more
 // than the compensated double-FP32 product, the line is kTcRangeDot2, and many blocks take that product.
 // A few loud samples (glitches, a planet, infinities and NaNs) are left out of the digits, and every block whose band
 // reaches one is formed again (tc_band). Tiles with extreme exponents, tiles mostly below the line, and bands whose
 // small or missing taps would send ordinary noise to the chain (tap_digits_kernel) form every block that way.
-// Measured (FP64 data, 32 x 131,071 samples, N^-1 alone, all tiles alike): 65 us in digits (58 without sums and check), 126 us
+// Measured (FP64 data, 32 x 131,071 samples, N^-1 alone, all tiles alike): 64 us in digits (58 without the checks), 126 us
 // with a glitch per tile (895 with the chain for the whole tile), 524 us with half of each tile 2^16 louder.
 #pragma once
 #include <cuda_fp16.h>
+#include <type_traits>
 #include "tile.cuh"
 #include "mbarrier.cuh"
 
@@ -67,7 +69,7 @@ constexpr int kTcNoTaps = -(1 << 20);                   // "exponent" of taps th
 constexpr int kTcBadTaps = -(1 << 21);                  // of taps that are not finite
 constexpr int kTcBlocks = kTcSlots / 8;                 // blocks of 8 samples
 constexpr int kTcReach = 17;                            // blocks that the band joins to a block of 8 outputs
-constexpr int kTcWeights = 16;                          // floats per detector: weights of the first 16 (the last is 0)
+constexpr int kTcWeights = 16;                          // floats per detector: weights of the first 15, then that of groups of 32
 constexpr int kTcSumRows = 64 + kTcReach - 1;
 constexpr uint32_t kTcOut28 = 1u << 28;                 // marks a sample above the cut in a sum of 25-bit magnitudes
 constexpr int kTcChainTaps = 16;                        // bands up to this long take the chain in either precision
@@ -89,6 +91,7 @@ struct TcCtl {
     __align__(16) unsigned ctl[kCtlWords];   // the handle's control block, copied with the taps
     unsigned gmax[kTcPer * (TT / 32)];   // largest |x| (high word) of each 32 samples
     __align__(16) float w[kTcWeights];   // the detector's weights
+    uint32_t least[TT / 32];             // per warp: smallest sum of |x| over 32 samples
     union {
         float sum[kTcSumRows][9];        // sum of |x| over 8 samples (tc_put_sum)
         uint16_t list[TILE / 8];         // blocks of outputs that are formed again
@@ -409,7 +412,7 @@ __device__ __forceinline__ bool tc_quiet(const TcCtl &C, int o, float line)
 #pragma unroll
     for (int m = 0; m < kTcReach; ++m) {
         any = fmaxf(any, x[9 * m]);
-        if (m < kTcWeights) s = fmaf(C.w[m], x[9 * m], s);
+        if (m < kTcWeights - 1) s = fmaf(C.w[m], x[9 * m], s);
     }
     return any > 0.f && (s < line || any > 1e30f);
 }
@@ -481,8 +484,11 @@ __device__ __forceinline__ bool tc_band(unsigned char *sm, const double (&v)[kTc
     const int ey = emax - 1022 + ec - 69;   // y = (H 2^32 + L) 2^ey
     digits = digits && emax >= 123 && emax < 2047 && ec > -900 && ec < 900 && ey > -900 && ey < 900;
     // the compensated product, well inside FP32's range
-    const bool may_dot2 = !f64 && emax > 1023 - 80 && (int)(gmax >> 20) < 1023 + 100;
+    const bool may_dot2 = !f64 && nv.ntaps > kTcChainTaps && emax > 1023 - 80 && (int)(gmax >> 20) < 1023 + 100;
     const uint32_t tmem = C.tmem;
+    // The chain takes 565 cycles a block with 64 taps, the compensated product, which walks 127 taps whatever their number,
+    // 15,000 for any few and 150 a block for many (normal operator with 8 taps: 282 us with the chain, 459 us).
+    constexpr int kDot2From = 32;
     int nredo = 0;
     if (digits) {
         unsigned char *px = sm + kTcOffX;
@@ -508,14 +514,28 @@ __device__ __forceinline__ bool tc_band(unsigned char *sm, const double (&v)[kTc
                 tc_put2(p + 12 * kTcPitch, wl, 0x4041);
             }
         }
-        // sums over blocks: slot u = threadIdx.x + 512 k is of block 64 k + threadIdx.x / 8
-        static_assert(kTcPer == 9 && TT == 512, "eight samples at once, then the ninth");
-        const int at = threadIdx.x >> 3;
-        tc_put_sum(C, at, lane & 7, tc_sum8(a));
-        if (512 + at < kTcBlocks) {   // whole warps
+        auto block_sums = [&] {
+            // sums over blocks: slot u = threadIdx.x + 512 k is of block 64 k + threadIdx.x / 8
+            static_assert(kTcPer == 9 && TT == 512, "eight samples at once, then the ninth");
+            const int at = threadIdx.x >> 3;
+            tc_put_sum(C, at, lane & 7, tc_sum8(a));
+            if (512 + at < kTcBlocks) {   // whole warps
 #pragma unroll
-            for (int o = 1; o < 8; o <<= 1) a[8] += __shfl_xor_sync(0xffffffffu, a[8], o);
-            if ((lane & 7) == 0) tc_put_sum(C, at, 8, a[8]);
+                for (int o = 1; o < 8; o <<= 1) a[8] += __shfl_xor_sync(0xffffffffu, a[8], o);
+                if ((lane & 7) == 0) tc_put_sum(C, at, 8, a[8]);
+            }
+        };
+        // Smallest sum over 32 samples, by which ordinary noise is accepted; vectors with gaps are not.
+        constexpr bool kQuick = std::is_same_v<std::decay_t<Used>, TcAll>;
+        uint32_t least = 0xffffffffu;
+        if constexpr (kQuick) {
+#pragma unroll
+            for (int k = 0; k < kTcPer; ++k)
+                if (k < kTcPer - 1 || warp < (kTcSlots - TT * (kTcPer - 1)) / 32)
+                    least = min(least, __reduce_add_sync(0xffffffffu, a[k]));
+            if (lane == 0) C.least[warp] = least;
+        } else {
+            block_sums();
         }
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // the digits, for the tensor core's reads
         __syncthreads();
@@ -534,13 +554,28 @@ __device__ __forceinline__ bool tc_band(unsigned char *sm, const double (&v)[kTc
             }
         }
         __syncwarp();
-        // while the products run: which blocks of outputs the digits do not resolve
-        const int t8 = 8 * threadIdx.x;
-        const bool redo = t8 < len && tc_quiet(C, threadIdx.x, ldexpf(1.f, 25 - range)) && used(t8);
-        nredo = __syncthreads_count(redo);
-        if (redo) C.list[atomicAdd(&C.nlist, 1u)] = (uint16_t)threadIdx.x;
+        // While the products run: which blocks of outputs the digits do not resolve. None if no 32 samples are quiet enough
+        // for three groups of them to be (ordinary noise, except at the ends of streams).
+        const float line = ldexpf(1.f, 25 - range);
+        if constexpr (kQuick) least = __reduce_min_sync(0xffffffffu, C.least[lane % (TT / 32)]);
+        if (!kQuick || emax < (int)(gmax >> 20) || (float)least * C.w[kTcWeights - 1] < line) {
+            if constexpr (kQuick) {
+                block_sums();
+                __syncthreads();
+            }
+            const int t8 = 8 * threadIdx.x;
+            const bool redo = t8 < len && tc_quiet(C, threadIdx.x, line) && used(t8);
+            nredo = __syncthreads_count(redo);
+            if (redo) C.list[atomicAdd(&C.nlist, 1u)] = (uint16_t)threadIdx.x;
+        }
         if (!mbar_wait(&C.mma_done, 0, err, budget)) C.gave_up = 1u;
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        if (nredo) {
+            double w[kTcPer];
+            again(w);
+            tc_put_samples(sm, w, may_dot2 && nredo > kDot2From);
+            __syncthreads();   // `again` may use the region of y
+        }
     } else {
         if (threadIdx.x == 0 && !mbar_wait(&C.taps_full, 0, err, wait_budget(err))) C.gave_up = 1u;   // written over below
         C.list[threadIdx.x] = (uint16_t)threadIdx.x;
@@ -558,15 +593,7 @@ __device__ __forceinline__ bool tc_band(unsigned char *sm, const double (&v)[kTc
             for (int r = 0; r < TR; ++r) tc_ys(sm)[spos(TR * threadIdx.x + r)] = 0.0;
         }
         __syncthreads();
-    }
-    // The chain takes 565 cycles a block with 64 taps, the compensated product, which walks 127 taps whatever their number,
-    // 15,000 for any few and 150 a block for many (normal operator with 8 taps: 282 us with the chain, 459 us).
-    const bool dot2 = may_dot2 && nredo > 32 && nv.ntaps > kTcChainTaps;
-    if (nredo) {
-        double w[kTcPer];
-        again(w);
-        tc_put_samples(sm, w, dot2);
-        __syncthreads();   // `again` may use the region of y
+        if (nredo) tc_put_samples(sm, v, may_dot2 && nredo > kDot2From);
     }
     if (digits) {   // sums that are not complete are dropped below
         // warps 4 b .. 4 b + 3 hold the 128 rows of block b & 1, one lane each, and half b >> 1 of their columns
@@ -601,7 +628,7 @@ __device__ __forceinline__ bool tc_band(unsigned char *sm, const double (&v)[kTc
         __syncthreads();
     } else if (nredo) {
         const double *c = nv.p64 + gdet * nv.ntaps;
-        if (dot2) tc_redo_dot2(sm, nredo, c, nv.ntaps);
+        if (may_dot2 && nredo > kDot2From) tc_redo_dot2(sm, nredo, c, nv.ntaps);
         else tc_redo_chain(sm, nredo, c, nv.ntaps);
         __syncthreads();
     }

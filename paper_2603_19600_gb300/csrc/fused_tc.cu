@@ -277,18 +277,35 @@ __global__ void __launch_bounds__(128) tap_digits_kernel(const double *__restric
     if (scalbn(m, -ec) > 0.99) ++ec;
     // Weight m: the smallest tap between sample block o + m and output block o (tap index 8 m - 7 .. 8 m + 7).
     __shared__ float w[kTcWeights];
-    if (threadIdx.x < kTcWeights) {
+    if (threadIdx.x < kTcWeights - 1) {
         double v = m;
         for (int j = 8 * (int)threadIdx.x - 7; j <= 8 * (int)threadIdx.x + 7; ++j)
             v = j < 0 || j >= kBand ? 0.0 : fmin(v, fabs(c[j < kHalo ? kHalo - j : j - kHalo]));
         w[threadIdx.x] = ok ? (float)scalbn(v, -ec) : 0.f;
         weights[det * kTcWeights + threadIdx.x] = w[threadIdx.x];
     }
+    // The same for groups of 32 samples: the smallest sum, over the 32 places an output can have, of the smallest tap of
+    // each group that lies within its band (three or four).
+    __shared__ double place[32];
+    if (threadIdx.x < 32) {
+        double sum = 0.0;
+        for (int j0 = (32 - (int)threadIdx.x) % 32; j0 + 32 <= kBand; j0 += 32) {
+            double v = m;
+            for (int j = j0; j < j0 + 32; ++j) v = fmin(v, fabs(c[j < kHalo ? kHalo - j : j - kHalo]));
+            sum += v;
+        }
+        place[threadIdx.x] = sum;
+    }
     __syncthreads();
+    if (threadIdx.x == 0) {
+        double v = place[0];
+        for (int i = 1; i < 32; ++i) v = fmin(v, place[i]);
+        weights[det * kTcWeights + kTcWeights - 1] = ok ? (float)scalbn(v, -ec) : 0.f;
+    }
     // Gaussian samples have sums of 6.4 sigma = 1.6 X where X = 4 sigma; twice that over the line on average leaves few
     // blocks of ordinary noise below it.
     float sum = 0.f;
-    for (int i = 0; i < kTcWeights; ++i) sum += w[i];
+    for (int i = 0; i < kTcWeights - 1; ++i) sum += w[i];
     ok = ok && 1.6f * sum >= ldexpf(2.f, -kTcRange);
     if (threadIdx.x == 0) exps[det] = ok ? ec : finite ? kTcNoTaps : kTcBadTaps;
     __half *o = reinterpret_cast<__half *>(out + det * kTcDetBytes);
