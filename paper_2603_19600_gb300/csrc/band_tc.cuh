@@ -240,7 +240,8 @@ __device__ __forceinline__ void dot2_step_x2(unsigned long long ch, unsigned lon
     E = f2_fma(cl, x, f2_add(E, f2_add(err, e)));
 }
 
-template <int R>
+// LOW: the samples have low words (FP32 data has none).
+template <int R, bool LOW>
 __device__ __forceinline__ void band_product_dfx2(const float *__restrict__ xs, const float *__restrict__ xl,
                                                   const float4 *__restrict__ C4, const float2 *__restrict__ CL2, int base,
                                                   float (&S)[R], float (&E)[R])
@@ -250,7 +251,7 @@ __device__ __forceinline__ void band_product_dfx2(const float *__restrict__ xs, 
 #pragma unroll
     for (int i = 0; i < H; ++i) {
         W[i] = pack_f32x2(xs[spos(base + i)], xs[spos(base + i + H)]);
-        WL[i] = pack_f32x2(xl[spos(base + i)], xl[spos(base + i + H)]);
+        if constexpr (LOW) WL[i] = pack_f32x2(xl[spos(base + i)], xl[spos(base + i + H)]);
         SS[i] = 0ull;
         EE[i] = 0ull;
     }
@@ -267,7 +268,7 @@ __device__ __forceinline__ void band_product_dfx2(const float *__restrict__ xs, 
 #pragma unroll
                 for (int i = 0; i < H; ++i) {
                     dot2_step_x2(ch, nch, cl, W[i], SS[i], EE[i]);
-                    EE[i] = f2_fma(ch, WL[i], EE[i]);
+                    if constexpr (LOW) EE[i] = f2_fma(ch, WL[i], EE[i]);
                 }
                 if (j < kBand - 1) {
                     float lo0, hi0;
@@ -276,7 +277,7 @@ __device__ __forceinline__ void band_product_dfx2(const float *__restrict__ xs, 
 #pragma unroll
                     for (int i = 0; i < H - 1; ++i) W[i] = W[i + 1];
                     W[H - 1] = wl;
-                    {
+                    if constexpr (LOW) {
                         unpack_f32x2(WL[0], lo0, hi0);
                         const unsigned long long wll = pack_f32x2(hi0, xl[spos(base + R + j)]);
 #pragma unroll
@@ -334,6 +335,7 @@ static __device__ __noinline__ void tc_redo_chain(unsigned char *sm, int n, cons
 }
 
 // The compensated product, a thread per block.
+template <bool LOW>
 static __device__ __noinline__ void tc_redo_dot2(unsigned char *sm, int n, const double *__restrict__ c, int ntaps)
 {
     const TcCtl &C = *reinterpret_cast<const TcCtl *>(sm + kTcOffCtl);
@@ -351,7 +353,7 @@ static __device__ __noinline__ void tc_redo_dot2(unsigned char *sm, int n, const
     if ((int)threadIdx.x >= n) return;
     float S[TR], E[TR];
     const int base = 8 * (int)C.list[threadIdx.x];
-    band_product_dfx2<TR>(xh, xl, C4, CL2, base, S, E);
+    band_product_dfx2<TR, LOW>(xh, xl, C4, CL2, base, S, E);
     double *ys = tc_ys(sm);
 #pragma unroll
     for (int r = 0; r < TR; ++r) ys[spos(base + r)] = (double)S[r] + (double)E[r];
@@ -434,11 +436,11 @@ struct TcAll {   // every output is used
 // tc_ys(sm)[spos(t)] = sum_k c_|k| x_{t+k} for the tile's len outputs t. v[k]: the sample of slot u = threadIdx.x +
 // 512 k (slot 63 is the tile's first output; zero outside the stream and past the loaded samples). Every thread
 // calls it after tc_begin; on return the results are visible to the CTA and no TMEM is held. f64: FP64 accuracy of
-// every output (else that of the compensated product). False if a wait gave up: there are no results then, and the error
+// every output (else that of the compensated product). LOW: samples may be wider than FP32. False if a wait gave up: there are no results then, and the error
 // word is set. again(w): w = v once more, for outputs that are formed again
 // (to keep v in registers past the products cost N^-1 alone 109 -> 121 us of 8.4 M samples). used(t): false if outputs
 // t .. t + 7 are not used.
-template <class Again, class Used = TcAll>
+template <bool LOW = true, class Again, class Used = TcAll>
 __device__ __forceinline__ bool tc_band(unsigned char *sm, const double (&v)[kTcPer], const NoiseView &nv, int64_t gdet,
                                         unsigned *err, bool f64, int len, Again &&again, Used &&used = Used{})
 {
@@ -628,7 +630,7 @@ __device__ __forceinline__ bool tc_band(unsigned char *sm, const double (&v)[kTc
         __syncthreads();
     } else if (nredo) {
         const double *c = nv.p64 + gdet * nv.ntaps;
-        if (may_dot2 && nredo > kDot2From) tc_redo_dot2(sm, nredo, c, nv.ntaps);
+        if (may_dot2 && nredo > kDot2From) tc_redo_dot2<LOW>(sm, nredo, c, nv.ntaps);
         else tc_redo_chain(sm, nredo, c, nv.ntaps);
         __syncthreads();
     }

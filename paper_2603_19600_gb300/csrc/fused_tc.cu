@@ -79,7 +79,7 @@ __global__ void __launch_bounds__(TT, 2) tc_operator_kernel(const Tile *__restri
         if constexpr (MODE == 0 && !FROM_TOD)   // the recipe costs more than the registers
             ok = tc_band(sm, v, nv, gdet, err, f64, tl.len, TcKeep{v});
         else
-            ok = tc_band(sm, v, nv, gdet, err, f64, tl.len, fill);
+            ok = tc_band<!FROM_TOD || sizeof(DT) == 8>(sm, v, nv, gdet, err, f64, tl.len, fill);
         if (!ok) return;
     }
     const double *ys = tc_ys(sm);

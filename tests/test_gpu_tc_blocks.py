@@ -98,3 +98,21 @@ def test_compensated_product_between_loud_samples(fx, dev, orc):
         np.add.at(ref[:, k], pix.ravel(), (y * w).ravel())
         np.add.at(scale[:, k], pix.ravel(), (a * np.abs(w)).ravel())
     assert np.all(np.abs(got - ref) <= (254 * 2.0 ** -24) ** 2 * scale)
+
+
+def test_compensated_product_of_fp32_data(fx, dev, orc):
+    """The same from FP32 data (no low words), every second half tile 2^16 louder, so that half of every tile takes it."""
+    nd, ns, nside = 3, 12288, 32
+    o = synth.Observation(nside, synth.satellite_scan(ns), synth.hex_focal_plane(nd))
+    P = fx.Pointing.from_observations([o], mode="cache_f64", device=dev)
+    taps = np.tile(synth.inverse_noise_taps(), (nd, 1))
+    pix, c, s, _ = orc.pointing(nside, o.q_bore, o.q_det)
+    d = np.random.default_rng(4).normal(size=(nd, ns)).astype(np.float32)
+    d[:, np.arange(ns) // 2048 % 2 == 1] *= np.float32(2.0 ** 16)
+    got = fx.rhs(P, fx.Noise.banded(P, taps), torch.as_tensor(d.ravel(), device=dev)).cpu().numpy()
+    ref, scale = np.zeros((2, o.npix, 3), np.longdouble)
+    y, a = _ref(d, taps), _ref(np.abs(d), np.abs(taps))
+    for k, w in enumerate((np.ones_like(c), c, s)):
+        np.add.at(ref[:, k], pix.ravel(), (y * w).ravel())
+        np.add.at(scale[:, k], pix.ravel(), (a * np.abs(w)).ravel())
+    assert np.all(np.abs(got - ref) <= (254 * 2.0 ** -24) ** 2 * scale)
