@@ -3,9 +3,9 @@
 // FURAX_F64 and FURAX_PREC_F32X2: the tile skeleton of fused_tc.cu, the band on the tensor cores.
 //
 // r stays in the registers it was formed in until y is known; the map records are gathered a second time for the
-// angle gradient. Bound by the FP64 pipe (10 instructions per sample and 8 more for angle offsets, where the FMA chain
+// angle gradient. Bound by the FP64 pipe (9 instructions per sample and 8 more for angle offsets, where the FMA chain
 // took 127 for the band alone) and the phases' latency: 128 x 131,072 samples, nside 256, FP64 cache: 4561 us with the
-// chain, 919 us with r formed a second time beside y and 256 threads, 872 us now.
+// chain, 919 us with r formed a second time beside y and 256 threads, 857 us now.
 #include "tc_sample.cuh"
 
 namespace fx {

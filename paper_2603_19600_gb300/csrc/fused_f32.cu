@@ -114,7 +114,7 @@ static furax_status dispatch_fused_f32(const furax_pointing *p, const furax_nois
 // On the fly: the certified pointing (pointing_fast.cu) of a chunk of tiles goes to a workspace, and the
 // pipelined operator of the cached pointing reads it from there, chunk by chunk. One kernel that did both per tile
 // had to be 72 KB of shared memory and 80 registers wide and ran its phases (pointing, exact recipe, gather, band,
-// scatter) one after the other. 64 x 262,144 samples, nside 512: 768 us that way, 648 us this way (626 us since the sums go straight into the output) with 32 tiles per SM
+// scatter) one after the other. 64 x 262,144 samples, nside 512: 768 us that way, 648 us this way (626 us since the sums go straight into the output, 617 us with dependent launches) with 32 tiles per SM
 // and chunk; with 16 some 60 us more, with 8, which stay in L2, 130 us more: the last round of every launch costs more than the 24
 // bytes per sample through memory. The workspace (250 MB) is all that on-the-fly pointing ever holds. The three kernels
 // of a chunk are dependent launches, each placed while the one before ends: 3 x 9001 samples with FP32 sums take 60 us in one kernel,

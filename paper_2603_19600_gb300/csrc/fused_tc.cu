@@ -8,13 +8,14 @@
 // pointing is read a second time for the scatter (from L2), which leaves the shared memory to the digits.
 // What bounds it: the L2's FP64 reductions (3 per sample, 18,000 cycles per tile and SM at the rate of
 // furax_probe_l2 kind 5) and the latency of the phases before them (fill 4,000 from data, 21,000 through a map;
-// digits 3,500; products 9,000; accumulators to y 5,000-7,000 cycles), which two CTAs per SM overlap in part.
+// digits and sums 4,000; products 9,000; accumulators to y 5,000-7,000 cycles), which two CTAs per SM overlap in part.
 // Each CTA has 512 threads at 64 registers: with 256 at 128 the same phases took 5,000 / 26,000, 4,000, 9,000 and
 // 6,000-10,000 cycles and the scatter 33,000 instead of 23,000. Measured (GB300): FP64 FMAs (double-FP32 for the
 // right-hand side), 256 threads, now:
-//   normal operator, 32 x 262,147 samples, nside 256, FP64 cache   2277, 329, 277 us
-//   right-hand side, 128 x 524,288 FP32 samples, mixed cache       3440, 1730, 1387 us
-//   N^-1 alone, 32 x 131,071 samples                               1011, 61, 58 us
+//   normal operator, 32 x 262,147 samples, nside 256, FP64 cache   2277, 329, 284 us
+//   right-hand side, 128 x 524,288 FP32 samples, mixed cache       3440, 1730, 1428 us
+//   N^-1 alone, 32 x 131,071 samples                               1011, 61, 64 us
+// (277, 1387 and 58 us before every block of outputs was checked and the taps had eight digits, band_tc.cuh.)
 #include "tc_sample.cuh"
 #include "tpl_eval.cuh"
 

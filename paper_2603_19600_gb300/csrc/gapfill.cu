@@ -181,8 +181,9 @@ __global__ void __launch_bounds__(FT) gf_dir_kernel(const Tile *__restrict__ til
 // The FP64-accurate iteration for short bands in two passes: the direction is formed where the band product
 // loads it, the product is masked and dotted where it leaves, and the detector's last tile forms the scalar that
 // the next pass reads. (With a pass per step: 113 B per sample and iteration and five launches; here 82 B and two. 32 x
-// 131,071 samples: 115 us an iteration before, 87 us now: 59 us the product, bound by its phases' latency (fused_tc.cu),
-// 28 us the step, 7.3 TB/s of its 48 B per sample.)
+// 131,071 samples: 115 us an iteration before, 90 us now: 62 us the product, bound by its phases' latency (fused_tc.cu),
+// 28 us the step, 7.3 TB/s of its 48 B per sample. Of the product's outputs only those of observed samples must keep
+// their accuracy: the check of the blocks asks the mask.)
 // ------------------------------------------------------------------------------------
 
 // Sum over the CTA's TT threads added to *sum; true in every thread of the detector's last tile.
@@ -327,8 +328,8 @@ furax_status gapfill(const furax_noise *n, const void *d, const uint8_t *valid, 
                      int maxiter, double tol, int precision, int32_t *iters_out, cudaStream_t st)
 {
     const bool f32 = precision == FURAX_F32;   // band product in FP32, vectors and scalars in FP64
-    // N y, of which the gaps' outputs are used: short bands on the tensor cores, FURAX_PREC_F32X2 with the
-    // compensated product for tiles outside the digits' range
+    // N y, of which the gaps' outputs are used, however far they lie from observed samples: every block is checked (7 of
+    // a tile's 512 formed again with 4 % of the samples in gaps of 120)
     auto ninv64 = [&](const double *in, double *o) {
         return long_band(n) ? launch_ninv(n, in, o, FURAX_F64, st) : launch_ninv_tc(n, in, o, precision == FURAX_F64, n->gf_err(), st);
     };

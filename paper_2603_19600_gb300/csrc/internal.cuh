@@ -405,8 +405,8 @@ furax_status launch_fused_f32(const furax_pointing *p, const furax_noise *n, con
 bool fused_f32_projects_templates(const furax_pointing *p);
 // FP64-accurate operator and right-hand side (fused_tc.cu): acc64 += P^T N^-1 P S^T x (valid may be NULL:
 // every pixel) and acc64 += P^T N^-1 d. tp: the template correction -P^T (W T) b is folded into the same pass,
-// with b already solved by launch_tpl_rhs_amplitudes. f64: tiles outside the digits' range take the FP64
-// FMA chain, else the compensated double-FP32 product (band_tc.cuh).
+// with b already solved by launch_tpl_rhs_amplitudes. f64: outputs that the digits do not resolve take the FP64
+// FMA chain, else many of them the compensated double-FP32 product (band_tc.cuh).
 furax_status launch_fused_tc(const furax_pointing *p, const furax_noise *n, const double *x, const uint8_t *valid, double *acc64,
                              bool f64, cudaStream_t st);
 // The same on the map already in ws_x4; returns at once when *done == n_obs (PCG iterations after convergence).

@@ -9,7 +9,7 @@
 // whichever of its blocks finishes last, which also forms the scalars (no launch of their own).
 // Iterations enqueued after every observation has converged return at once: the host looks at the
 // convergence flags every check_every iterations only. Whole solves (GB300): FP64, white noise, 4 x 65,536
-// samples, nside 16: 1043 -> 268 us; mixed, 64 x 131,072 samples, nside 256: 6490 -> 4440 us.
+// samples, nside 16: 1043 -> 270 us; mixed, 64 x 131,072 samples, nside 256: 6490 -> 4484 us.
 // The iteration body is a fixed sequence of launches on one stream, captured once into a
 // CUDA graph and replayed; the host reads the convergence flags every few iterations.
 //

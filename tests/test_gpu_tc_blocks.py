@@ -116,3 +116,25 @@ def test_compensated_product_of_fp32_data(fx, dev, orc):
         np.add.at(ref[:, k], pix.ravel(), (y * w).ravel())
         np.add.at(scale[:, k], pix.ravel(), (a * np.abs(w)).ravel())
     assert np.all(np.abs(got - ref) <= (254 * 2.0 ** -24) ** 2 * scale)
+
+
+@pytest.mark.parametrize("n", [1, 11, 12, 13, 60])
+@pytest.mark.parametrize("loud", [2.0 ** 10, 2.0 ** 40, 1e300, np.inf, np.nan])
+def test_loud_samples_around_the_number_left_out(fx, dev, n, loud):
+    """Up to 12 groups of 32 samples of a tile may hold samples that stay out of the digits: both sides of that number,
+    with samples that are not finite acting only where their band reaches."""
+    ns = 4096
+    g = np.random.default_rng(n)
+    x = g.normal(size=(3, ns))
+    at = 32 * (g.permutation(ns // 32)[:n]) + g.integers(0, 32, n)
+    x[:2, at] *= loud
+    x[1, :] *= 2.0 ** -100
+    taps = np.tile(synth.inverse_noise_taps(), (3, 1))
+    if np.isfinite(loud):
+        _check(fx, dev, x, taps)
+        return
+    got, clean = _apply(fx, dev, x, taps), np.where(np.isfinite(x), x, 0.0)
+    ref, scale = _ref(clean, taps), _ref(np.abs(clean), np.abs(taps))
+    reach = _ref((~np.isfinite(x)).astype(float), np.ones((3, 64))) > 0
+    assert not np.isfinite(got[reach]).any()
+    assert np.all(np.abs(got[~reach] - ref[~reach]) <= 127 * 2.0 ** -53 * scale[~reach])
